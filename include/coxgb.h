@@ -75,7 +75,9 @@ enum {
     COX_SPLIT_E4M3 = 0, /* tcgen05 tensor cores (kind::f8f6f4): genotype codes as
                            e4m3, coefficients split into 4 e4m3 limbs under a
                            power-of-two column scale, FP32 accumulation; FP64
-                           risk-set scans (default)                            */
+                           risk-set scans (default).  For k <= 12, unless the
+                           options force a pipeline shape, the same coefficient
+                           values run as ten e2m1 digits each (kind::mxf4)     */
     COX_FP64 = 1,       /* FP64 everywhere, dense X (COX_X_F64_HOST)          */
     COX_FP32_GEMV = 2,  /* baseline: one lambda at a time, FP32 CUDA-core GEMV
                            on the packed genotypes, unfused soft threshold    */
@@ -359,8 +361,9 @@ int cox_autotune(cox_h h, int k, int reps, cox_tune_choice *xb, cox_tune_choice 
  * without a device or handle: for k coefficient columns (1..64) and a shape
  * (tile_m 128-row tiles per CTA, chunks 128-wide K chunks per stage, issue as
  * cox_options.issue; 0 = the built-in default) at a shared-memory depth
- * (stages; 0 = the deepest that fits), the plan cox_setup's handles would
- * launch.  Every plan it returns keeps the pipeline's invariants: ring >=
+ * (stages; 0 = the deepest that fits), the plan of the e4m3 kernel that
+ * cox_setup's handles would launch (for k <= 12 they do when the options force
+ * a shape).  Every plan it returns keeps the pipeline's invariants: ring >=
  * decoder_groups, ring < stages (e2m1: ring < limb_stages), named_barriers <= 15, tmem_cols <= 512,
  * smem_bytes within the device's per-block limit, and for issue 2 two decoder
  * groups with an even ring and an even number of stages.  Errors: COX_ERR_ARG

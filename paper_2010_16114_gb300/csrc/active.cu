@@ -161,6 +161,45 @@ __global__ void k_prep_limbs_active4(const float *__restrict__ beta, int64_t p, 
     }
 }
 
+// wide e2m1 limbs of the e4m3 split at the active SNPs (bytes as above)
+__global__ void k_prep_limbs_active_wide(const float *__restrict__ beta, int64_t p, const int32_t *__restrict__ Aidx,
+                                         int64_t nA, int64_t Kpad, int nb, const float *__restrict__ maxp,
+                                         uint8_t *__restrict__ Bq, int *__restrict__ bs, int *err)
+{
+    __shared__ int s_sh;
+    const int kk = blockIdx.y;
+    if (threadIdx.x < 32) {
+        float m = 0.f;
+        for (int b = threadIdx.x; b < nb; b += 32) m = fmaxf(m, maxp[kk * nb + b]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (threadIdx.x == 0) {
+            if (!isfinite(m)) {
+                atomicOr(err, DEVERR_NONFINITE);
+                m = 0.f;
+            }
+            s_sh = limb_scale(m);
+            if (blockIdx.x == 0) bs[kk] = s_sh;
+        }
+    }
+    __syncthreads();
+    const int s = s_sh;
+    const int64_t rb = Kpad / 2;
+    for (int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; t < rb;
+         t += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t t0 = ((t >> 3) << 4) + (t & 7);
+        uint8_t d[LIMBS], d0[LIMBS_W], d1[LIMBS_W];
+        const float *bc = beta + static_cast<int64_t>(kk) * p;
+        const float ra = t0 < nA ? ldexpf(bc[Aidx[t0]], -s) : 0.f, rc = t0 + 8 < nA ? ldexpf(bc[Aidx[t0 + 8]], -s) : 0.f;
+        // a NaN passes the maximum and has no digits (as e4m3 it would reach eta)
+        if (!isfinite(ra) || !isfinite(rc)) atomicOr(err, DEVERR_NONFINITE);
+        split_wide(split_e4m3_units(ra, d), d0);
+        split_wide(split_e4m3_units(rc, d), d1);
+#pragma unroll
+        for (int l = 0; l < LIMBS_W; ++l) Bq[(LIMBS_W * kk + l) * rb + t] = static_cast<uint8_t>(d0[l] | (d1[l] << 4));
+    }
+}
+
 unsigned grid_over(int64_t total, int sms)
 {
     return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 16LL * sms)));
@@ -266,11 +305,11 @@ int active_prepare(cox_handle *h, const float *beta, int k, cudaStream_t st, int
         dfree(ws.Bqa);
         ws.Bqa = nullptr;
         const int64_t bpk = ws.g1.f4 ? 2 : 1;  // K positions per limb byte
-        COX_TRY(dmalloc(h, reinterpret_cast<void **>(&ws.Bqa), static_cast<size_t>(ws.NP) * h->act_Kpad / bpk));
-        COX_CUDA(cudaMemsetAsync(ws.Bqa, 0, static_cast<size_t>(ws.NP) * h->act_Kpad / bpk, st));
+        COX_TRY(dmalloc(h, reinterpret_cast<void **>(&ws.Bqa), static_cast<size_t>(ws.g1.NP) * h->act_Kpad / bpk));
+        COX_CUDA(cudaMemsetAsync(ws.Bqa, 0, static_cast<size_t>(ws.g1.NP) * h->act_Kpad / bpk, st));
         const int issue = ws.g1.alt ? 2 : ws.g1.pair ? 3 : 1;
-        COX_TRY(plan_gemm(h, ws.g1a, h->d_A1act, h->n_pad, h->act_Kpad, ws.Bqa, k, ws.g1.T, ws.g1.CH, ws.g1.stages,
-                          issue));
+        COX_TRY(plan_gemm(h, ws.g1a, h->d_A1act, h->n_pad, h->act_Kpad, ws.Bqa, k, ws.g1.f4, ws.g1.T, ws.g1.CH,
+                          ws.g1.stages, issue));
         if (ws.g1a.max_slots > ws.part1_slots) {
             dfree(ws.part1);
             ws.part1 = nullptr;
@@ -282,7 +321,10 @@ int active_prepare(cox_handle *h, const float *beta, int k, cudaStream_t st, int
         ws.g1a_K = h->act_Kpad;
     }
     const int64_t gx = std::min<int64_t>((h->act_Kpad + 255) / 256, std::max<int64_t>(1, 4LL * h->sm_count / k));
-    if (ws.g1.f4)
+    if (ws.g1.f4 == FORM_WIDE)
+        k_prep_limbs_active_wide<<<dim3(static_cast<unsigned>(gx), k), 256, 0, st>>>(
+            beta, p, h->d_Aidx, h->nA, h->act_Kpad, h->l1_blocks, ws.bmaxp, ws.Bqa, ws.bs1, h->d_err);
+    else if (ws.g1.f4)
         k_prep_limbs_active4<<<dim3(static_cast<unsigned>(gx), k), 256, 0, st>>>(
             beta, p, h->d_Aidx, h->nA, h->act_Kpad, h->l1_blocks, ws.bmaxp, ws.Bqa, ws.bs1, h->d_err);
     else

@@ -102,6 +102,18 @@ int tune_key(const cox_handle *h, int k) { return is_e2m1(h) ? k + 4096 : k; }
 // largest k of the tensor-core products: 128 e2m1 limb columns hold 16 coefficients
 int max_k_tc(const cox_handle *h) { return is_e2m1(h) ? MAX_K_E2M1 : MAX_K_TC; }
 
+// The operand form of a handle's products for k columns when the options force
+// no pipeline shape: an e4m3 handle takes the wide form where it holds k
+// columns, k <= 12 (the same coefficients and exact window sums; the product
+// is then bound by HBM, not by MMA issue).  Past 12 columns the wide limbs
+// would need more than 128 MMA columns, twice the e4m3 kernel's MMA cycles.
+int default_form(const cox_handle *h, int k)
+{
+    if (is_e2m1(h)) return FORM_E2M1;
+    const bool forced = h->opt.tile_m || h->opt.chunks || h->opt.stages || h->opt.issue;
+    return !forced && limb_cols_wide(k) ? FORM_WIDE : FORM_E4M3;
+}
+
 cudaEvent_t get_event(cox_handle *h)
 {
     if (h->ev_used == h->ev_pool.size()) {
@@ -434,31 +446,31 @@ int ensure_workspace(cox_handle *h, int k)
         cudaMemset(ws.gamma, 0, static_cast<size_t>(k) * h->q * sizeof(double));
     }
     if (is_split(h)) {
+        // pipeline shapes and operand forms: forced by the options, else autotuned for k, else default
+        int T1 = h->opt.tile_m, C1 = h->opt.chunks, S1 = h->opt.stages, A1 = h->opt.issue;
+        int T4 = T1, C4 = C1, S4 = S1, A4 = A1;
+        int F1 = default_form(h, k), F4 = F1;
+        const auto tc = h->tuned.find(tune_key(h, k));
+        if (tc != h->tuned.end() && !T1 && !C1 && !S1 && !A1) {
+            T1 = tc->second.T1, C1 = tc->second.CH1, S1 = tc->second.S1, A1 = tc->second.A1, F1 = tc->second.F1;
+            T4 = tc->second.T4, C4 = tc->second.CH4, S4 = tc->second.S4, A4 = tc->second.A4, F4 = tc->second.F4;
+        }
         // limb rows of K_pad e4m3 bytes, or K_pad / 2 bytes of e2m1 pairs
-        const int NP = is_e2m1(h) ? limb_cols4(k) : limb_cols(k);
-        const int64_t bpk = is_e2m1(h) ? 2 : 1;  // K positions per byte
-        A(ws.Bq, static_cast<size_t>(NP) * h->p_pad / bpk);
-        A(ws.Vq, static_cast<size_t>(NP) * h->n_pad / bpk);
+        const size_t Bq_bytes = static_cast<size_t>(limb_cols_of(F1, k)) * h->p_pad / (F1 ? 2 : 1);
+        const size_t Vq_bytes = static_cast<size_t>(limb_cols_of(F4, k)) * h->n_pad / (F4 ? 2 : 1);
+        A(ws.Bq, Bq_bytes);
+        A(ws.Vq, Vq_bytes);
         A(ws.bs1, k);
         A(ws.bs4, k);
         A(ws.bmaxp, static_cast<size_t>(k) * h->l1_blocks);
         A(ws.vmaxp, k * nch);
-        // limb rows past LIMBS k and K positions of padding stay zero
-        cudaMemset(ws.Bq, 0, static_cast<size_t>(NP) * h->p_pad / bpk);
-        cudaMemset(ws.Vq, 0, static_cast<size_t>(NP) * h->n_pad / bpk);
-        ws.NP = NP;
+        // limb rows past the coefficients' and K positions of padding stay zero
+        cudaMemset(ws.Bq, 0, Bq_bytes);
+        cudaMemset(ws.Vq, 0, Vq_bytes);
         cudaMemset(ws.bs1, 0, k * sizeof(int));
         cudaMemset(ws.bs4, 0, k * sizeof(int));
-        // pipeline shapes: forced by the options, else autotuned for k, else default
-        int T1 = h->opt.tile_m, C1 = h->opt.chunks, S1 = h->opt.stages, A1 = h->opt.issue;
-        int T4 = T1, C4 = C1, S4 = S1, A4 = A1;
-        const auto tc = h->tuned.find(tune_key(h, k));
-        if (tc != h->tuned.end() && !T1 && !C1 && !S1 && !A1) {
-            T1 = tc->second.T1, C1 = tc->second.CH1, S1 = tc->second.S1, A1 = tc->second.A1;
-            T4 = tc->second.T4, C4 = tc->second.CH4, S4 = tc->second.S4, A4 = tc->second.A4;
-        }
-        if ((r = plan_gemm(h, ws.g1, h->d_A1, h->n_pad, h->p_pad, ws.Bq, k, T1, C1, S1, A1)) != COX_OK ||
-            (r = plan_gemm(h, ws.g4, h->d_A4, h->p_pad, h->n_pad, ws.Vq, k, T4, C4, S4, A4)) != COX_OK) {
+        if ((r = plan_gemm(h, ws.g1, h->d_A1, h->n_pad, h->p_pad, ws.Bq, k, F1, T1, C1, S1, A1)) != COX_OK ||
+            (r = plan_gemm(h, ws.g4, h->d_A4, h->p_pad, h->n_pad, ws.Vq, k, F4, T4, C4, S4, A4)) != COX_OK) {
             free_workspace(h);
             return r;
         }
@@ -722,13 +734,21 @@ int cox_autotune(cox_h h, int k, int reps, cox_tune_choice *xb, cox_tune_choice 
     h->tuned.erase(tune_key(h, k));
     COX_TRY(ensure_workspace(h, k));  // limb buffers (zero) and scale arrays for the timing launches
     Workspace &ws = h->ws;
-    int Ts[16], Cs[16], As[16];
-    const int nshape = gemm_shapes(k, Ts, Cs, As, 16, is_e2m1(h));
+    // every compiled shape of the handle's operand forms: e2m1, or e4m3 and, where it
+    // holds k columns, the wide form
+    int Ts[20], Cs[20], As[20], Fs[20];
+    int nshape = 0;
+    const int forms[2] = {is_e2m1(h) ? FORM_E2M1 : FORM_E4M3, FORM_WIDE};
+    for (int f = 0; f < (is_e2m1(h) ? 1 : 2); ++f) {
+        const int c = gemm_shapes(k, Ts + nshape, Cs + nshape, As + nshape, 20 - nshape, forms[f]);
+        for (int j = 0; j < c; ++j) Fs[nshape + j] = forms[f];
+        nshape += c;
+    }
     // the planner's depth only: four-stage plans measured 2-3x slower for every
     // shape at full size (the bench's workloads), so they are not timed
     const int depth_req[1] = {0};
     cox_tune_choice best[2];
-    int cand[2] = {0, 0};
+    int cand[2] = {0, 0}, best_form[2] = {0, 0};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     COX_CUDA(cudaEventCreate(&e0));
     if (cudaEventCreate(&e1) != cudaSuccess) {
@@ -740,13 +760,18 @@ int cox_autotune(cox_h h, int k, int reps, cox_tune_choice *xb, cox_tune_choice 
         best[prod] = cox_tune_choice{0, 0, 0, 0, 1e300, 0};
         const uint32_t *A = prod == 0 ? h->d_A1 : h->d_A4;
         const int64_t rows = prod == 0 ? h->n_pad : h->p_pad, K = prod == 0 ? h->p_pad : h->n_pad;
-        const uint8_t *B = prod == 0 ? ws.Bq : ws.Vq;
+        uint8_t *B = nullptr;  // zero limbs, large enough for every form
+        size_t bb = 0;
+        for (int j = 0; j < nshape; ++j)
+            bb = std::max(bb, static_cast<size_t>(limb_cols_of(Fs[j], k)) * K / (Fs[j] ? 2 : 1));
+        if ((rc = dmalloc(nullptr, reinterpret_cast<void **>(&B), bb)) != COX_OK) break;
+        if (cudaMemset(B, 0, bb) != cudaSuccess) rc = COX_ERR_CUDA;
         for (int j = 0; j < nshape && rc == COX_OK; ++j) {
             int last_S = -1;
             if (As[j] == 3) continue;  // pair commits: not timed (no faster than per-stage commits)
             for (int dq = 0; dq < 1 && rc == COX_OK; ++dq) {
                 GemmPlan g;
-                if (plan_gemm(h, g, A, rows, K, B, k, Ts[j], Cs[j], depth_req[dq], As[j]) != COX_OK) continue;
+                if (plan_gemm(h, g, A, rows, K, B, k, Fs[j], Ts[j], Cs[j], depth_req[dq], As[j]) != COX_OK) continue;
                 if (g.stages == last_S) continue;  // the two depths coincide
                 last_S = g.stages;
                 float *part = nullptr;
@@ -774,17 +799,22 @@ int cox_autotune(cox_h h, int k, int reps, cox_tune_choice *xb, cox_tune_choice 
                 if ((rc = check_device_error(h, 0)) != COX_OK) break;
                 ++cand[prod];
                 const double m = static_cast<double>(ms) / reps;
-                if (m < best[prod].ms) best[prod] = cox_tune_choice{g.T, g.CH, g.stages, 0, m, As[j]};
+                if (m < best[prod].ms) {
+                    best[prod] = cox_tune_choice{g.T, g.CH, g.stages, 0, m, As[j]};
+                    best_form[prod] = Fs[j];
+                }
             }
         }
         best[prod].candidates = cand[prod];
+        dfree(B);
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc != COX_OK) return rc;
     if (!cand[0] || !cand[1]) return COX_ERR_ARG;
     h->tuned[tune_key(h, k)] = cox_handle::TuneChoice{best[0].tile_m, best[0].chunks, best[0].stages, best[0].issue,
-                                         best[1].tile_m, best[1].chunks, best[1].stages, best[1].issue};
+                                         best[1].tile_m, best[1].chunks, best[1].stages, best[1].issue,
+                                         best_form[0], best_form[1]};
     cudaDeviceSynchronize();
     free_workspace(h);  // the next call with k columns plans the chosen shapes
     if (xb) *xb = best[0];

@@ -1,5 +1,5 @@
 // gemm_f4.cu -- the e2m1 instantiations of the genotype-product kernel
-// (gemm_kernel.cuh): codes as e2m1 nibbles, coefficients as LIMBS4 e2m1 limbs,
+// (gemm_kernel.cuh): codes as e2m1 nibbles, coefficients as LIMBS4 or LIMBS_W e2m1 limbs,
 // tcgen05.mma kind::mxf4 with unit block scales (K = 64 per instruction).  In a
 // translation unit of their own so that the two forms compile in parallel.
 #include "gemm_kernel.cuh"
@@ -14,12 +14,22 @@ namespace coxgb {
 // is compiled.  One tile x four chunks is compiled at 64 columns only: at 128
 // its 32 KB limb slots leave no ring depths that keep every parity wait
 // unambiguous (the planner's ring_safe) within 227 KB.
-GemmKernelFn pick_kernel_f4(int T, int CH, int NP)
+GemmKernelFn pick_kernel_f4(int T, int CH, int NP, int form)
 {
+    if (form == FORM_WIDE) {
+        if (T != 2 || CH != 2) return nullptr;
+        switch (NP) {
+        case 16: return k_packed_gemm<2, 2, 16, DEC_GROUPS, false, LIMBS_W>;
+        case 32: return k_packed_gemm<2, 2, 32, DEC_GROUPS, false, LIMBS_W>;
+        case 64: return k_packed_gemm<2, 2, 64, DEC_GROUPS, false, LIMBS_W>;
+        case 128: return k_packed_gemm<2, 2, 128, DEC_GROUPS, false, LIMBS_W>;
+        default: return nullptr;
+        }
+    }
     switch ((T * 10 + CH) * 1000 + NP) {
-    case 22064: return k_packed_gemm<2, 2, 64, DEC_GROUPS, false, true>;
-    case 14064: return k_packed_gemm<1, 4, 64, DEC_GROUPS, false, true>;
-    case 22128: return k_packed_gemm<2, 2, 128, DEC_GROUPS, false, true>;
+    case 22064: return k_packed_gemm<2, 2, 64, DEC_GROUPS, false, LIMBS4>;
+    case 14064: return k_packed_gemm<1, 4, 64, DEC_GROUPS, false, LIMBS4>;
+    case 22128: return k_packed_gemm<2, 2, 128, DEC_GROUPS, false, LIMBS4>;
     default: return nullptr;
     }
 }

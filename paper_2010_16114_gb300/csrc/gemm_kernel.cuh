@@ -37,6 +37,15 @@
 // matters.  A limb panel of 128-byte rows covers two K chunks, so the e2m1
 // stages hold an even number of chunks.
 //
+// The wide form (FL = LIMBS_W) is the e2m1 kernel on the e4m3 form's
+// coefficients: the value of a column's four e4m3 limbs, a 30-bit integer, as
+// ten e2m1 digits (split_wide).  Same operands, exact window sums, half the MMA
+// instructions per code, so the product is bound by HBM instead of by MMA
+// issue (16 MMAs of ~57 cycles per 16 KB stage in the e4m3 kernel at any N up
+// to 64).  Ten limb columns per coefficient fill 128 at k = 12.  Measured at
+// k = 1: a whole step at n = 100,000, p = 50,000 takes 566 us against 695 with
+// the e4m3 kernel, 20 iterations at n = 200,000, p = 10,000 6.79 ms against 7.75.
+//
 // Pipeline per CTA (one per SM): two TMA warps fill a ring of shared-memory
 // stages (T row tiles x CH K chunks of codes, and the matching limb panels);
 // groups of four decoder warps turn a stage into e4m3 in a ring of TMEM slots,
@@ -104,7 +113,7 @@ struct KParams {
 using GemmKernelFn = void (*)(const CUtensorMap, const CUtensorMap, const KParams);
 
 // The e2m1 shapes (gemm_f4.cu); null when (T, CH, NP) is not compiled.
-GemmKernelFn pick_kernel_f4(int T, int CH, int NP);
+GemmKernelFn pick_kernel_f4(int T, int CH, int NP, int form);
 
 namespace {
 
@@ -201,16 +210,17 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, long lo
 // it (they first wait, through the TMEM slot chain, for MMAs that this issuer
 // issues after it).  Decoders arrive on every path, so an issuer's (unbounded)
 // hardware-barrier wait always ends.
-template <int T, int CH, int NP, int G, bool ALT, bool F4>
+// FL: limbs per coefficient of the e2m1 forms (LIMBS4, LIMBS_W); 0 for e4m3 operands.
+template <int T, int CH, int NP, int G, bool ALT, int FL>
 __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
     k_packed_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const KParams P)
 {
+    constexpr bool F4 = FL > 0;           // e2m1 operands
     constexpr int I = ALT ? 2 : T;        // MMA issuers: one per row tile, or two on alternate stages
     static_assert(!ALT || G == 2, "alternating issuers pair with two decoder groups");
-    static_assert(!F4 || (!ALT && CH % 2 == 0 && NP % 8 == 0 && LIMBS4 == 8),
-                  "e2m1 operands: per-tile issuers, chunk pairs, one coefficient per 8 columns");
-    constexpr int NL = F4 ? LIMBS4 : LIMBS;  // limbs per coefficient column
+    static_assert(!F4 || (!ALT && CH % 2 == 0 && NP % 8 == 0), "e2m1 operands: per-tile issuers, chunk pairs");
+    constexpr int NL = F4 ? FL : LIMBS;   // limbs per coefficient column
     constexpr int KH = NP / NL;           // lambda columns a decoder thread folds (>= k)
     // B: one panel of NP rows x 128 bytes per K chunk (e4m3), or per two K
     // chunks (e2m1, two values per byte)
@@ -221,7 +231,9 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
     constexpr int CW = F4 ? 16 : 32;      // TMEM columns of 128 A values (one tile and chunk) per lane
     constexpr int SLOT_COLS = T * CH * CW;
     constexpr int MQ = F4 ? 2 * CH : 4 * CH;  // MMAs per tile and stage (K = 64 e2m1, 32 e4m3)
-    constexpr int SH = F4 ? 0 : 9;        // code scale: e2m1 codes are c, e4m3 codes c 2^-9
+    // scale of the folded sums beside the column's 2^s: e4m3 codes are c 2^-9, e2m1
+    // codes c; the wide limbs' leading digit is worth 2^(s+7) (split_wide)
+    constexpr int SH = FL == LIMBS_W ? 7 : F4 ? 0 : 9;
     constexpr int DEC0 = 2 + I;           // first decoder warp
     constexpr int NB_COUNT = 32 * 5;      // a decoder group and the tile's issuer warp
 
@@ -590,7 +602,35 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
             }
             fold_phase ^= 1u;
             tc_fence_after();
-            if constexpr (F4) {
+            if constexpr (FL == LIMBS_W) {
+                // lambda columns of ten e2m1 limbs (weights 8^-l), up to four (40 TMEM
+                // columns, five loads of eight) at a time
+#pragma unroll
+                for (int tt = 0; tt < T; ++tt) {
+#pragma unroll
+                    for (int e0 = 0; e0 < KH; e0 += 4) {
+                        constexpr int LD = 5;
+                        uint32_t u[8 * LD];
+#pragma unroll
+                        for (int b = 0; b < LD; ++b)
+                            if (8 * b < 10 * (KH - e0)) {
+                                uint32_t v[8];
+                                tmem_ld_32x32b_x8(lane_base + static_cast<uint32_t>(tt * NP + 10 * e0 + 8 * b), v);
+#pragma unroll
+                                for (int m = 0; m < 8; ++m) u[8 * b + m] = v[m];
+                            }
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (e0 + e < KH) {
+                                float x = __uint_as_float(u[10 * e + 9]);
+#pragma unroll
+                                for (int l = 8; l >= 0; --l) x = fmaf(x, 0.125f, __uint_as_float(u[10 * e + l]));
+                                acc(tt, e0 + e) += x;
+                            }
+                    }
+                }
+            } else if constexpr (F4) {
                 // one lambda column of eight e2m1 limbs (weights 8^-l) per 8 columns
 #pragma unroll
                 for (int tt = 0; tt < T; ++tt) {

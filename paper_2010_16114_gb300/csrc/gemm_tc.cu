@@ -80,6 +80,47 @@ __global__ void k_prep_limbs_beta4(const float *__restrict__ beta, int64_t p, in
     }
 }
 
+// beta -> wide e2m1 limbs [NP][p_pad / 2] of the e4m3 split (byte order as
+// k_prep_limbs_beta4, scales as k_prep_limbs_beta).
+__global__ void k_prep_limbs_beta_wide(const float *__restrict__ beta, int64_t p, int64_t p_pad, int nb,
+                                       const float *__restrict__ maxp, uint8_t *__restrict__ Bq,
+                                       int *__restrict__ bs, int *err)
+{
+    __shared__ int s_sh;
+    const int kk = blockIdx.y;
+    if (threadIdx.x < 32) {
+        float m = 0.f;
+        for (int b = threadIdx.x; b < nb; b += 32) m = fmaxf(m, maxp[kk * nb + b]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if (threadIdx.x == 0) {
+            if (!isfinite(m)) {
+                atomicOr(err, DEVERR_NONFINITE);
+                m = 0.f;
+            }
+            s_sh = limb_scale(m);
+            if (blockIdx.x == 0) bs[kk] = s_sh;
+        }
+    }
+    __syncthreads();
+    const int s = s_sh;
+    const int64_t rb = p_pad / 2;
+    for (int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; j < rb;
+         j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t j0 = ((j >> 3) << 4) + (j & 7);
+        if (j0 >= p) continue;
+        uint8_t d[LIMBS], d0[LIMBS_W], d1[LIMBS_W];
+        const float *bc = beta + static_cast<int64_t>(kk) * p;
+        const float ra = ldexpf(bc[j0], -s), rc = j0 + 8 < p ? ldexpf(bc[j0 + 8], -s) : 0.f;
+        // a NaN passes the maximum and has no digits (as e4m3 it would reach eta)
+        if (!isfinite(ra) || !isfinite(rc)) atomicOr(err, DEVERR_NONFINITE);
+        split_wide(split_e4m3_units(ra, d), d0);
+        split_wide(split_e4m3_units(rc, d), d1);
+#pragma unroll
+        for (int l = 0; l < LIMBS_W; ++l) Bq[(LIMBS_W * kk + l) * rb + j] = static_cast<uint8_t>(d0[l] | (d1[l] << 4));
+    }
+}
+
 using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                  const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
                                  const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
@@ -122,32 +163,32 @@ constexpr int G_WIDE = 2;  // decoder groups of the 2 x 2 shape at 128 limb colu
 
 KernelFn pick_kernel(int T, int CH, int NP, int alt, int f4)
 {
-    if (f4) return alt ? nullptr : pick_kernel_f4(T, CH, NP);
+    if (f4) return alt ? nullptr : pick_kernel_f4(T, CH, NP, f4);
     switch (((alt ? 100 : 0) + T * 10 + CH) * 1000 + NP) {
-    case 22016: return k_packed_gemm<2, 2, 16, DEC_GROUPS, false, false>;
-    case 21016: return k_packed_gemm<2, 1, 16, DEC_GROUPS, false, false>;
-    case 12016: return k_packed_gemm<1, 2, 16, DEC_GROUPS, false, false>;
-    case 22032: return k_packed_gemm<2, 2, 32, DEC_GROUPS, false, false>;
-    case 21032: return k_packed_gemm<2, 1, 32, DEC_GROUPS, false, false>;
-    case 12032: return k_packed_gemm<1, 2, 32, DEC_GROUPS, false, false>;
-    case 22064: return k_packed_gemm<2, 2, 64, DEC_GROUPS, false, false>;
-    case 21064: return k_packed_gemm<2, 1, 64, DEC_GROUPS, false, false>;
-    case 12064: return k_packed_gemm<1, 2, 64, DEC_GROUPS, false, false>;
-    case 21128: return k_packed_gemm<2, 1, 128, DEC_GROUPS, false, false>;
-    case 12128: return k_packed_gemm<1, 2, 128, DEC_GROUPS, false, false>;
-    case 11128: return k_packed_gemm<1, 1, 128, DEC_GROUPS, false, false>;
+    case 22016: return k_packed_gemm<2, 2, 16, DEC_GROUPS, false, 0>;
+    case 21016: return k_packed_gemm<2, 1, 16, DEC_GROUPS, false, 0>;
+    case 12016: return k_packed_gemm<1, 2, 16, DEC_GROUPS, false, 0>;
+    case 22032: return k_packed_gemm<2, 2, 32, DEC_GROUPS, false, 0>;
+    case 21032: return k_packed_gemm<2, 1, 32, DEC_GROUPS, false, 0>;
+    case 12032: return k_packed_gemm<1, 2, 32, DEC_GROUPS, false, 0>;
+    case 22064: return k_packed_gemm<2, 2, 64, DEC_GROUPS, false, 0>;
+    case 21064: return k_packed_gemm<2, 1, 64, DEC_GROUPS, false, 0>;
+    case 12064: return k_packed_gemm<1, 2, 64, DEC_GROUPS, false, 0>;
+    case 21128: return k_packed_gemm<2, 1, 128, DEC_GROUPS, false, 0>;
+    case 12128: return k_packed_gemm<1, 2, 128, DEC_GROUPS, false, 0>;
+    case 11128: return k_packed_gemm<1, 1, 128, DEC_GROUPS, false, 0>;
     // two decoder groups: 2 tiles x 2 chunks at 128 limb columns, whose two
     // 128-column TMEM slots beside 256 accumulator columns leave no third slot
-    case 22128: return k_packed_gemm<2, 2, 128, G_WIDE, false, false>;
+    case 22128: return k_packed_gemm<2, 2, 128, G_WIDE, false, 0>;
     // two decoder groups: 2 tiles x 3 chunks at 64 limb columns (12 MMAs per
     // commit per issuer; two 192-column slots beside 128 accumulator columns)
-    case 23064: return k_packed_gemm<2, 3, 64, G_WIDE, false, false>;
-    case 11256: return k_packed_gemm<1, 1, 256, DEC_GROUPS, false, false>;
+    case 23064: return k_packed_gemm<2, 3, 64, G_WIDE, false, 0>;
+    case 11256: return k_packed_gemm<1, 1, 256, DEC_GROUPS, false, 0>;
     // alternating issuers: 16 MMAs per commit up to N = 64, 8 at N = 128
-    case 122016: return k_packed_gemm<2, 2, 16, G_ALT, true, false>;
-    case 122032: return k_packed_gemm<2, 2, 32, G_ALT, true, false>;
-    case 122064: return k_packed_gemm<2, 2, 64, G_ALT, true, false>;
-    case 112128: return k_packed_gemm<1, 2, 128, G_ALT, true, false>;
+    case 122016: return k_packed_gemm<2, 2, 16, G_ALT, true, 0>;
+    case 122032: return k_packed_gemm<2, 2, 32, G_ALT, true, 0>;
+    case 122064: return k_packed_gemm<2, 2, 64, G_ALT, true, 0>;
+    case 112128: return k_packed_gemm<1, 2, 128, G_ALT, true, 0>;
     default: return nullptr;
     }
 }
@@ -194,7 +235,7 @@ bool ring_safe(int G, int R, int n) { return n >= G + R || n % G == 0; }
 // measured 0.65 of HBM against 0.84).  The code ring takes the rest of the
 // shared memory (at most 12, at least G + 1), the deepest safe depth.  The
 // largest TMEM ring for which such depths exist is taken.
-int plan_e2m1(GemmPlan &g, int T, int CH, int NP, int G, int stages_req, int fold_bytes)
+int plan_e2m1(GemmPlan &g, int T, int CH, int NP, int form, int G, int stages_req, int fold_bytes)
 {
     const int xb = T * CH * BLOCK_BYTES, bb = (CH / 2) * NP * 128;
     const int acc_cols = T * NP;
@@ -227,7 +268,7 @@ int plan_e2m1(GemmPlan &g, int T, int CH, int NP, int G, int stages_req, int fol
     g.T = T;
     g.CH = CH;
     g.NP = NP;
-    g.f4 = 1;
+    g.f4 = form;
     g.alt = 0;
     g.pair = 0;
     g.G = G;
@@ -245,7 +286,7 @@ int plan_e2m1(GemmPlan &g, int T, int CH, int NP, int G, int stages_req, int fol
 
 int gemm_shapes(int k, int *T, int *CH, int *issue, int max, int f4)
 {
-    const int NP = f4 ? limb_cols4(k) : limb_cols(k);
+    const int NP = limb_cols_of(f4, k);
     if (NP == 0) return 0;
     int n = 0;
     for (int is = 1; is <= (f4 ? 1 : 3); ++is)
@@ -268,8 +309,8 @@ int plan_shape(GemmPlan &g, int k, int T_req, int CH_req, int stages_req, int is
 {
     if (k < 1 || k > MAX_K_TC) return COX_ERR_ARG;
     if (issue_req < 0 || issue_req > 3) return COX_ERR_ARG;
-    if (f4 && (issue_req > 1 || limb_cols4(k) == 0)) return COX_ERR_ARG;  // e2m1: per-tile issuers, k <= 16
-    const int np_cls = f4 ? limb_cols4(k) : limb_cols(k);
+    const int np_cls = limb_cols_of(f4, k);
+    if (f4 && (issue_req > 1 || np_cls == 0)) return COX_ERR_ARG;  // e2m1: per-tile issuers; k <= 16, wide 12
     int T = 2, CH = 1, alt = 0;
     shape_for(np_cls, &T, &CH, &alt, f4);
     if (issue_req > 0) alt = issue_req == 2;
@@ -280,10 +321,10 @@ int plan_shape(GemmPlan &g, int k, int T_req, int CH_req, int stages_req, int is
     if (G == G_WIDE && !alt && issue_req == 3) return COX_ERR_ARG;  // pair commits: not planned for it
     // limb panels of 128-byte rows: one per K chunk (e4m3), one per chunk pair (e2m1)
     const int stage = (f4 ? CH / 2 : CH) * np_cls * 128 + CH * T * BLOCK_BYTES;
-    const int kh = np_cls / (f4 ? LIMBS4 : LIMBS);  // coefficient columns the fold holds
+    const int kh = np_cls / limbs_of(f4);  // coefficient columns the fold holds
     // group 0's window sums, then four per-column constants
     const int fold_bytes = T * kh * 128 * 4 + 4 * kh * 4;
-    if (f4) return plan_e2m1(g, T, CH, np_cls, G, stages_req, fold_bytes);
+    if (f4) return plan_e2m1(g, T, CH, np_cls, f4, G, stages_req, fold_bytes);
     int S = stages_req > 0 ? stages_req : (225 * 1024 - 2048 - fold_bytes) / stage;
     if (S > 12) S = 12;
     if (alt && stages_req <= 0 && S % 2) --S;  // the parity classes need an even stage ring
@@ -330,9 +371,9 @@ int plan_shape(GemmPlan &g, int k, int T_req, int CH_req, int stages_req, int is
 }
 
 int plan_gemm(cox_handle *h, GemmPlan &g, const uint32_t *A, int64_t rows_pad, int64_t K_pad,
-              const uint8_t *B, int k, int T_req, int CH_req, int stages_req, int issue_req)
+              const uint8_t *B, int k, int form, int T_req, int CH_req, int stages_req, int issue_req)
 {
-    COX_TRY(plan_shape(g, k, T_req, CH_req, stages_req, issue_req, is_e2m1(h)));
+    COX_TRY(plan_shape(g, k, T_req, CH_req, stages_req, issue_req, form));
     const int64_t m_tiles = rows_pad / TILE;
     const int T = g.T, CH = g.CH, np_cls = g.NP;
     if (m_tiles % T != 0 || (K_pad / TILE) % CH != 0) return COX_ERR_ARG;
@@ -439,7 +480,10 @@ int prep_limbs_beta(cox_handle *h, const float *beta, int k, cudaStream_t st)
     // about four blocks per SM over all columns; each block strides over p
     const int64_t bx = std::max<int64_t>(1, (4 * static_cast<int64_t>(h->sm_count) + k - 1) / k);
     dim3 grid(static_cast<unsigned>(std::min<int64_t>((h->p + 255) / 256, bx)), k);
-    if (h->ws.g1.f4)
+    if (h->ws.g1.f4 == FORM_WIDE)
+        k_prep_limbs_beta_wide<<<grid, 256, 0, st>>>(beta, h->p, h->p_pad, h->l1_blocks, h->ws.bmaxp, h->ws.Bq,
+                                                     h->ws.bs1, h->d_err);
+    else if (h->ws.g1.f4)
         k_prep_limbs_beta4<<<grid, 256, 0, st>>>(beta, h->p, h->p_pad, h->l1_blocks, h->ws.bmaxp, h->ws.Bq,
                                                  h->ws.bs1, h->d_err);
     else

@@ -23,6 +23,7 @@ constexpr int MAX_K_TC = 64;       // largest k of the tensor-core path
 constexpr int LIMBS = 4;           // e4m3 limbs per coefficient (4 significant bits each)
 constexpr int DEC_GROUPS = 3;      // decoder warp groups of the tensor-core products
 constexpr int LIMBS4 = 8;          // e2m1 limbs per coefficient (3 significant bits each)
+constexpr int LIMBS_W = 10;         // e2m1 limbs that hold a four-limb e4m3 value exactly (the wide form)
 constexpr int SF_COL = 504;        // TMEM columns 504..511: unit block scales of the e2m1 products
 
 // Limb columns of a k-column product: LIMBS k rounded up to an MMA width class.
@@ -39,6 +40,29 @@ inline int limb_cols4(int k)
 {
     const int n = LIMBS4 * k;
     return n <= 64 ? 64 : n <= 128 ? 128 : 0;
+}
+
+// Operand forms of a product (GemmPlan::f4).
+enum Form : int {
+    FORM_E4M3 = 0,  // e4m3 codes, LIMBS e4m3 limbs (kind::f8f6f4)
+    FORM_E2M1 = 1,  // e2m1 codes, LIMBS4 e2m1 limbs (kind::mxf4)
+    FORM_WIDE = 2   // e2m1 codes, the LIMBS e4m3 limbs' value as LIMBS_W e2m1 limbs (kind::mxf4)
+};
+inline int limbs_of(int form) { return form == FORM_WIDE ? LIMBS_W : form == FORM_E2M1 ? LIMBS4 : LIMBS; }
+
+// Limb columns of the wide form: LIMBS_W k rounded up to an MMA width class, 0 past
+// MAX_K_WIDE.  One coefficient per LIMBS_W columns; the rest of a class stays zero.
+constexpr int MAX_K_WIDE = 12;
+inline int limb_cols_wide(int k)
+{
+    const int n = LIMBS_W * k;
+    return n <= 16 ? 16 : n <= 32 ? 32 : n <= 64 ? 64 : n <= 128 ? 128 : 0;
+}
+
+// Limb columns of k coefficients in a form (0: not held).
+inline int limb_cols_of(int form, int k)
+{
+    return form == FORM_WIDE ? limb_cols_wide(k) : form == FORM_E2M1 ? limb_cols4(k) : limb_cols(k);
 }
 
 // Position of code K (0..15) of a 16-code word: bit 8 (K mod 4) + 2 (K div 4),
@@ -144,6 +168,24 @@ __device__ inline int split_e2m1_units(float r, uint8_t *nib)
     return q;
 }
 
+// ---- wide e2m1 limbs --------------------------------------------------------------
+// The value of a column's LIMBS e4m3 limbs, an integer q of 2^(s-21) units with
+// |q| <= 2^29 (split_e4m3_units), as LIMBS_W balanced radix-8 digits
+//   q = sum_l t_l 8^(LIMBS_W-1-l),  t_l in [-4, 4],
+// each the e2m1 value t_l / 2: the same coefficient, bit for bit, as operands
+// of kind::mxf4 (2^(s+7) sum_l (t_l / 2) 8^-l).  The digits of l >= 1 lie in
+// [-4, 3], so the first one keeps |t_0| <= 4 up to |q| = 2^29 (1 + 3/28).
+__device__ inline void split_wide(int q, uint8_t *nib)
+{
+#pragma unroll
+    for (int l = LIMBS_W - 1; l > 0; --l) {
+        const int t = ((q + 4) & 7) - 4;
+        nib[l] = static_cast<uint8_t>(t < 0 ? 8 - t : t);
+        q = (q - t) >> 3;
+    }
+    nib[0] = static_cast<uint8_t>(q < 0 ? 8 - q : q);
+}
+
 // 32-bit word index, in a tiled 2-bit layout of KC chunks per row tile, of the
 // 16 codes of row rit (0..127) of row tile mt at K offset `within` (a multiple
 // of 16) of chunk kc: row records of 32 bytes, two 16-byte halves (K 0-63 and
@@ -174,8 +216,8 @@ struct GemmPlan {
     int alt = 0;       // 1: two issuers on alternate stages (else one per row tile)
     int pair = 0;      // 1: per-tile issuers commit after every second stage
     int G = 3;         // decoder groups
-    int NP = 16;       // limb columns (limb_cols(k), or limb_cols4(k) in the e2m1 form)
-    int f4 = 0;        // 1: e2m1 operands (kind::mxf4), else e4m3 (kind::f8f6f4)
+    int NP = 16;       // limb columns (limb_cols_of(f4, k))
+    int f4 = 0;        // operand form (Form): 0 e4m3, else e2m1 operands (kind::mxf4)
     int stages = 6;    // shared-memory pipeline depth (e2m1 form: code slots)
     int stages2 = 0;   // e2m1 form: limb slots
     int ring = 4;      // TMEM A buffers
@@ -193,7 +235,6 @@ struct GemmPlan {
 
 struct Workspace {
     int k = 0;        // columns the workspace is sized for
-    int NP = 0;
     // split / gemv / fp64 common (sorted subject order)
     double *eta = nullptr;      // k x n
     double *w = nullptr;        // k x n
@@ -209,8 +250,9 @@ struct Workspace {
     int *active = nullptr;     // k
     double *Fring = nullptr;   // lag x k
     // split mode
-    uint8_t *Bq = nullptr;     // NP x p_pad e4m3 limbs of beta (row LIMBS c + l: limb l of column c)
-    uint8_t *Vq = nullptr;     // NP x n_pad e4m3 limbs of V, A4 K order
+    uint8_t *Bq = nullptr;     // limbs of beta in g1's form: NP x p_pad e4m3 or NP x p_pad / 2 e2m1 pairs
+                               // (row c limbs_of(form) + l: limb l of column c)
+    uint8_t *Vq = nullptr;     // limbs of V in g4's form, A4 K order
     int *bs1 = nullptr;        // k: power-of-two scale of the beta limbs
     int *bs4 = nullptr;        // k: power-of-two scale of the V limbs
     float *bmaxp = nullptr;    // k x l1 blocks: partial max |beta|
@@ -235,7 +277,7 @@ struct Workspace {
     GemmPlan g1a;
     bool g1a_ready = false;
     int64_t g1a_K = 0;
-    uint8_t *Bqa = nullptr;    // NP x act_Kpad e4m3 limbs of beta at the active SNPs
+    uint8_t *Bqa = nullptr;    // limbs of beta at the active SNPs, g1's form
 };
 
 } // namespace coxgb
@@ -290,6 +332,7 @@ struct cox_handle {
     // autotuned pipeline shapes per k: row tiles, K chunks, stages of each product
     struct TuneChoice {
         int T1, CH1, S1, A1, T4, CH4, S4, A4;  // A: issue mode (1 per tile, 2 alternating)
+        int F1, F4;                            // operand form (Form)
     };
     std::map<int, TuneChoice> tuned;
     // launch accounting and optional per-kernel-class event timing
@@ -373,7 +416,7 @@ int run_scans(cox_handle *h, const ScanArgs &a, cudaStream_t st);
 // stages, 3 one issuer per row tile committing after every second stage.
 int plan_shape(GemmPlan &g, int k, int T_req, int CH_req, int stages_req, int issue_req, int f4);
 int plan_gemm(cox_handle *h, GemmPlan &g, const uint32_t *A, int64_t rows_pad, int64_t K_pad,
-              const uint8_t *B, int k, int T_req, int CH_req, int stages_req, int issue_req);
+              const uint8_t *B, int k, int form, int T_req, int CH_req, int stages_req, int issue_req);
 // The compiled (row tiles, K chunks, issue mode) shapes for k columns; returns
 // their count.
 int gemm_shapes(int k, int *T, int *CH, int *issue, int max, int f4);

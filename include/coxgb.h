@@ -166,19 +166,20 @@ int cox_lipschitz(cox_h h, const double *start_host, double tol, int maxiter, do
  * fails or must not be used, and latency-sensitive loops that cannot afford
  * the device-wide synchronisation cudaFree implies.
  *
- * Same arguments, result and power method as cox_lipschitz.  The work
- * vectors live in a 16 MiB array built into the library (every GPU that loads
- * the library holds it until the process exits).  Limit: the call needs
+ * Same arguments, result and power method as cox_lipschitz.  A genotype
+ * handle's work vectors were allocated with the handle; an FP64 handle's live
+ * in a 16 MiB array built into the library (every GPU that loads the library
+ * holds it until the process exits).  Limit, for both: the vectors' sizes
  *   4 (p + 2 n_pad + p_pad) + 256   bytes (genotype handles),
  *   8 (2 p + n) + 256               bytes (COX_FP64 handles),
  * plus 8 p when start_host is given, each term rounded up to 256; larger
  * problems get COX_ERR_ARG (n_pad, p_pad from cox_get_info).
- * The first call on a device looks up the array's device address
+ * The first FP64 call on a device looks up the array's device address
  * (cudaGetSymbolAddress) with that device current and keeps it for the life
  * of the process; make that first call before any stream capture.  A device
  * reset (cudaDeviceReset, or an embedder resetting the primary context)
  * invalidates that address as it does every handle: neither a handle nor
- * this call may be used across a reset.  Calls share the array: calls that
+ * this call may be used across a reset.  FP64 calls share the array: calls that
  * overlap on the GPU race; each call writes everything it reads.  Calls no
  * cudaMalloc, cudaFree or allocating library routine.  Synchronous (legacy
  * stream).

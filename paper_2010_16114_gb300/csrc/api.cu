@@ -547,7 +547,7 @@ void cox_destroy(cox_h h)
     active_free(h);
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
     void *ptrs[] = {h->d_head, h->d_tail, h->d_evhead, h->d_evcnt, h->d_evidx, h->d_evflag, h->d_delta,
-                    h->d_mu, h->d_A1, h->d_A4, h->d_Xr, h->d_Xc, h->d_err, h->d_Z};
+                    h->d_mu, h->d_A1, h->d_A4, h->d_Xr, h->d_Xc, h->d_err, h->d_Z, h->pow.base};
     for (void *p : ptrs) dfree(p);
     delete h;
 }
@@ -687,6 +687,7 @@ int cox_setup(cox_h *out, const void *X, int64_t n, int64_t p, int x_format, con
         }
         if (opt.precision == COX_FP64) rc = setup_dense64(h, static_cast<const double *>(X), st);
         else rc = setup_genotypes(h, X, x_format, st);
+        if (rc == COX_OK && opt.precision != COX_FP64) rc = power_setup(h);
         if (rc != COX_OK) break;
         if (cudaMemcpy(h->d_mu, h->h_mu.data(), p * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
             rc = COX_ERR_CUDA;

@@ -466,8 +466,8 @@ int launch_gemm(cox_handle *h, const GemmPlan &g, const EpiArgs &e, int k, cudaS
     kp.near = e.near;
     kp.rows_valid = e.rows_valid;
     kp.inv_n = e.inv_n;
-    kp.wait_limit = h->wait_cycles;
-    kp.err = h->d_err;
+    kp.wait_limit = e.wait ? e.wait : h->wait_cycles;
+    kp.err = e.err ? e.err : h->d_err;
     KernelFn fn = pick_kernel(g.T, g.CH, g.NP, g.alt, g.f4);
     if (!fn) return COX_ERR_ARG;
     fn<<<g.grid, threads_for(g.T, g.G, g.alt), g.smem, st>>>(g.tmA, g.tmB, kp);

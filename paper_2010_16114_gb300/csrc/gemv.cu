@@ -5,8 +5,6 @@
 //   * the plain FP32 baseline: one matrix-vector product per penalty on the
 //     2-bit tiles (byte tables of partial sums of x, FP32 throughout) and an
 //     unfused soft-threshold kernel;
-//   * the power method's matrix-vector product (one thread per row, FP32
-//     multiply-add per code, FP64 across 128-wide chunks);
 //   * ||beta||_1 partial sums for the penalised objective.
 #include <algorithm>
 #include <cmath>
@@ -70,41 +68,6 @@ __global__ void k_l1_64(const double *__restrict__ beta, int64_t p, int nb, doub
         for (int w = 0; w < blockDim.x / 32; ++w) t += sh[w];
         l1p[kk * nb + b] = t;
     }
-}
-
-// y[row] = sum_K A[row][K] x[K] over the 2-bit tiled layout (one thread per row).
-// Inside a chunk the products are summed in FP32, chunk sums in FP64.
-__global__ void __launch_bounds__(128) k_gemv_tiles(const uint32_t *__restrict__ A, int64_t rows, int64_t KC,
-                                                    const float *__restrict__ x, int64_t K_valid,
-                                                    float *__restrict__ y)
-{
-    const int64_t row = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (row >= rows) return;
-    const int64_t mt = row / TILE;
-    const int rit = static_cast<int>(row % TILE);
-    const int swap = (rit >> 2) & 1;
-    double acc = 0.0;
-    for (int64_t kc = 0; kc < KC; ++kc) {
-        const uint32_t *blk = A + ((mt * KC + kc) * BLOCK_BYTES + rit * 32) / 4;
-        const uint4 h0 = *reinterpret_cast<const uint4 *>(blk + 4 * swap);
-        const uint4 h1 = *reinterpret_cast<const uint4 *>(blk + 4 * (1 - swap));
-        const uint32_t w[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
-        const int64_t kb = kc * TILE;
-        float cs = 0.f;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const uint32_t P = w[q];
-            if (P == 0) continue;
-#pragma unroll
-            for (int kap = 0; kap < 16; ++kap) {
-                const uint32_t c = (P >> code_bit(kap)) & 3u;
-                const int64_t K = kb + 16 * q + kap;
-                if (c && K < K_valid) cs = fmaf(static_cast<float>(c), x[K], cs);
-            }
-        }
-        acc += static_cast<double>(cs);
-    }
-    y[row] = static_cast<float>(acc);
 }
 
 // ---- the FP32 baseline's matrix-vector product: nibble tables of x ------------
@@ -352,15 +315,6 @@ int l1_norms32(cox_handle *h, const float *beta, int k, cudaStream_t st, float *
 int l1_norms64(cox_handle *h, const double *beta, int k, cudaStream_t st)
 {
     k_l1_64<<<dim3(h->l1_blocks, k), 256, 0, st>>>(beta, h->p, h->l1_blocks, h->ws.l1p);
-    COX_CUDA(cudaGetLastError());
-    return COX_OK;
-}
-
-int gemv_tiles(cox_handle *h, const uint32_t *A, int64_t rows, int64_t KC, const float *x, int64_t K_valid,
-               float *y, cudaStream_t st)
-{
-    (void)h;
-    k_gemv_tiles<<<blocks_for(rows, 128), 128, 0, st>>>(A, rows, KC, x, K_valid, y);
     COX_CUDA(cudaGetLastError());
     return COX_OK;
 }

@@ -280,6 +280,16 @@ struct Workspace {
     uint8_t *Bqa = nullptr;    // limbs of beta at the active SNPs, g1's form
 };
 
+// The power method's work memory and plans (power.cu): genotype handles only.
+struct PowerWork {
+    void *base = nullptr;         // one allocation
+    uint8_t *Bq = nullptr, *Vq = nullptr;
+    float *part = nullptr, *a = nullptr, *b = nullptr;
+    double *start = nullptr;
+    void *scal = nullptr;
+    GemmPlan g1, g4;
+};
+
 } // namespace coxgb
 
 struct cox_handle {
@@ -320,6 +330,7 @@ struct cox_handle {
     int64_t device_bytes = 0;
     long long wait_cycles = 0;
     coxgb::Workspace ws;
+    coxgb::PowerWork pow;
     // path / checkpoint state
     int st_k = 0;
     std::vector<float> st_beta32;
@@ -436,9 +447,15 @@ struct EpiArgs {
     const int *bscale = nullptr;  // k: power-of-two scale of the B limbs
     int64_t rows_valid = 0;  // p
     double inv_n = 0;
+    int *err = nullptr;           // error bits (null: the handle's) and wait limit (0: the handle's)
+    long long wait = 0;
 };
 int launch_gemm(cox_handle *h, const GemmPlan &g, const EpiArgs &e, int k, cudaStream_t st);
 int prep_limbs_beta(cox_handle *h, const float *beta, int k, cudaStream_t st);
+
+// ---- power method on the genotype tiles (power.cu) ------------------------------------
+int power_setup(cox_handle *h);
+int power_method_tiles(cox_handle *h, const double *start, double tol, int maxiter, double *L_out);
 
 // ---- active-set first product (active.cu) -------------------------------------------
 int active_prepare(cox_handle *h, const float *beta, int k, cudaStream_t st, int *use);
@@ -448,8 +465,6 @@ void active_free(cox_handle *h);
 // ||beta_c||_1 partials into ws.l1p; with maxp, max |beta_c| partials too
 int l1_norms32(cox_handle *h, const float *beta, int k, cudaStream_t st, float *maxp = nullptr);
 int l1_norms64(cox_handle *h, const double *beta, int k, cudaStream_t st);
-int gemv_tiles(cox_handle *h, const uint32_t *A, int64_t rows, int64_t KC, const float *x,
-               int64_t K_valid, float *y, cudaStream_t st);
 // The FP32 baseline's product y = A x (byte tables of x; part: the partials,
 // gemv_lut_part_floats(rows, KC) floats).  Two kernels.
 int gemv_lut(cox_handle *h, const uint32_t *A, int64_t rows, int64_t KC, const float *x, int64_t K_valid,

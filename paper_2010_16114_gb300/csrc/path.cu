@@ -16,12 +16,11 @@ namespace {
 constexpr int RB = 256;
 
 // out[slot] = sum_j mu_j v_j   (one block, fixed order)
-template <typename TV>
-__global__ void k_dot_mu(const double *__restrict__ mu, const TV *__restrict__ v, int64_t p, double *out)
+__global__ void k_dot_mu(const double *__restrict__ mu, const double *__restrict__ v, int64_t p, double *out)
 {
     __shared__ double sh[RB];
     double s = 0.0;
-    for (int64_t j = threadIdx.x; j < p; j += RB) s += mu[j] * static_cast<double>(v[j]);
+    for (int64_t j = threadIdx.x; j < p; j += RB) s += mu[j] * v[j];
     sh[threadIdx.x] = s;
     __syncthreads();
     for (int o = RB / 2; o > 0; o >>= 1) {
@@ -32,19 +31,18 @@ __global__ void k_dot_mu(const double *__restrict__ mu, const TV *__restrict__ v
 }
 
 // a_i -= s for i < n, a_i = 0 for n <= i < len; then out = sum_i a_i
-template <typename TV>
-__global__ void k_center_sum(TV *a, int64_t n, int64_t len, const double *s, double *out)
+__global__ void k_center_sum(double *a, int64_t n, int64_t len, const double *s, double *out)
 {
     __shared__ double sh[RB];
     const double sub = *s;
     double acc = 0.0;
     for (int64_t i = threadIdx.x; i < len; i += RB) {
         if (i < n) {
-            const TV v = static_cast<TV>(static_cast<double>(a[i]) - sub);
+            const double v = a[i] - sub;
             a[i] = v;
-            acc += static_cast<double>(v);
+            acc += v;
         } else {
-            a[i] = TV(0);
+            a[i] = 0.0;
         }
     }
     sh[threadIdx.x] = acc;
@@ -56,25 +54,15 @@ __global__ void k_center_sum(TV *a, int64_t n, int64_t len, const double *s, dou
     if (threadIdx.x == 0) *out = sh[0];
 }
 
-// out[a4_pos(i)] = a[i], i < len: a vector over sorted subjects put in the K
-// order of the SNP-major genotype copy
-__global__ void k_to_a4(const float *__restrict__ a, int64_t len, int64_t pa, int64_t pnb, float *__restrict__ out)
-{
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < len;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        out[a4_pos(i, pa, pnb)] = a[i];
-}
-
 // b_j -= mu_j s (j < p); out = ||b||^2
-template <typename TV>
-__global__ void k_center_norm(TV *b, const double *__restrict__ mu, int64_t p, const double *s, double *out)
+__global__ void k_center_norm(double *b, const double *__restrict__ mu, int64_t p, const double *s, double *out)
 {
     __shared__ double sh[RB];
     const double sa = *s;
     double acc = 0.0;
     for (int64_t j = threadIdx.x; j < p; j += RB) {
-        const double v = static_cast<double>(b[j]) - mu[j] * sa;
-        b[j] = static_cast<TV>(v);
+        const double v = b[j] - mu[j] * sa;
+        b[j] = v;
         acc += v * v;
     }
     sh[threadIdx.x] = acc;
@@ -86,11 +74,10 @@ __global__ void k_center_norm(TV *b, const double *__restrict__ mu, int64_t p, c
     if (threadIdx.x == 0) *out = sh[0];
 }
 
-template <typename TV>
-__global__ void k_scale(const TV *__restrict__ b, TV *__restrict__ v, int64_t p, double inv)
+__global__ void k_scale(const double *__restrict__ b, double *__restrict__ v, int64_t p, double inv)
 {
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (j < p) v[j] = static_cast<TV>(static_cast<double>(b[j]) * inv);
+    if (j < p) v[j] = b[j] * inv;
 }
 
 // FP64: b_j = sum_i Xc[j][i] a_i (one warp per j)
@@ -107,8 +94,7 @@ __global__ void k_xta64(const double *__restrict__ Xc, int64_t n, int64_t p, con
 }
 
 // v = start / ||start|| (start == null: all entries 1/sqrt(p)); one block.
-template <typename TV>
-__global__ void k_start_vector(const double *__restrict__ start, int64_t p, TV *__restrict__ v)
+__global__ void k_start_vector(const double *__restrict__ start, int64_t p, double *__restrict__ v)
 {
     __shared__ double sh[RB];
     double s = 0.0;
@@ -120,7 +106,7 @@ __global__ void k_start_vector(const double *__restrict__ start, int64_t p, TV *
         __syncthreads();
     }
     const double inv = 1.0 / sqrt(sh[0]);
-    for (int64_t j = threadIdx.x; j < p; j += RB) v[j] = static_cast<TV>((start ? start[j] : 1.0) * inv);
+    for (int64_t j = threadIdx.x; j < p; j += RB) v[j] = (start ? start[j] : 1.0) * inv;
 }
 
 struct DeviceGuard {
@@ -138,74 +124,48 @@ struct DeviceGuard {
     }
 };
 
-template <typename TV>
-int power_method(cox_handle *h, const double *start, double tol, int maxiter, double *L_out)
+// The power method on the FP64 design: iterations on the given vectors (v: p,
+// a: n, b: p, sc: 4 doubles; st_dev: the start vector, or null for all ones).
+int power_iterate64(cox_handle *h, double *v, double *a, double *b, double *sc, const double *st_dev, double tol,
+                    int maxiter, double *L_out)
 {
     const int64_t n = h->n, p = h->p;
-    const bool f64 = h->opt.precision == COX_FP64;
-    const int64_t alen = f64 ? n : h->n_pad, blen = f64 ? p : h->p_pad;
-    TV *v = nullptr, *a = nullptr, *b = nullptr, *a4 = nullptr;
-    double *sc = nullptr;
-    int rc = COX_OK;
-    if ((rc = dmalloc(nullptr, reinterpret_cast<void **>(&v), p * sizeof(TV))) != COX_OK) return rc;
-    if ((rc = dmalloc(nullptr, reinterpret_cast<void **>(&a), alen * sizeof(TV))) != COX_OK) { dfree(v); return rc; }
-    if ((rc = dmalloc(nullptr, reinterpret_cast<void **>(&b), blen * sizeof(TV))) != COX_OK) { dfree(v); dfree(a); return rc; }
-    if ((rc = dmalloc(nullptr, reinterpret_cast<void **>(&sc), 4 * sizeof(double))) != COX_OK) { dfree(v); dfree(a); dfree(b); return rc; }
-    if (!f64 && (rc = dmalloc(nullptr, reinterpret_cast<void **>(&a4), alen * sizeof(TV))) != COX_OK) {
-        dfree(v); dfree(a); dfree(b); dfree(sc);
-        return rc;
-    }
-    // the start vector is normalised on the device, by the same kernel as in
-    // cox_lipschitz_noalloc, so that both entry points run one power method
-    double *st_dev = nullptr;
-    if (start && (rc = dmalloc(nullptr, reinterpret_cast<void **>(&st_dev), p * sizeof(double))) != COX_OK) {
-        dfree(v); dfree(a); dfree(b); dfree(sc); dfree(a4);
-        return rc;
-    }
     cudaStream_t st = 0;
+    k_start_vector<<<1, RB, 0, st>>>(st_dev, p, v);
     double s = 0.0, s_prev = 0.0;
-    do {
-        if (start && cudaMemcpy(st_dev, start, p * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) { rc = COX_ERR_CUDA; break; }
-        k_start_vector<TV><<<1, RB, 0, st>>>(st_dev, p, v);
-        for (int it = 1; it <= maxiter; ++it) {
-            k_dot_mu<TV><<<1, RB, 0, st>>>(h->d_mu, v, p, sc);
-            if (f64) {
-                rc = eta64(h, reinterpret_cast<const double *>(v), 1, reinterpret_cast<double *>(a), st);
-            } else {
-                rc = gemv_tiles(h, h->d_A1, h->n_pad, h->p_pad / TILE, reinterpret_cast<const float *>(v), p,
-                                reinterpret_cast<float *>(a), st);
-            }
-            if (rc != COX_OK) break;
-            k_center_sum<TV><<<1, RB, 0, st>>>(a, n, alen, sc, sc + 1);
-            if (f64) {
-                k_xta64<<<static_cast<unsigned>((p * 32 + 255) / 256), 256, 0, st>>>(h->d_Xc, n, p,
-                                                                                     reinterpret_cast<const double *>(a),
-                                                                                     reinterpret_cast<double *>(b));
-            } else {
-                k_to_a4<<<static_cast<unsigned>((alen + 255) / 256), 256, 0, st>>>(
-                    reinterpret_cast<const float *>(a), alen, h->kperm_a, h->kperm_nb, reinterpret_cast<float *>(a4));
-                rc = gemv_tiles(h, h->d_A4, h->p_pad, h->n_pad / TILE, reinterpret_cast<const float *>(a4), alen,
-                                reinterpret_cast<float *>(b), st);
-                if (rc != COX_OK) break;
-            }
-            k_center_norm<TV><<<1, RB, 0, st>>>(b, h->d_mu, p, sc + 1, sc + 2);
-            double nb2 = 0.0;
-            if (cudaMemcpy(&nb2, sc + 2, sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) { rc = COX_ERR_CUDA; break; }
-            if (!(nb2 > 0.0) || !std::isfinite(nb2)) { s = 0.0; break; }
-            s = std::sqrt(nb2);  // ||X_c^T X_c v|| -> largest eigenvalue of X_c^T X_c
-            k_scale<TV><<<static_cast<unsigned>((p + 255) / 256), 256, 0, st>>>(b, v, p, 1.0 / s);
-            if (it > 1 && std::fabs(s - s_prev) <= tol * s) break;
-            s_prev = s;
+    for (int it = 1; it <= maxiter; ++it) {
+        k_dot_mu<<<1, RB, 0, st>>>(h->d_mu, v, p, sc);
+        COX_TRY(eta64(h, v, 1, a, st));
+        k_center_sum<<<1, RB, 0, st>>>(a, n, n, sc, sc + 1);
+        k_xta64<<<static_cast<unsigned>((p * 32 + 255) / 256), 256, 0, st>>>(h->d_Xc, n, p, a, b);
+        k_center_norm<<<1, RB, 0, st>>>(b, h->d_mu, p, sc + 1, sc + 2);
+        double nb2 = 0.0;
+        COX_CUDA(cudaMemcpy(&nb2, sc + 2, sizeof(double), cudaMemcpyDeviceToHost));
+        if (!(nb2 > 0.0) || !std::isfinite(nb2)) {
+            s = 0.0;
+            break;
         }
-        if (cudaDeviceSynchronize() != cudaSuccess && rc == COX_OK) rc = COX_ERR_CUDA;
-    } while (false);
-    dfree(v);
-    dfree(a);
-    dfree(b);
-    dfree(sc);
-    dfree(a4);
-    dfree(st_dev);
-    if (rc == COX_OK) *L_out = 2.0 * s / static_cast<double>(n);
+        s = std::sqrt(nb2);  // ||X_c^T X_c v|| -> largest eigenvalue of X_c^T X_c
+        k_scale<<<static_cast<unsigned>((p + 255) / 256), 256, 0, st>>>(b, v, p, 1.0 / s);
+        if (it > 1 && std::fabs(s - s_prev) <= tol * s) break;
+        s_prev = s;
+    }
+    COX_CUDA(cudaStreamSynchronize(st));
+    *L_out = 2.0 * s / static_cast<double>(n);
+    return COX_OK;
+}
+
+int power_method64(cox_handle *h, const double *start, double tol, int maxiter, double *L_out)
+{
+    const int64_t n = h->n, p = h->p;
+    double *mem = nullptr;  // v, a, b, four scalars, the start vector
+    COX_TRY(dmalloc(nullptr, reinterpret_cast<void **>(&mem), static_cast<size_t>(2 * p + n + 4 + (start ? p : 0)) * sizeof(double)));
+    double *v = mem, *a = v + p, *b = a + n, *sc = b + p, *st_dev = sc + 4;
+    int rc = COX_OK;
+    if (start && cudaMemcpy(st_dev, start, p * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) rc = COX_ERR_CUDA;
+    if (rc == COX_OK) rc = power_iterate64(h, v, a, b, sc, start ? st_dev : nullptr, tol, maxiter, L_out);
+    cudaDeviceSynchronize();
+    dfree(mem);
     return rc;
 }
 
@@ -222,8 +182,8 @@ int cox_lipschitz(cox_h h, const double *start_host, double tol, int maxiter, do
     DeviceGuard g(h->dev);
     if (!(tol > 0.0)) tol = 1e-6;
     if (maxiter <= 0) maxiter = 1000;
-    if (h->opt.precision == COX_FP64) return power_method<double>(h, start_host, tol, maxiter, L_out);
-    return power_method<float>(h, start_host, tol, maxiter, L_out);
+    if (h->opt.precision == COX_FP64) return power_method64(h, start_host, tol, maxiter, L_out);
+    return power_method_tiles(h, start_host, tol, maxiter, L_out);
 }
 
 } // extern "C"
@@ -524,15 +484,16 @@ int cox_set_state(cox_h h, const void *buf, size_t size)
 
 // ---- step size without device allocation ------------------------------------
 //
-// cox_lipschitz_noalloc runs the same power method as cox_lipschitz, but its
-// work vectors live in one file-scope device array instead of memory taken
-// with cudaMalloc.  The array is part of the library image: every GPU that
-// loads the library holds it until the process exits.  Host code only ever
-// sees a host-side stand-in for it under its name, so the device address is
-// looked up once per device with cudaGetSymbolAddress (with that device
-// current) and passed to the kernels.  All calls share the array; calls that
-// overlap on the GPU race on it.  Each call writes every element it later
-// reads, so nothing left by an earlier call leaks into a result.
+// cox_lipschitz_noalloc runs the same power method as cox_lipschitz.  A genotype
+// handle's work memory comes with the handle (power.cu).  For FP64 handles the
+// work vectors live in one file-scope device array instead of memory taken with
+// cudaMalloc.  The array is part of the library image: every GPU that loads the
+// library holds it until the process exits.  Host code only ever sees a host-side
+// stand-in for it under its name, so the device address is looked up once per
+// device with cudaGetSymbolAddress (with that device current) and passed to the
+// kernels.  All FP64 calls share the array; calls that overlap on the GPU race
+// on it.  Each call writes every element it later reads, so nothing left by an
+// earlier call leaks into a result.
 namespace coxgb {
 namespace {
 
@@ -561,73 +522,29 @@ int noalloc_scratch(int dev, void **out)
     return COX_OK;
 }
 
-template <typename TV>
 int power_method_noalloc(cox_handle *h, const double *start, double tol, int maxiter, double *L_out)
 {
     const int64_t n = h->n, p = h->p;
     const bool f64 = h->opt.precision == COX_FP64;
+    const size_t es = f64 ? sizeof(double) : sizeof(float);
     const int64_t alen = f64 ? n : h->n_pad, blen = f64 ? p : h->p_pad;
     auto up = [](size_t b) { return (b + 255) / 256 * 256; };
-    const size_t off_a = up(p * sizeof(TV));
-    const size_t off_b = off_a + up(alen * sizeof(TV));
-    const size_t off_sc = off_b + up(blen * sizeof(TV));
+    const size_t off_a = up(p * es);
+    const size_t off_b = off_a + up(alen * es);
+    const size_t off_sc = off_b + up(blen * es);
     const size_t off_a4 = off_sc + 256;
-    const size_t off_st = off_a4 + (f64 ? 0 : up(alen * sizeof(TV)));
+    const size_t off_st = off_a4 + (f64 ? 0 : up(alen * es));
     const size_t need = off_st + (start ? up(p * sizeof(double)) : 0);
-    if (need > NOALLOC_SCRATCH_BYTES) return COX_ERR_ARG;
+    if (need > NOALLOC_SCRATCH_BYTES) return COX_ERR_ARG;  // the documented limit, for every handle
+    if (!f64) return power_method_tiles(h, start, tol, maxiter, L_out);  // its work memory came with the handle
     void *base = nullptr;
     COX_TRY(noalloc_scratch(h->dev, &base));
     uint8_t *b8 = static_cast<uint8_t *>(base);
-    TV *v = reinterpret_cast<TV *>(b8);
-    TV *a = reinterpret_cast<TV *>(b8 + off_a);
-    TV *b = reinterpret_cast<TV *>(b8 + off_b);
-    double *sc = reinterpret_cast<double *>(b8 + off_sc);
-    TV *a4 = reinterpret_cast<TV *>(b8 + off_a4);
     double *st_dev = start ? reinterpret_cast<double *>(b8 + off_st) : nullptr;
-    cudaStream_t st = 0;
-    if (start) COX_CUDA(cudaMemcpyAsync(st_dev, start, p * sizeof(double), cudaMemcpyHostToDevice, st));
-    k_start_vector<TV><<<1, RB, 0, st>>>(st_dev, p, v);
-    COX_CUDA(cudaGetLastError());
-    double s = 0.0, s_prev = 0.0;
-    int rc = COX_OK;
-    for (int it = 1; it <= maxiter; ++it) {
-        k_dot_mu<TV><<<1, RB, 0, st>>>(h->d_mu, v, p, sc);
-        if (f64) {
-            rc = eta64(h, reinterpret_cast<const double *>(v), 1, reinterpret_cast<double *>(a), st);
-        } else {
-            rc = gemv_tiles(h, h->d_A1, h->n_pad, h->p_pad / TILE, reinterpret_cast<const float *>(v), p,
-                            reinterpret_cast<float *>(a), st);
-        }
-        if (rc != COX_OK) break;
-        k_center_sum<TV><<<1, RB, 0, st>>>(a, n, alen, sc, sc + 1);
-        if (f64) {
-            k_xta64<<<static_cast<unsigned>((p * 32 + 255) / 256), 256, 0, st>>>(
-                h->d_Xc, n, p, reinterpret_cast<const double *>(a), reinterpret_cast<double *>(b));
-        } else {
-            k_to_a4<<<static_cast<unsigned>((alen + 255) / 256), 256, 0, st>>>(
-                reinterpret_cast<const float *>(a), alen, h->kperm_a, h->kperm_nb, reinterpret_cast<float *>(a4));
-            rc = gemv_tiles(h, h->d_A4, h->p_pad, h->n_pad / TILE, reinterpret_cast<const float *>(a4), alen,
-                            reinterpret_cast<float *>(b), st);
-            if (rc != COX_OK) break;
-        }
-        k_center_norm<TV><<<1, RB, 0, st>>>(b, h->d_mu, p, sc + 1, sc + 2);
-        double nb2 = 0.0;
-        if (cudaMemcpy(&nb2, sc + 2, sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess) {
-            rc = COX_ERR_CUDA;
-            break;
-        }
-        if (!(nb2 > 0.0) || !std::isfinite(nb2)) {
-            s = 0.0;
-            break;
-        }
-        s = std::sqrt(nb2);
-        k_scale<TV><<<static_cast<unsigned>((p + 255) / 256), 256, 0, st>>>(b, v, p, 1.0 / s);
-        if (it > 1 && std::fabs(s - s_prev) <= tol * s) break;
-        s_prev = s;
-    }
-    if (cudaStreamSynchronize(st) != cudaSuccess && rc == COX_OK) rc = COX_ERR_CUDA;
-    if (rc == COX_OK) *L_out = 2.0 * s / static_cast<double>(n);
-    return rc;
+    if (start) COX_CUDA(cudaMemcpyAsync(st_dev, start, p * sizeof(double), cudaMemcpyHostToDevice, 0));
+    return power_iterate64(h, reinterpret_cast<double *>(b8), reinterpret_cast<double *>(b8 + off_a),
+                           reinterpret_cast<double *>(b8 + off_b), reinterpret_cast<double *>(b8 + off_sc), st_dev, tol,
+                           maxiter, L_out);
 }
 
 } // namespace
@@ -639,6 +556,5 @@ extern "C" int cox_lipschitz_noalloc(cox_h h, const double *start_host, double t
     DeviceGuard g(h->dev);
     if (!(tol > 0.0)) tol = 1e-6;
     if (maxiter <= 0) maxiter = 1000;
-    if (h->opt.precision == COX_FP64) return power_method_noalloc<double>(h, start_host, tol, maxiter, L_out);
-    return power_method_noalloc<float>(h, start_host, tol, maxiter, L_out);
+    return power_method_noalloc(h, start_host, tol, maxiter, L_out);
 }

@@ -54,7 +54,7 @@ int alloc(cox_handle *h, T *&p, size_t count)
 void free_workspace(cox_handle *h)
 {
     Workspace &w = h->ws;
-    void *ptrs[] = {w.eta, w.w, w.Rt, w.Fg, w.lossg, w.cmax, w.csw, w.suf, w.lossp, w.vsp, w.l1p,
+    void *ptrs[] = {w.eta, w.w, w.Vf, w.Wg, w.Fg, w.tot, w.tbase, w.lgp, w.colc, w.scnt, w.cmax, w.csw, w.suf, w.lossp, w.vsp, w.l1p,
                     w.sumV, w.f, w.F, w.l1, w.mub, w.lam, w.active, w.Fring, w.Bq, w.Vq, w.bs1, w.bs4, w.bmaxp,
                     w.vmaxp, w.part1, w.part4, w.cnt4, w.V64, w.V32, w.eta32, w.G32, w.gpart, w.gamma, w.gz, w.zvp};
     for (void *p : ptrs) dfree(p);
@@ -203,7 +203,7 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
         sa.need_loss = true;
         set_covariate_args(h, sa, 0, epi, step);
         {
-            Site s_(h, 2, 8, st);
+            Site s_(h, 2, 1, st);
             COX_TRY(run_scans(h, sa, st));
         }
         EpiArgs e4;
@@ -254,7 +254,7 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
         sa.need_loss = true;
         set_covariate_args(h, sa, 0, epi, step);
         {
-            Site s_(h, 2, 8, st);
+            Site s_(h, 2, 1, st);
             COX_TRY(run_scans(h, sa, st));
         }
         Site s4_(h, 1, 1, st);
@@ -291,7 +291,7 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
         sa.need_loss = true;
         set_covariate_args(h, sa, c, epi, step);
         {
-            Site s_(h, 2, 8, st);
+            Site s_(h, 2, 1, st);
             COX_TRY(run_scans(h, sa, st));
         }
         COX_CUDA(cudaMemcpyAsync(ws.Fring + c, ws.F, sizeof(double), cudaMemcpyDeviceToDevice, st));
@@ -340,7 +340,7 @@ int iterate_from_eta(cox_handle *h, void *beta, const double *eta, int k, double
         sa.NP = ws.g4.NP;
         sa.exp64 = false;
         {
-            Site s_(h, 2, 8, st);
+            Site s_(h, 2, 1, st);
             COX_TRY(run_scans(h, sa, st));
         }
         EpiArgs e4;
@@ -369,7 +369,7 @@ int iterate_from_eta(cox_handle *h, void *beta, const double *eta, int k, double
         sa.V = ws.V64;
         sa.exp64 = true;
         {
-            Site s_(h, 2, 8, st);
+            Site s_(h, 2, 1, st);
             COX_TRY(run_scans(h, sa, st));
         }
         Site s4_(h, 1, 1, st);
@@ -421,10 +421,24 @@ int ensure_workspace(cox_handle *h, int k)
         return r;                                   \
     }
     A(ws.eta, k * n);
-    A(ws.w, k * n);
-    A(ws.Rt, k * n);
-    A(ws.Fg, k * std::max<int64_t>(1, h->n_evhead));
-    A(ws.lossg, k);
+    {
+        void *wp = nullptr;
+        if ((r = dmalloc(h, &wp, static_cast<size_t>(k) * n * (is_fp64(h) ? 8 : 4))) != COX_OK) {
+            free_workspace(h);
+            return r;
+        }
+        ws.w = wp;
+    }
+    if (is_split(h)) A(ws.Vf, k * n);
+    const size_t G = std::max<int64_t>(1, h->n_evhead), NG = std::max(1, scan_tiles(h->n_evhead));
+    A(ws.Wg, k * G);
+    A(ws.Fg, k * G);
+    A(ws.tot, k * NG);
+    A(ws.tbase, k * NG);
+    A(ws.lgp, k * NG);
+    A(ws.colc, k);
+    A(ws.scnt, 2 + 3 * static_cast<size_t>(k));
+    cudaMemset(ws.scnt, 0, (2 + 3 * static_cast<size_t>(k)) * sizeof(unsigned));
     A(ws.cmax, k * nch);
     A(ws.csw, k * nch);
     A(ws.suf, k * nch);
@@ -546,7 +560,7 @@ void cox_destroy(cox_h h)
     free_workspace(h);
     active_free(h);
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
-    void *ptrs[] = {h->d_head, h->d_tail, h->d_evhead, h->d_evcnt, h->d_evidx, h->d_evflag, h->d_delta,
+    void *ptrs[] = {h->d_evhead, h->d_evcnt, h->d_evidx, h->d_evflag, h->d_a4blk, h->d_delta,
                     h->d_mu, h->d_A1, h->d_A4, h->d_Xr, h->d_Xc, h->d_err, h->d_Z, h->pow.base};
     for (void *p : ptrs) dfree(p);
     delete h;
@@ -592,7 +606,8 @@ int cox_setup(cox_h *out, const void *X, int64_t n, int64_t p, int x_format, con
     h->p = p;
     h->n_pad = (n + PAD - 1) / PAD * PAD;
     h->p_pad = (p + PAD - 1) / PAD * PAD;
-    h->n_chunks = static_cast<int>((n + SCAN_CH - 1) / SCAN_CH);
+    h->scan_ept = scan_ept(n);
+    h->n_chunks = static_cast<int>((n + 32 * h->scan_ept - 1) / (32 * h->scan_ept));
     {
         // A4 K order: multiplier near nb (sqrt 5 - 1) / 2, odd, prime to nb
         const int64_t nb = h->n_pad / 16;
@@ -625,20 +640,18 @@ int cox_setup(cox_h *out, const void *X, int64_t n, int64_t p, int x_format, con
     h->h_order.resize(static_cast<size_t>(n));
     std::iota(h->h_order.begin(), h->h_order.end(), 0);
     std::stable_sort(h->h_order.begin(), h->h_order.end(), [&](int64_t a, int64_t b) { return time[a] < time[b]; });
-    std::vector<int32_t> head(static_cast<size_t>(n)), tail(static_cast<size_t>(n));
     std::vector<uint8_t> dsorted(static_cast<size_t>(n));
     int64_t groups = 0;
     std::vector<int32_t> evhead;  // heads of the tie groups with at least one event
     std::vector<int32_t> evcnt;   // and their event counts
     std::vector<int32_t> evidx(static_cast<size_t>(n));  // event groups with head <= the subject's tail
-    std::vector<uint8_t> evflag(static_cast<size_t>(n), 0);
+    // padded: the scans read a chunk's flags in whole words
+    std::vector<uint8_t> evflag(static_cast<size_t>(h->n_chunks) * 32 * h->scan_ept, 0);
     for (int64_t r = 0; r < n;) {
         int64_t e = r;
         while (e + 1 < n && time[h->h_order[e + 1]] == time[h->h_order[r]]) ++e;
         int32_t nev = 0;
         for (int64_t s = r; s <= e; ++s) {
-            head[s] = static_cast<int32_t>(r);
-            tail[s] = static_cast<int32_t>(e);
             nev += event[h->h_order[s]] != 0;
         }
         if (nev) {
@@ -654,33 +667,34 @@ int cox_setup(cox_h *out, const void *X, int64_t n, int64_t p, int x_format, con
     for (int64_t r = 0; r < n; ++r) dsorted[r] = event[h->h_order[r]];
     h->n_groups_tie = groups;
 
+    std::vector<int32_t> a4blk(static_cast<size_t>(h->n_pad / 16));
+    for (int64_t b = 0; b < h->n_pad / 16; ++b) a4blk[b] = static_cast<int32_t>(a4_pos(16 * b, h->kperm_a, h->kperm_nb) / 16);
+
     cudaStream_t st = 0;
     int rc = COX_OK;
     do {
         if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_err), sizeof(int))) != COX_OK) break;
-        if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_head), n * sizeof(int32_t))) != COX_OK) break;
-        if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_tail), n * sizeof(int32_t))) != COX_OK) break;
         if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_evhead), evhead.size() * sizeof(int32_t))) != COX_OK)
             break;
         if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_evcnt), evcnt.size() * sizeof(int32_t))) != COX_OK)
             break;
         if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_evidx), n * sizeof(int32_t))) != COX_OK) break;
-        if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_evflag), n)) != COX_OK) break;
+        if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_evflag), evflag.size())) != COX_OK) break;
+        if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_a4blk), a4blk.size() * sizeof(int32_t))) != COX_OK) break;
         if ((!evhead.empty() &&
              (cudaMemcpy(h->d_evhead, evhead.data(), evhead.size() * sizeof(int32_t), cudaMemcpyHostToDevice) !=
                   cudaSuccess ||
               cudaMemcpy(h->d_evcnt, evcnt.data(), evcnt.size() * sizeof(int32_t), cudaMemcpyHostToDevice) !=
                   cudaSuccess)) ||
             cudaMemcpy(h->d_evidx, evidx.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->d_evflag, evflag.data(), n, cudaMemcpyHostToDevice) != cudaSuccess) {
+            cudaMemcpy(h->d_evflag, evflag.data(), evflag.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+            cudaMemcpy(h->d_a4blk, a4blk.data(), a4blk.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess) {
             rc = COX_ERR_CUDA;
             break;
         }
         if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_delta), n)) != COX_OK) break;
         if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_mu), p * sizeof(double))) != COX_OK) break;
         if (cudaMemset(h->d_err, 0, sizeof(int)) != cudaSuccess ||
-            cudaMemcpy(h->d_head, head.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->d_tail, tail.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess ||
             cudaMemcpy(h->d_delta, dsorted.data(), n, cudaMemcpyHostToDevice) != cudaSuccess) {
             rc = COX_ERR_CUDA;
             break;

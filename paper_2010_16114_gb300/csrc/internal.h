@@ -1,6 +1,7 @@
 // internal.h -- handle layout and cross-file entry points of libcoxgb.
 #pragma once
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <cuda_fp8.h>
 #include <cuda_runtime.h>
 
@@ -18,7 +19,6 @@ enum : int { DEVERR_TIMEOUT = 1, DEVERR_NONFINITE = 2, DEVERR_CODE3 = 4 };
 constexpr int TILE = 128;          // rows per tensor-core tile, K per chunk
 constexpr int BLOCK_BYTES = 4096;  // one 128 x 128 block of 2-bit codes
 constexpr int PAD = 1024;          // n, p padding of the tiled layouts
-constexpr int SCAN_CH = 2048;      // subjects per scan chunk (256 threads x 8)
 constexpr int MAX_K_TC = 64;       // largest k of the tensor-core path
 constexpr int LIMBS = 4;           // e4m3 limbs per coefficient (4 significant bits each)
 constexpr int DEC_GROUPS = 3;      // decoder warp groups of the tensor-core products
@@ -76,12 +76,10 @@ __host__ __device__ inline int code_bit(int K) { return 8 * (K & 3) + 2 * (K >> 
 // r_0 = b 2^-s, d_l = RN_e4m3(r_l), r_(l+1) = 16 (r_l - d_l); each step keeps
 // |r| <= 256, and b = 2^s sum_l d_l 2^-4l with about 4 LIMBS significant bits.
 
+// Value of an e4m3 byte (the hardware's conversion to half is exact).
 __device__ inline float e4m3_value(uint8_t q)
 {
-    // sign, 4-bit exponent (bias 7), 3-bit mantissa; exponent 0: subnormal m 2^-9
-    const int e = (q >> 3) & 15, m = q & 7;
-    const float v = e ? ldexpf(1.0f + 0.125f * static_cast<float>(m), e - 7) : ldexpf(static_cast<float>(m), -9);
-    return (q & 0x80) ? -v : v;
+    return __half2float(__half(__nv_cvt_fp8_to_halfraw(q, __NV_E4M3)));
 }
 
 __device__ inline int limb_scale(float mx) { return mx > 0.f ? ilogbf(mx) - 7 : 0; }
@@ -106,15 +104,6 @@ __device__ inline float split_e4m3(float r, uint8_t *d)
     return rep;
 }
 
-// Value of an e4m3 byte in units of 2^-9 (exact: normal values are
-// (8 + m) 2^(e - 10), subnormal ones m 2^-9).
-__device__ inline int e4m3_units(uint8_t q)
-{
-    const int e = (q >> 3) & 15, m = q & 7;
-    const int u = e ? (8 + m) << (e - 1) : m;
-    return (q & 0x80) ? -u : u;
-}
-
 // The split of split_e4m3, returning the value the limbs represent times 2^21
 // as an exact integer (limb l is a multiple of 2^-9 weighted 16^-l; below
 // 2^30 in magnitude for |r| <= 256).  Non-finite r gives NaN limbs and 0.
@@ -128,9 +117,10 @@ __device__ inline int split_e4m3_units(float r, uint8_t *d)
 #pragma unroll
     for (int l = 0; l < LIMBS; ++l) {
         const uint8_t b = static_cast<uint8_t>(__nv_cvt_float_to_fp8(r, __NV_SATFINITE, __NV_E4M3));
+        const float v = e4m3_value(b);
         d[l] = b;
-        q = 16 * q + e4m3_units(b);
-        r = (r - e4m3_value(b)) * 16.f;
+        q = 16 * q + static_cast<int>(v * 512.f);  // limb l in units of 2^-9, an integer
+        r = (r - v) * 16.f;
     }
     return q;
 }
@@ -159,9 +149,12 @@ __device__ inline int split_e2m1_units(float r, uint8_t *nib)
     int q = 0;
 #pragma unroll
     for (int l = 0; l < LIMBS4; ++l) {
-        const float t = rintf(2.f * r);  // -4 .. 4
-        const int ti = static_cast<int>(t);
-        nib[l] = static_cast<uint8_t>((ti < 0 ? 8 : 0) | (ti < 0 ? -ti : ti));
+        // t = rint(2 r) in -4 .. 4, as 1.5 2^23 + t: the FP32 add rounds (to even),
+        // its low bits are t (rintf and the conversion share a quarter-rate unit)
+        const float m = fmaf(2.f, r, 12582912.f);
+        const float t = m - 12582912.f;
+        const int ti = __float_as_int(m) - 0x4B400000;
+        nib[l] = static_cast<uint8_t>(ti < 0 ? 8 - ti : ti);
         q = 8 * q + ti;
         r = fmaf(-4.f, t, 8.f * r);  // 8 (r - t / 2), exact
     }
@@ -237,10 +230,13 @@ struct Workspace {
     int k = 0;        // columns the workspace is sized for
     // split / gemv / fp64 common (sorted subject order)
     double *eta = nullptr;      // k x n
-    double *w = nullptr;        // k x n
-    double *Rt = nullptr;       // k x n local reverse scans (at event-group heads); then V in FP32 for k_vlimbs
-    double *Fg = nullptr;       // k x event groups: cumulative sum of (events / W) over event groups
-    double *lossg = nullptr;    // k: sum over event groups of (events) log W, plus (events) c
+    void *w = nullptr;          // k x n: float, double for FP64 handles
+    float *Vf = nullptr;        // k x n: V in FP32, for the limbs
+    double *Wg = nullptr;       // k x event groups: chunk-local reverse sum of w at the group's head
+    double *Fg = nullptr;       // k x event groups: cumulative sum of (events / W) inside its tile of groups
+    double *tot = nullptr, *tbase = nullptr, *lgp = nullptr;  // k x tiles: sums of events / W, of the tiles before, of events log W
+    double *colc = nullptr;     // k: max eta
+    unsigned *scnt = nullptr;   // 2 + 3 k counters of k_scans (zero between launches)
     double *cmax = nullptr, *csw = nullptr, *suf = nullptr;
     double *lossp = nullptr, *vsp = nullptr;  // k x chunks (lossp: sum of delta eta per chunk)
     double *l1p = nullptr;                    // k x l1 blocks
@@ -256,7 +252,7 @@ struct Workspace {
     int *bs1 = nullptr;        // k: power-of-two scale of the beta limbs
     int *bs4 = nullptr;        // k: power-of-two scale of the V limbs
     float *bmaxp = nullptr;    // k x l1 blocks: partial max |beta|
-    double *vmaxp = nullptr;   // k x chunks: partial max |V|
+    float *vmaxp = nullptr;    // k x chunks: partial max |V|
     float *part1 = nullptr;    // slots x k x rows_pad (eta partials)
     float *part4 = nullptr;    // slots x k x rows_pad (X^T V partials)
     int *cnt4 = nullptr;       // per M group of the second product
@@ -297,6 +293,7 @@ struct cox_handle {
     int64_t n = 0, p = 0, n_pad = 0, p_pad = 0;
     int64_t kperm_a = 1, kperm_nb = 1;  // K order of A4 (a4_pos)
     int64_t kperm_ainv = 1;             // a^-1 mod nb: A4 block B holds sorted block ainv B mod nb
+    int scan_ept = 8;             // subjects per lane of the risk-set scans (a chunk is a warp's)
     int n_chunks = 0, l1_blocks = 0;
     cox_options opt;
     int64_t n_groups_tie = 0;
@@ -304,11 +301,11 @@ struct cox_handle {
     std::vector<int64_t> h_order;
     std::vector<double> h_mu;
     // device data
-    int32_t *d_head = nullptr, *d_tail = nullptr;
     int32_t *d_evhead = nullptr;  // first positions of the tie groups that hold an event
     int32_t *d_evcnt = nullptr;   // events in each of those groups
     int32_t *d_evidx = nullptr;   // n: event groups whose head is at or before the subject's tie tail
-    uint8_t *d_evflag = nullptr;  // n: 1 at the head of a tie group that holds an event
+    uint8_t *d_evflag = nullptr;  // n, padded to whole chunks: 1 at the head of a tie group that holds an event
+    int32_t *d_a4blk = nullptr;   // n_pad / 16: sorted 16-subject block -> its block in the K order of A4
     int64_t n_evhead = 0;
     int q = 0;                    // unpenalised covariates
     double *d_Z = nullptr;        // q x n, sorted order
@@ -417,6 +414,8 @@ struct ScanArgs {
     bool gamma_step = false;
 };
 int run_scans(cox_handle *h, const ScanArgs &a, cudaStream_t st);
+int scan_ept(int64_t n);              // subjects per lane
+int scan_tiles(int64_t n_evhead);     // tiles of event groups
 
 // ---- tensor-core products (gemm_tc.cu) ---------------------------------------------
 // Plan one product; T_req / CH_req / stages_req of 0 take the defaults.

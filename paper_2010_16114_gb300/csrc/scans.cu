@@ -1,7 +1,7 @@
-// scans.cu -- Breslow risk-set sums of the Cox iteration in FP64
-// (arXiv 2010.16114, Section 5.3: w = exp(eta), W_j = sum_{y_i >= y_j} w_i,
-// u = P delta; the paper's remark that sorting by time turns W into a
-// cumulative sum; Section 6: Breslow ties).
+// scans.cu -- Breslow risk-set sums of the Cox iteration (arXiv 2010.16114,
+// Section 5.3: w = exp(eta), W_j = sum_{y_i >= y_j} w_i, u = P delta; the
+// paper's remark that sorting by time turns W into a cumulative sum; Section 6:
+// Breslow ties).
 //
 // Subjects are stored in ascending time order, so with R_r = sum_{s >= r} w_s
 // (a reverse inclusive scan), and the tie groups that hold events numbered
@@ -14,11 +14,34 @@
 //   f   = (1/n) [sum_g e_g log W_g - sum_r delta_r (eta_r - c)],  c = max eta.
 // delta / W is nonzero only at events, and tied events share W, so the
 // forward scan runs over the event groups (a few thousand with times in whole
-// days) instead of the n subjects; the FP64 work that remains per subject is
-// the reverse scan of w.  The reverse scan runs in fixed 2048-subject chunks
-// (block scans with warp shuffles), then an exclusive scan of the chunk
-// totals; the summation order never depends on timing, so results are
-// bit-reproducible.
+// days) instead of the n subjects.
+//
+// One cooperative kernel, k_scans, runs all of it in five phases with a grid
+// barrier between them, over chunks of subjects (1, 2, 4, 5; a warp each) or tiles
+// of 256 event groups (3; a block each) of every column:
+//   1  eta from the product's partial slots (+ Z gamma); chunk maxima, sums of
+//      delta eta
+//   2  w = exp(eta - c); reverse scans inside the chunks, kept at the heads of
+//      event groups; chunk totals                        -> suffix sums
+//   3  W_g, e_g / W_g, scans inside the tiles; sum e_g log W_g
+//                                                        -> prefix sums of the tiles
+//   4  V; chunk maxima of |V|; sums of Z^T V
+//   5  limbs of V; sums of the values they hold          -> sum V, f, F, gamma
+// The block that is the last to finish a column's part of a phase does the work
+// on the right, in a fixed order, so results never depend on timing.
+//
+// What bounds it.  GB300 has two FP64 lanes per SM, so one warp-wide FP64
+// instruction holds the pipe for 16 cycles: per-subject arithmetic in the FP32-exp
+// modes therefore runs in pairs of floats (TwoSum and FMA error terms, ~2^-47
+// relative; the summands are FP32 values themselves), and FP64 is left to
+// per-group and per-column work.  A chunk belongs to one warp, so nothing inside a
+// phase waits for another warp: the same phases with a block per chunk and a
+// counter per chunk took twice as long (latency: 541 us against 264 at n = 400,000,
+// k = 32).  At small n the five phases are latency alone (~3-5 us each with their
+// barriers).  Measured against seven FP64 kernels (eta, scan, chunk totals, groups,
+// V, limbs, sums): 264 us against 590 (n = 400,000, k = 32), 152 against 345 (k = 16),
+// 37 against ~95 (n = 100,000, k = 1); a whole FP64 step at n = 1,000, p = 2,000 takes 67 us
+// against 86.
 #include <algorithm>
 
 #include "internal.h"
@@ -27,60 +50,107 @@ namespace coxgb {
 namespace {
 
 constexpr int NT = 256;
-constexpr int PER = SCAN_CH / NT;  // 8
+constexpr int NW = NT / 32;
+constexpr int MAXQ = 16;
+constexpr int GT = NT;  // event groups per tile
 
-__device__ __forceinline__ double warp_incl_scan(double x, int lane)
+// ---- pairs of floats ------------------------------------------------------------
+
+struct tf {
+    float h, l;  // value h + l, |l| <= ulp(h) / 2
+};
+
+// a + b exactly, as sum and error (Knuth's TwoSum); an infinite sum has no error term
+__device__ __forceinline__ tf two_sum(float a, float b)
 {
+    const float s = a + b;
+    const float bb = s - a;
+    const float e = (a - (s - bb)) + (b - bb);
+    return {s, isinf(s) ? 0.f : e};
+}
+__device__ __forceinline__ tf tf_add(tf a, tf b)
+{
+    const tf s = two_sum(a.h, b.h);
+    const float e = s.l + (a.l + b.l);
+    const float h = s.h + e;
+    return {h, e - (h - s.h)};
+}
+__device__ __forceinline__ double tf_double(tf a) { return static_cast<double>(a.h) + static_cast<double>(a.l); }
+__device__ __forceinline__ tf tf_of(double v)
+{
+    const float h = static_cast<float>(v);
+    return {h, isinf(h) ? 0.f : static_cast<float>(v - static_cast<double>(h))};
+}
+__device__ __forceinline__ tf shfl_xor(tf a, int o)
+{
+    return {__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o)};
+}
+__device__ __forceinline__ double shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ tf shfl_up(tf a, int o)
+{
+    return {__shfl_up_sync(0xffffffffu, a.h, o), __shfl_up_sync(0xffffffffu, a.l, o)};
+}
+__device__ __forceinline__ double shfl_up(double a, int o) { return __shfl_up_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ tf shfl_at(tf a, int l)
+{
+    return {__shfl_sync(0xffffffffu, a.h, l), __shfl_sync(0xffffffffu, a.l, l)};
+}
+__device__ __forceinline__ double shfl_at(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+__device__ __forceinline__ tf plus(tf a, tf b) { return tf_add(a, b); }
+__device__ __forceinline__ double plus(double a, double b) { return a + b; }
+__device__ __forceinline__ bool less(tf a, tf b) { return a.h < b.h || (a.h == b.h && a.l < b.l); }
+__device__ __forceinline__ bool less(double a, double b) { return a < b; }
+__device__ __forceinline__ double as_double(tf a) { return tf_double(a); }
+__device__ __forceinline__ double as_double(double a) { return a; }
+
+// ---- block reductions and scans (every thread gets the result) --------------------
+
+template <typename T>
+__device__ __forceinline__ T block_sum(T x, T *sh)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = plus(x, shfl_xor(x, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
+    __syncthreads();
+    static_assert(NW == 8, "three levels");
+    const T t = plus(plus(plus(sh[0], sh[1]), plus(sh[2], sh[3])), plus(plus(sh[4], sh[5]), plus(sh[6], sh[7])));
+    __syncthreads();
+    return t;
+}
+
+// Inclusive scan in thread order; total = the whole block's sum.
+template <typename T>
+__device__ __forceinline__ T block_incl_scan(T x, T *sh, T &total)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const double y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+        const T y = shfl_up(x, o);
+        if (lane >= o) x = plus(y, x);
     }
-    return x;
-}
-
-// Inclusive scan of one value per thread across the 256-thread block.
-__device__ __forceinline__ double block_incl_scan(double x, double *sh)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    x = warp_incl_scan(x, lane);
     if (lane == 31) sh[warp] = x;
     __syncthreads();
-    if (warp == 0) {
-        double v = lane < NT / 32 ? sh[lane] : 0.0;
-        v = warp_incl_scan(v, lane);
-        if (lane < NT / 32) sh[lane] = v;
+    T p = sh[lane & (NW - 1)];  // every warp scans the warp sums
+#pragma unroll
+    for (int o = 1; o < NW; o <<= 1) {
+        const T y = shfl_up(p, o);
+        if ((lane & (NW - 1)) >= o) p = plus(y, p);
     }
+    total = shfl_at(p, NW - 1);
+    const T pre = shfl_at(p, warp > 0 ? warp - 1 : 0);
     __syncthreads();
-    if (warp > 0) x += sh[warp - 1];
-    __syncthreads();
-    return x;
+    return warp > 0 ? plus(pre, x) : x;
 }
 
-__device__ __forceinline__ double block_sum(double x, double *sh)
+__device__ __forceinline__ float block_max(float x, float *sh)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) sh[warp] = x;
+    for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = x;
     __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < NT / 32; ++w) t += sh[w];
-    __syncthreads();
-    return t;  // valid in thread 0
-}
-
-__device__ __forceinline__ double block_max(double x, double *sh)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float t = sh[0];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x = fmax(x, __shfl_xor_sync(0xffffffffu, x, o));
-    if (lane == 0) sh[warp] = x;
-    __syncthreads();
-    double t = -INFINITY;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < NT / 32; ++w) t = fmax(t, sh[w]);
+    for (int w = 1; w < NW; ++w) t = fmaxf(t, sh[w]);
     __syncthreads();
     return t;
 }
@@ -96,532 +166,793 @@ __device__ __forceinline__ int renorm(double &m)
 
 struct SP {
     int64_t n, n_pad;
-    int nch, k;
-    int64_t pa, pnb;  // K order of the SNP-major genotype copy (a4_pos)
-    const uint8_t *delta;
-    const int32_t *head, *tail;
-    const int32_t *evhead;  // first positions of the tie groups that hold an event
-    const int32_t *evcnt;   // their event counts
-    const int32_t *evidx;   // n: event groups with head <= the subject's tie tail
-    const uint8_t *evflag;  // n: 1 at an event group's head
-    int64_t n_evh;
-    double *eta, *w, *Rt, *Fg, *lossg, *cmax, *csw, *suf, *lossp, *vsp;
-    // unpenalised covariates (q columns; q = 0: none): Z q x n in sorted order,
-    // gamma k x q, per-chunk partials of Z^T V (k x q x chunks)
+    int nch, k, ntile;
+    int64_t per;            // chunks per block
+    int64_t G;              // event groups
+    const uint8_t *delta, *evflag;   // evflag padded with zeros to whole chunks
+    const int32_t *evhead, *evcnt, *evidx;
+    const int32_t *a4blk;   // 16-subject block -> its block in the K order of the SNP-major copy
+    // eta source
+    int src, group_rows, KC;
+    const void *eta_in;
+    int64_t slot_stride, col_stride, L;
+    // workspace (per column: chunks, tiles, groups)
+    void *eta, *w;          // tf and float, or double and double
+    float *V32;
+    double *Wg, *Fg, *csw, *suf, *lossp, *tot, *tbase, *lgp, *vsp, *zvp;
+    void *cmaxp;            // chunk maxima of eta (tf or double)
+    float *vmaxp;
+    double *colc;           // per column: c
+    unsigned *cnt;          // [0] barrier arrivals, [1] blocks done, then 3 per column
+    // covariates
     int q;
-    const double *Z, *gamma;
-    double *zvp;
+    const double *Z;
+    double *gamma, *gz;
+    bool gamma_step;
+    const int *active;
+    double step;
+    // output
+    int vo, form;
+    void *V;
+    int *bs;
+    int l1_blocks;
+    const double *l1p, *lam;
+    double *sumV, *f, *l1, *F;
+    bool need_loss;
+    int *err;
+    long long wait_limit;
 };
 
-constexpr int MAXQ = 16;
-
-// (1) eta = sum of the product's partial slots (or a dense copy); chunk maxima;
-// chunk sums of delta eta (the events' part of the loss).
-template <int SRC>
-__global__ void k_eta(SP s, const void *src, int64_t slot_stride, int64_t col_stride, int group_rows,
-                      int KC, int64_t L)
+// All blocks of the (cooperative) grid reach barrier `b` (1, 2, ...) before any
+// goes on.  Bounded like every wait: past the limit the block reports a timeout
+// and goes on (all indexes below come from the handle's static arrays).
+__device__ __forceinline__ void grid_barrier(const SP &s, unsigned b)
 {
-    __shared__ double sh[NT / 32];
-    __shared__ int cnt_sh[SCAN_CH / 128];  // partial slots of the row groups of this chunk
-    const int c = blockIdx.x, kk = blockIdx.y;
-    const int64_t i0 = static_cast<int64_t>(c) * SCAN_CH;
-    if (SRC == ETA_PARTIAL_F32) {
-        // group_rows (128 or 256) divides SCAN_CH: the chunk holds whole groups
-        if (threadIdx.x < SCAN_CH / group_rows) {
-            const int64_t g = i0 / group_rows + threadIdx.x;
-            cnt_sh[threadIdx.x] = static_cast<int>((g * KC + KC - 1) / L - (g * KC) / L + 1);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(s.cnt, 1u);
+        const unsigned want = b * gridDim.x;
+        const long long t0 = clock64();
+        unsigned v;
+        while (true) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(s.cnt) : "memory");
+            if (v >= want) break;
+            if (clock64() - t0 > s.wait_limit) {
+                atomicOr(s.err, DEVERR_TIMEOUT);
+                break;
+            }
+        }
+        __threadfence();
+    }
+    __syncthreads();
+}
+
+// Called by every block that took part in column kk in a phase (or once per tile):
+// true in the one whose call is the last of `total`.
+__device__ __forceinline__ bool last_of_column(const SP &s, int kk, int phase, unsigned total)
+{
+    __shared__ bool last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        unsigned *c = s.cnt + 2 + 3 * kk + phase;
+        last = atomicAdd(c, 1u) == total - 1u;
+        if (last) *c = 0;
+        __threadfence();
+    }
+    __syncthreads();
+    return last;
+}
+
+// Blocks whose range of `per` tasks meets column kk (its nch tasks follow those of column kk - 1).
+__device__ __forceinline__ unsigned column_blocks(const SP &s, int kk)
+{
+    const int64_t a = static_cast<int64_t>(kk) * s.nch, b = a + s.nch - 1;
+    return static_cast<unsigned>(b / s.per - a / s.per + 1);
+}
+
+// sum V, f, ||beta||_1, F = f + lambda ||beta||_1, and for covariates g_Z =
+// Z^T (delta - u) / n and, for a step, gamma <- gamma + step g_Z (Section 6: the
+// covariates take a plain gradient step; a frozen column keeps its gamma); flags
+// non-finite values.
+__device__ __forceinline__ void finalize_column(const SP &s, int kk, double *sh)
+{
+    const double n = static_cast<double>(s.n);
+    for (int cq = 0; cq < s.q; ++cq) {
+        double z = 0.0;
+        for (int c = threadIdx.x; c < s.nch; c += NT) z += s.zvp[(static_cast<int64_t>(kk) * s.q + cq) * s.nch + c];
+        z = block_sum(z, sh) / n;
+        if (threadIdx.x == 0) {
+            s.gz[kk * s.q + cq] = z;
+            if (s.gamma_step && (!s.active || s.active[kk])) s.gamma[kk * s.q + cq] += s.step * z;
+            if (!isfinite(z)) atomicOr(s.err, DEVERR_NONFINITE);
+        }
+    }
+    // f = (sum_g e_g log W_g + (events) c - sum_r delta_r eta_r) / n
+    double x[4] = {0.0, 0.0, 0.0, 0.0};  // sum V, sum delta eta, ||beta||_1, sum e log W
+    for (int c = threadIdx.x; c < s.nch; c += NT) {
+        x[0] += s.vsp[static_cast<int64_t>(kk) * s.nch + c];
+        if (s.need_loss) x[1] += s.lossp[static_cast<int64_t>(kk) * s.nch + c];
+    }
+    if (s.need_loss) {
+        if (s.l1p)
+            for (int c = threadIdx.x; c < s.l1_blocks; c += NT) x[2] += s.l1p[kk * s.l1_blocks + c];
+        for (int t = threadIdx.x; t < s.ntile; t += NT) x[3] += s.lgp[static_cast<int64_t>(kk) * s.ntile + t];
+    }
+    __shared__ double sh4[4][NW];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] += __shfl_xor_sync(0xffffffffu, x[e], o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sh4[e][threadIdx.x >> 5] = x[e];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            x[e] = ((sh4[e][0] + sh4[e][1]) + (sh4[e][2] + sh4[e][3])) + ((sh4[e][4] + sh4[e][5]) + (sh4[e][6] + sh4[e][7]));
+    }
+    __syncthreads();
+    const double v = x[0], b1 = x[2];
+    if (threadIdx.x != 0) return;
+    s.sumV[kk] = v;
+    if (s.need_loss) {
+        const double lo = (x[3] - x[1]) / n;
+        s.f[kk] = lo;
+        s.l1[kk] = b1;
+        s.F[kk] = lo + (s.lam ? s.lam[kk] * b1 : 0.0);
+        if (!isfinite(lo)) atomicOr(s.err, DEVERR_NONFINITE);
+    }
+    if (!isfinite(v)) atomicOr(s.err, DEVERR_NONFINITE);
+}
+
+// Exclusive prefix (of `in`, this thread's run in thread order) from the block's
+// inclusive scan.
+template <typename T>
+__device__ __forceinline__ T block_excl(T run, T *sh, T zero)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T total;
+    const T in = block_incl_scan(run, sh, total);
+    T ex = shfl_up(in, 1);
+    if (lane == 31) sh[warp] = in;
+    __syncthreads();
+    if (lane == 0) ex = warp > 0 ? sh[warp - 1] : zero;
+    __syncthreads();
+    return ex;
+}
+
+// Partial slots of row group g: the CTAs whose unit ranges meet it.
+__device__ __forceinline__ int slot_count(const SP &s, int64_t g)
+{
+    const int64_t a = g * s.KC, b = a + s.KC - 1;
+    if (b < (int64_t(1) << 31) && s.L < (int64_t(1) << 31))
+        return static_cast<int>(static_cast<uint32_t>(b) / static_cast<uint32_t>(s.L) -
+                                static_cast<uint32_t>(a) / static_cast<uint32_t>(s.L)) + 1;
+    return static_cast<int>(b / s.L - a / s.L + 1);
+}
+
+// Padded shared-memory index of element e of a chunk (the scan reads runs of
+// EPT elements per lane: without the padding 8-way bank conflicts).
+__device__ __forceinline__ int padded(int e) { return e + (e >> 5); }
+
+// EPT: subjects per lane (a chunk is the 32 EPT subjects of one warp); F64: FP64
+// throughout (COX_FP64); Q: with unpenalised covariates (their sums take 32
+// registers).  Block b takes the chunks [b per, (b + 1) per) of the column-major
+// list, its warps in turn; nothing inside a chunk waits for another warp.
+template <int EPT, bool F64, bool Q>
+__global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
+{
+    constexpr int CW = 32 * EPT;
+    constexpr int BW = CW + CW / 32;  // doubles of a warp's buffer
+    using acc_t = typename std::conditional<F64, double, tf>::type;
+    using w_t = typename std::conditional<F64, double, float>::type;
+    acc_t zero, low;  // 0 and minus infinity
+    if constexpr (F64) {
+        zero = 0.0;
+        low = -INFINITY;
+    } else {
+        zero = tf{0.f, 0.f};
+        low = tf{-INFINITY, 0.f};
+    }
+    __shared__ __align__(16) double buf_all[NW * BW];  // per warp: w of a chunk (2), C of its event groups (4)
+    __shared__ double shd[NW];
+    __shared__ acc_t sha[NW];
+    __shared__ float shf[NW];
+    __shared__ long long shl[NW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double *const buf = buf_all + warp * BW;
+    const int64_t nch = s.nch, tasks = nch * s.k;
+    const int64_t lo = min(tasks, blockIdx.x * s.per), hi = min(tasks, lo + s.per);
+
+    // ---- phase 1: eta, chunk maxima, chunk sums of delta eta ----
+    for (int64_t t = lo + warp; t < hi; t += NW) {
+        const int kk = static_cast<int>(t / nch);
+        const int64_t c = t - kk * nch, i0 = c * CW;
+        int cnt0 = 1, cnt1 = 1;
+        if (s.src == ETA_PARTIAL_F32) {  // a chunk meets at most two row groups (of 128 or 256)
+            cnt0 = slot_count(s, i0 / s.group_rows);
+            cnt1 = EPT == 8 ? slot_count(s, (i0 + 128) / s.group_rows) : cnt0;
+        }
+        acc_t v[EPT];
+        uint8_t ev[EPT];
+#pragma unroll
+        for (int j = 0; j < EPT; ++j) {
+            const int64_t i = min(i0 + lane + 32 * j, s.n - 1);
+            ev[j] = s.delta[i];
+            if (s.src == ETA_PARTIAL_F32 || s.src == ETA_DENSE_F32) {
+                const float a = static_cast<const float *>(s.eta_in)[kk * s.col_stride + i];
+                if constexpr (F64) v[j] = static_cast<double>(a);
+                else v[j] = tf{a, 0.f};
+            } else {
+                const double a = static_cast<const double *>(s.eta_in)[kk * s.col_stride + i];
+                if constexpr (F64) v[j] = a;
+                else v[j] = tf_of(a);
+            }
+        }
+        if (cnt0 > 1 || cnt1 > 1) {  // a row group cut between CTAs
+#pragma unroll
+            for (int j = 0; j < EPT; ++j) {
+                const int64_t i = min(i0 + lane + 32 * j, s.n - 1);
+                const float *part = static_cast<const float *>(s.eta_in) + kk * s.col_stride + i;
+                const int cnt = EPT == 8 && j >= 4 ? cnt1 : cnt0;
+                for (int sl = 1; sl < cnt; ++sl) {
+                    const float b = part[sl * s.slot_stride];
+                    if constexpr (F64) v[j] += static_cast<double>(b);
+                    else v[j] = tf_add(v[j], tf{b, 0.f});
+                }
+            }
+        }
+        acc_t mx = low, de = zero;
+#pragma unroll
+        for (int j = 0; j < EPT; ++j) {
+            const int64_t i = i0 + lane + 32 * j;
+            if (i >= s.n) break;
+            if (Q) {  // eta += Z gamma (Section 6 unpenalised covariates), in FP64
+                double zg = 0.0;
+#pragma unroll 4
+                for (int cq = 0; cq < s.q; ++cq) zg += s.Z[cq * s.n + i] * s.gamma[kk * s.q + cq];
+                const double vd = as_double(v[j]) + zg;
+                if constexpr (F64) v[j] = vd;
+                else v[j] = tf_of(vd);
+            }
+            static_cast<acc_t *>(s.eta)[kk * s.n + i] = v[j];
+            if (less(mx, v[j])) mx = v[j];
+            if (ev[j]) de = plus(de, v[j]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const acc_t y = shfl_xor(mx, o);
+            if (less(mx, y)) mx = y;
+            de = plus(de, shfl_xor(de, o));
+        }
+        if (lane == 0) {
+            static_cast<acc_t *>(s.cmaxp)[t] = mx;
+            s.lossp[t] = as_double(de);
+        }
+    }
+    grid_barrier(s, 1);
+
+    // ---- phase 2: w = exp(eta - c); chunk-local reverse scan of w, kept at the
+    // heads of the tie groups that hold events (the only places W is read) ----
+    for (int64_t t0 = lo; t0 < hi;) {
+        const int kk = static_cast<int>(t0 / nch);
+        const int64_t t1 = min(hi, (kk + 1) * nch);
+        acc_t cm = low;  // c: the column's largest eta (every block for itself)
+#pragma unroll 4
+        for (int64_t q = tid; q < nch; q += NT) {
+            const acc_t y = static_cast<const acc_t *>(s.cmaxp)[kk * nch + q];
+            if (less(cm, y)) cm = y;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const acc_t y = shfl_xor(cm, o);
+            if (less(cm, y)) cm = y;
+        }
+        if (lane == 0) sha[warp] = cm;
+        __syncthreads();
+        cm = sha[0];
+#pragma unroll
+        for (int w = 1; w < NW; ++w)
+            if (less(cm, sha[w])) cm = sha[w];
+        __syncthreads();
+        if (tid == 0 && t0 == kk * nch) s.colc[kk] = as_double(cm);
+        for (int64_t t = t0 + warp; t < t1; t += NW) {
+            const int64_t c = t - kk * nch, i0 = c * CW;
+            w_t *wb = reinterpret_cast<w_t *>(buf);
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < EPT; ++j) {
+                const int64_t i = i0 + lane + 32 * j;
+                w_t wv = 0;
+                if (i < s.n) {
+                    const acc_t v = static_cast<const acc_t *>(s.eta)[kk * s.n + i];
+                    if constexpr (F64) {
+                        wv = exp(v - cm);
+                    } else {
+                        const tf d = two_sum(v.h, -cm.h);
+                        wv = expf(d.h + (d.l + (v.l - cm.l)));  // the FP32 rounding of eta - c
+                    }
+                    static_cast<w_t *>(s.w)[kk * s.n + i] = wv;
+                }
+                wb[padded(lane + 32 * j)] = wv;
+            }
+            const int64_t ib = i0 + CW - EPT * (lane + 1);  // this lane's subjects: ib .. ib + EPT - 1
+            uint64_t fl;  // their event-group flags, a byte each
+            if constexpr (EPT == 8) fl = *reinterpret_cast<const uint64_t *>(s.evflag + ib);
+            else if constexpr (EPT == 4) fl = *reinterpret_cast<const uint32_t *>(s.evflag + ib);
+            else if constexpr (EPT == 2) fl = *reinterpret_cast<const uint16_t *>(s.evflag + ib);
+            else fl = s.evflag[ib];
+            __syncwarp();
+            // lane l owns reversed positions [EPT l, EPT l + EPT): elements CW-1-(EPT l + j)
+            acc_t loc[EPT], run = zero;
+#pragma unroll
+            for (int j = 0; j < EPT; ++j) {
+                const w_t wv = wb[padded(CW - 1 - (EPT * lane + j))];
+                if constexpr (F64) run += wv;
+                else run = tf_add(run, tf{wv, 0.f});
+                loc[j] = run;
+            }
+            acc_t incl = run;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const acc_t y = shfl_up(incl, o);
+                if (lane >= o) incl = plus(y, incl);
+            }
+            acc_t excl = shfl_up(incl, 1);
+            if (lane == 0) excl = zero;
+            if (fl) {
+#pragma unroll
+                for (int j = 0; j < EPT; ++j)
+                    if ((fl >> (8 * (EPT - 1 - j))) & 0xff)
+                        s.Wg[kk * s.G + s.evidx[ib + EPT - 1 - j] - 1] = as_double(plus(excl, loc[j]));
+            }
+            if (lane == 31) s.csw[t] = as_double(incl);
+        }
+        if (last_of_column(s, kk, 0, column_blocks(s, kk))) {
+            // exclusive suffix sums of the chunk totals; thread t owns a contiguous run
+            // of chunks in scan order
+            const double *src = s.csw + kk * nch;
+            double *dst = s.suf + kk * nch;
+            const int64_t per = (nch + NT - 1) / NT;
+            double tot = 0.0;
+#pragma unroll 8
+            for (int64_t j = 0; j < per; ++j)
+                if (tid * per + j < nch) tot += src[nch - 1 - (tid * per + j)];
+            double acc = block_excl(tot, shd, 0.0);
+#pragma unroll 8
+            for (int64_t j = 0; j < per; ++j) {
+                const int64_t q = tid * per + j;
+                if (q < nch) {
+                    dst[nch - 1 - q] = acc;
+                    acc += src[nch - 1 - q];
+                }
+            }
+        }
+        t0 = t1;
+    }
+    grid_barrier(s, 2);
+
+    // ---- phase 3: W_g = the chunk-local reverse sum at the group's head plus the
+    // suffix of later chunks; D_g = e_g / W_g (one FP64 division per event time:
+    // tied events share W, Breslow); scans of D inside tiles of GT groups ----
+    const int64_t tiles = static_cast<int64_t>(s.ntile) * s.k;
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int kk = static_cast<int>(t / s.ntile);
+        const int64_t g = (t - static_cast<int64_t>(kk) * s.ntile) * GT + tid;
+        double D = 0.0;
+        if (g < s.G) {
+            const double W = s.Wg[kk * s.G + g] + s.suf[kk * nch + s.evhead[g] / CW];
+            D = static_cast<double>(s.evcnt[g]) / W;
+        }
+        double total;
+        const double incl = block_incl_scan(D, shd, total);
+        if (g < s.G) s.Fg[kk * s.G + g] = incl;  // within the tile; the tile's base is added in phase 4
+        if (tid == 0) s.tot[t] = total;
+        if (last_of_column(s, kk, 1, s.ntile)) {
+            const double *src = s.tot + static_cast<int64_t>(kk) * s.ntile;
+            double *dst = s.tbase + static_cast<int64_t>(kk) * s.ntile;
+            const int per = (s.ntile + NT - 1) / NT;
+            double run = 0.0;
+            for (int j = 0; j < per; ++j)
+                if (tid * per + j < s.ntile) run += src[tid * per + j];
+            double acc = block_excl(run, shd, 0.0);
+            for (int j = 0; j < per; ++j)
+                if (tid * per + j < s.ntile) {
+                    dst[tid * per + j] = acc;
+                    acc += src[tid * per + j];
+                }
+        }
+    }
+    // ---- beside phase 3, on the last blocks: the loss term sum_g e_g log W_g +
+    // (events) c of the tiles, of products carried as (mantissa, exponent), one log
+    // per tile (FP64 log is costly) ----
+    for (int64_t t = gridDim.x - 1 - blockIdx.x; s.need_loss && t < tiles; t += gridDim.x) {
+        const int kk = static_cast<int>(t / s.ntile);
+        const int64_t g = (t - static_cast<int64_t>(kk) * s.ntile) * GT + tid;
+        double pm = 1.0, lsum = 0.0;
+        int pe = 0, ev = 0;
+        if (g < s.G) {
+            const double W = s.Wg[kk * s.G + g] + s.suf[kk * nch + s.evhead[g] / CW];
+            ev = s.evcnt[g];
+            if (ev <= 64 && W >= 0x1p-1000 && W <= 0x1p+1000) {
+                double b = W;  // W^ev by squaring, both factors renormalised at every step
+                int be = renorm(b);
+                for (int x = ev; x > 0; x >>= 1) {
+                    if (x & 1) {
+                        pm *= b;
+                        pe += be + renorm(pm);
+                    }
+                    b *= b;
+                    be = 2 * be + renorm(b);
+                }
+            } else {
+                lsum = static_cast<double>(ev) * log(W);  // many tied events, or W zero, huge, subnormal, NaN
+            }
+        }
+        lsum = block_sum(lsum, shd);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {  // 32 factors in [1, 2): no overflow
+            pm *= __shfl_xor_sync(0xffffffffu, pm, o);
+            pe += __shfl_xor_sync(0xffffffffu, pe, o);
+            ev += __shfl_xor_sync(0xffffffffu, ev, o);
+        }
+        if (lane == 0) {
+            shd[warp] = pm;
+            shl[warp] = (static_cast<long long>(pe) << 32) | static_cast<unsigned>(ev);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            long long pes = pe, evs = ev;
+            for (int w = 1; w < NW; ++w) {
+                pes += renorm(pm);
+                pm *= shd[w];
+                pes += shl[w] >> 32;
+                evs += shl[w] & 0xffffffffLL;
+            }
+            s.lgp[t] = lsum + (log(pm) + static_cast<double>(pes) * 0.6931471805599453 + static_cast<double>(evs) * s.colc[kk]);
         }
         __syncthreads();
     }
-    double mx = -INFINITY, de = 0.0;
-    for (int e = threadIdx.x; e < SCAN_CH; e += NT) {
-        const int64_t i = i0 + e;
-        if (i >= s.n) break;
-        double v;
-        if (SRC == ETA_PARTIAL_F32) {
-            const float *part = static_cast<const float *>(src);
-            const int cnt = cnt_sh[e / group_rows];
-            v = 0.0;
-            for (int sl = 0; sl < cnt; ++sl) v += static_cast<double>(part[sl * slot_stride + kk * col_stride + i]);
-        } else if (SRC == ETA_DENSE_F32) {
-            v = static_cast<double>(static_cast<const float *>(src)[kk * col_stride + i]);
-        } else {
-            v = static_cast<const double *>(src)[kk * col_stride + i];
-        }
-        if (s.q) {  // eta += Z gamma (Section 6 unpenalised covariates), in FP64
-            double zg = 0.0;
-            for (int cq = 0; cq < s.q; ++cq) zg += s.Z[cq * s.n + i] * s.gamma[kk * s.q + cq];
-            v += zg;
-        }
-        s.eta[kk * s.n + i] = v;
-        mx = fmax(mx, v);
-        if (s.delta[i]) de += v;
-    }
-    const double m = block_max(mx, sh);
-    if (threadIdx.x == 0) s.cmax[kk * s.nch + c] = m;
-    const double t = block_sum(de, sh);
-    if (threadIdx.x == 0) s.lossp[kk * s.nch + c] = t;
-}
 
-__device__ __forceinline__ double column_max(const SP &s, int kk, double *sh)
-{
-    double m = -INFINITY;
-    for (int c = threadIdx.x; c < s.nch; c += NT) m = fmax(m, s.cmax[kk * s.nch + c]);
-    m = block_max(m, sh);
-    if (threadIdx.x == 0) sh[0] = m;
-    __syncthreads();
-    m = sh[0];
-    __syncthreads();
-    return m;
-}
+    grid_barrier(s, 3);
 
-// (2) w = exp(eta - c); chunk-local reverse inclusive scan of w, kept at the
-// heads of the tie groups that hold events (the only places W is read);
-// chunk totals.
-template <bool EXP64>
-__global__ void k_rev(SP s)
-{
-    __shared__ double sh[NT / 32];
-    __shared__ double buf[SCAN_CH];
-    const int c = blockIdx.x, kk = blockIdx.y;
-    const double cmx = column_max(s, kk, sh);
-    const int64_t i0 = static_cast<int64_t>(c) * SCAN_CH;
-    for (int e = threadIdx.x; e < SCAN_CH; e += NT) {
-        const int64_t i = i0 + e;
-        double wv = 0.0;
-        if (i < s.n) {
-            const double x = s.eta[kk * s.n + i] - cmx;
-            wv = EXP64 ? exp(x) : static_cast<double>(expf(static_cast<float>(x)));
-            s.w[kk * s.n + i] = wv;
-        }
-        buf[e] = wv;
-    }
-    __syncthreads();
-    // thread t owns reversed positions [PER t, PER t + PER): elements SCAN_CH-1-(PER t + j)
-    double loc[PER];
-    double run = 0.0;
+    // ---- phase 4: C = F of the last event group at or before the tie tail; u = w C;
+    // V = delta - u.  The FP32 dense form feeds a product over the SNP-major copy and
+    // is written at its K positions; the FP64 form stays in sorted order; for the
+    // limbs, V goes to V32 with chunk maxima of |V| ----
+    const bool limbs = s.vo == V_LIMBS_E4M3;
+    for (int64_t t = lo + warp; t < hi; t += NW) {
+        const int kk = static_cast<int>(t / nch);
+        const int64_t c = t - kk * nch, i0 = c * CW;
+        w_t wv[EPT];
+        int gi[EPT];
+        uint8_t ev[EPT];
 #pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        run += buf[SCAN_CH - 1 - (PER * threadIdx.x + j)];
-        loc[j] = run;
-    }
-    const double incl = block_incl_scan(run, sh);
-    const double excl = incl - run;
-#pragma unroll
-    for (int j = 0; j < PER; ++j) {
-        const int64_t i = i0 + SCAN_CH - 1 - (PER * threadIdx.x + j);
-        if (i < s.n && s.evflag[i]) s.Rt[kk * s.n + i] = loc[j] + excl;
-    }
-    if (threadIdx.x == NT - 1) s.csw[kk * s.nch + c] = incl;
-}
-
-// exclusive suffix scans of the chunk totals of w; one warp per column, lane
-// l owning a contiguous run of chunks in scan order.
-__global__ void k_chunks(SP s)
-{
-    const int kk = blockIdx.x, lane = threadIdx.x;
-    const double *src = s.csw + static_cast<int64_t>(kk) * s.nch;
-    double *dst = s.suf + static_cast<int64_t>(kk) * s.nch;
-    const int per = (s.nch + 31) / 32;
-    auto at = [&](int q) { return s.nch - 1 - q; };  // q-th chunk in scan order
-    double tot = 0.0;
-    for (int j = 0; j < per; ++j) {
-        const int q = lane * per + j;
-        if (q < s.nch) tot += src[at(q)];
-    }
-    const double incl = warp_incl_scan(tot, lane);
-    double acc = __shfl_up_sync(0xffffffffu, incl, 1);
-    if (lane == 0) acc = 0.0;
-    for (int j = 0; j < per; ++j) {
-        const int q = lane * per + j;
-        if (q < s.nch) {
-            dst[at(q)] = acc;
-            acc += src[at(q)];
+        for (int j = 0; j < EPT; ++j) {
+            const int64_t i = min(i0 + lane + 32 * j, s.n - 1);
+            wv[j] = static_cast<const w_t *>(s.w)[kk * s.n + i];
+            gi[j] = s.evidx[i];
+            ev[j] = s.delta[i];
         }
-    }
-}
-
-// (3) One block per column, over the tie groups that hold events: W_g = the
-// chunk-local reverse sum at the group's head plus the suffix of later chunks,
-// D_g = e_g / W_g (one FP64 division per event time: tied events share W,
-// Breslow), F = the inclusive scan of D over the groups, and the loss term
-// sum_g e_g log W_g + (events) c.  Thread t takes a contiguous run of groups;
-// the logs are taken of products carried as (mantissa, exponent), one log per
-// thread (FP64 log is costly).
-__global__ void k_group(SP s, bool need_loss)
-{
-    __shared__ double sh[NT / 32];
-    const int kk = blockIdx.x;
-    const int64_t G = s.n_evh;
-    const int64_t per = (G + NT - 1) / NT;
-    const int64_t g0 = min(G, per * threadIdx.x), g1 = min(G, g0 + per);
-    const double cmx = need_loss ? column_max(s, kk, sh) : 0.0;
-    double run = 0.0, pm = 1.0, lsum = 0.0;
-    int pe = 0;
-    long long nev = 0;
-    for (int64_t g = g0; g < g1; ++g) {
-        const int64_t hd = s.evhead[g];
-        const double W = s.Rt[kk * s.n + hd] + s.suf[kk * s.nch + hd / SCAN_CH];
-        const int e = s.evcnt[g];
-        run += static_cast<double>(e) / W;
-        s.Fg[kk * G + g] = run;  // local; the block offset is added below
-        if (need_loss) {
-            nev += e;
-            if (e <= 8 && W >= 0x1p-1000 && W <= 0x1p+1000) {
-                for (int q = 0; q < e; ++q) {
-                    pm *= W;
-                    pe += renorm(pm);
+        // C at the event groups the chunk reads (at most one more per subject), as
+        // pairs of floats unless covariates need V in FP64 or some C leaves FP32's range
+        const int glo = __shfl_sync(0xffffffffu, gi[0], 0), ghi = __shfl_sync(0xffffffffu, gi[EPT - 1], 31);
+        __syncwarp();
+        bool wide = F64 || Q;
+        for (int pass = 0; pass < 2; ++pass) {
+            bool big = false;
+            for (int u = lane; u <= ghi - glo; u += 32) {
+                const int g = glo + u;
+                const double C = g > 0 ? s.Fg[kk * s.G + g - 1] + s.tbase[static_cast<int64_t>(kk) * s.ntile + (g - 1) / GT] : 0.0;
+                if (wide) {
+                    buf[u] = C;
+                } else {
+                    big |= !(C < 1e37);
+                    reinterpret_cast<tf *>(buf)[u] = tf_of(C);
                 }
+            }
+            big = __any_sync(0xffffffffu, big);
+            if (wide || !big) break;
+            wide = true;
+        }
+        __syncwarp();
+        acc_t vs = zero;
+        float vm32 = 0.f;
+        double zv[Q ? MAXQ : 1];  // Z^T V over this lane's subjects (unpenalised covariates)
+        if (Q) {
+#pragma unroll
+            for (int cq = 0; cq < MAXQ; ++cq) zv[Q ? cq : 0] = 0.0;
+        }
+#pragma unroll
+        for (int j = 0; j < EPT; ++j) {
+            const int64_t i = i0 + lane + 32 * j;
+            if (i >= s.n) break;
+            const int u = gi[j] - glo;
+            float v32;
+            double V = 0.0;
+            if (wide) {
+                V = (ev[j] ? 1.0 : 0.0) - static_cast<double>(wv[j]) * buf[u];
+                v32 = static_cast<float>(V);
             } else {
-                lsum += static_cast<double>(e) * log(W);  // many tied events, or W zero, huge, subnormal, NaN
+                const tf C = reinterpret_cast<const tf *>(buf)[u];
+                const float wf = static_cast<float>(wv[j]);
+                const float p = wf * C.h;
+                const float r = fmaf(wf, C.l, fmaf(wf, C.h, -p));  // w C = p + r
+                const tf d = two_sum(ev[j] ? 1.f : 0.f, -p);
+                v32 = d.h + (d.l - r);
+            }
+            if (Q) {
+#pragma unroll
+                for (int cq = 0; cq < MAXQ; ++cq)
+                    if (cq < s.q) zv[Q ? cq : 0] += s.Z[cq * s.n + i] * V;
+            }
+            // sum V in the form the product reads: X^T V - mu sum V is then
+            // exactly the centred product of that V.  (Censored subjects between
+            // two event times share one V, so their rounding errors do not
+            // cancel; with the exact sum, mu times their sum would remain.)
+            if (limbs) {
+                s.V32[kk * s.n + i] = v32;
+                vm32 = fmaxf(vm32, fabsf(v32));
+            } else if constexpr (F64) {
+                static_cast<double *>(s.V)[kk * s.n + i] = V;
+                vs += V;
+            } else {
+                static_cast<float *>(s.V)[static_cast<int64_t>(s.a4blk[i >> 4]) * 16 + (i & 15) + kk * s.n_pad] = v32;
+                vs = tf_add(vs, tf{v32, 0.f});
             }
         }
-    }
-    const double incl = block_incl_scan(run, sh);
-    const double excl = incl - run;
-    if (excl != 0.0)
-        for (int64_t g = g0; g < g1; ++g) s.Fg[kk * G + g] += excl;
-    if (need_loss) {
-        lsum += log(pm) + static_cast<double>(pe) * 0.6931471805599453 + static_cast<double>(nev) * cmx;
-        const double t = block_sum(lsum, sh);
-        if (threadIdx.x == 0) s.lossg[kk] = t;
-    }
-}
-
-// (4) C = F of the last event group at or before the tie tail; u = w C;
-// V = delta - u -> output form; sum of V.
-// The FP32 form feeds a product over the SNP-major copy and is written at its
-// K positions (a4_pos); the FP64 form stays in sorted order.  For the e4m3
-// limbs, V goes to Rt (free once the group kernel read it) with chunk maxima of |V|,
-// and k_vlimbs splits it once the column's scale is known.
-template <int VO>
-__global__ void k_uv(SP s, void *Vout, int64_t n_pad, double *vmaxp)
-{
-    __shared__ double sh[NT / 32];
-    const int c = blockIdx.x, kk = blockIdx.y;
-    const int64_t i0 = static_cast<int64_t>(c) * SCAN_CH;
-    double vs = 0.0;
-    float vm32 = 0.f;
-    double zv[MAXQ];  // Z^T V over this thread's subjects (unpenalised covariates)
+        if (limbs) {
 #pragma unroll
-    for (int cq = 0; cq < MAXQ; ++cq) zv[cq] = 0.0;
-    for (int e = threadIdx.x; e < SCAN_CH; e += NT) {
-        const int64_t i = i0 + e;
-        if (i >= s.n) break;
-        const int32_t gi = s.evidx[i];
-        const double C = gi > 0 ? s.Fg[kk * s.n_evh + gi - 1] : 0.0;
-        const double u = s.w[kk * s.n + i] * C;
-        const double V = static_cast<double>(s.delta[i]) - u;
-        if (s.q) {
+            for (int o = 16; o > 0; o >>= 1) vm32 = fmaxf(vm32, __shfl_xor_sync(0xffffffffu, vm32, o));
+            if (lane == 0) s.vmaxp[t] = vm32;
+        } else {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) vs = plus(vs, shfl_xor(vs, o));
+            if (lane == 0) s.vsp[t] = as_double(vs);
+        }
+        if (Q) {
 #pragma unroll
             for (int cq = 0; cq < MAXQ; ++cq)
-                if (cq < s.q) zv[cq] += s.Z[cq * s.n + i] * V;
-        }
-        // sum V in the form the product reads: X^T V - mu sum V is then
-        // exactly the centred product of that V.  (Censored subjects between
-        // two event times share one V, so their rounding errors do not
-        // cancel; with the exact sum, mu times their sum would remain.)
-        if (VO == V_LIMBS_E4M3) {
-            // k_vlimbs splits the FP32 value: hand it over in FP32 (the max of
-            // the rounded values is the rounded max, so the scale is unchanged)
-            const float v32 = static_cast<float>(V);
-            reinterpret_cast<float *>(s.Rt)[kk * s.n + i] = v32;
-            vm32 = fmaxf(vm32, fabsf(v32));
-        } else if (VO == V_DENSE_F64) {
-            static_cast<double *>(Vout)[kk * s.n + i] = V;
-            vs += V;
-        } else {
-            const float v32 = static_cast<float>(V);
-            static_cast<float *>(Vout)[a4_pos(i, s.pa, s.pnb) + kk * n_pad] = v32;
-            vs += static_cast<double>(v32);
-        }
-    }
-    if (VO == V_LIMBS_E4M3) {
-        const double m = block_max(static_cast<double>(vm32), sh);
-        if (threadIdx.x == 0) vmaxp[kk * s.nch + c] = m;
-    } else {
-        const double t = block_sum(vs, sh);
-        if (threadIdx.x == 0) s.vsp[kk * s.nch + c] = t;
-    }
-    for (int cq = 0; cq < s.q; ++cq) {  // block-uniform trip count
-        double zc = 0.0;
+                if (cq < s.q) {
+                    double x = zv[Q ? cq : 0];
 #pragma unroll
-        for (int q2 = 0; q2 < MAXQ; ++q2)
-            if (q2 == cq) zc = zv[q2];
-        const double t = block_sum(zc, sh);
-        if (threadIdx.x == 0) s.zvp[(static_cast<int64_t>(kk) * s.q + cq) * s.nch + c] = t;
-    }
-}
-
-// (4b) V (FP32, in Rt) -> e4m3 limbs at the A4 K positions, one power-of-two
-// scale per column (from all chunk maxima); chunk sums of the values the limbs
-// hold, exact: each is an integer number of 2^(sc-21) units below 2^30, so
-// a chunk's sum is an integer below 2^42, exact in FP64.
-__global__ void k_vlimbs(SP s, uint8_t *__restrict__ Vq, int64_t n_pad, const double *__restrict__ vmaxp,
-                         int *__restrict__ bs, int *err)
-{
-    __shared__ double sh[NT / 32];
-    __shared__ int s_sh;
-    const int c = blockIdx.x, kk = blockIdx.y;
-    double m = 0.0;
-    for (int q = threadIdx.x; q < s.nch; q += NT) m = fmax(m, vmaxp[kk * s.nch + q]);
-    m = block_max(m, sh);
-    if (threadIdx.x == 0) {
-        float mf = static_cast<float>(m);
-        if (!isfinite(mf)) {
-            atomicOr(err, DEVERR_NONFINITE);
-            mf = 0.f;
+                    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                    if (lane == 0) s.zvp[(static_cast<int64_t>(kk) * s.q + cq) * nch + c] = x;
+                }
         }
-        s_sh = limb_scale(mf);
-        if (c == 0) bs[kk] = s_sh;
     }
+    if (limbs) grid_barrier(s, 4);
+
+    // ---- phase 5: V (FP32) -> limbs at the A4 K positions under the column's
+    // power-of-two scale; chunk sums of the values the limbs hold, exact integers:
+    // units of 2^(s-21) (e4m3 values, below 2^30 each) or 2^(s-22) (e2m1) ----
+    for (int64_t t0 = lo; t0 < hi;) {
+        const int kk = static_cast<int>(t0 / nch);
+        const int64_t t1 = min(hi, (kk + 1) * nch);
+        if (limbs) {
+            float m = 0.f;  // the column's largest |V| (every block for itself)
+#pragma unroll 4
+            for (int64_t q = tid; q < nch; q += NT) m = fmaxf(m, s.vmaxp[kk * nch + q]);
+            m = block_max(m, shf);
+            const bool bad = !isfinite(m);
+            if (bad) m = 0.f;
+            const int sc = s.form == FORM_E2M1 ? limb_scale4(m) : limb_scale(m);
+            if (tid == 0 && t0 == kk * nch) {
+                s.bs[kk] = sc;
+                if (bad) atomicOr(s.err, DEVERR_NONFINITE);
+            }
+            // V 2^-sc, in two exact factors (sc lies in [-156, 127]; |V| >= 1/n whenever
+            // V is not all zero, so nothing the limbs can hold becomes subnormal)
+            const float s1 = ldexpf(1.f, -(sc / 2)), s2 = ldexpf(1.f, -(sc - sc / 2));
+            uint8_t *Vq = static_cast<uint8_t *>(s.V);
+            const float *V32 = s.V32 + kk * s.n;
+            for (int64_t t = t0 + warp; t < t1; t += NW) {
+                const int64_t i0 = (t - kk * nch) * CW;
+                long long q = 0;
+                bool finite = true;
+                if (s.form == FORM_E4M3) {
+#pragma unroll
+                    for (int j = 0; j < EPT; ++j) {
+                        const int64_t i = i0 + lane + 32 * j;
+                        if (i >= s.n) break;
+                        uint8_t d[LIMBS];
+                        const float r = V32[i] * s1 * s2;
+                        finite = finite && isfinite(r);
+                        q += split_e4m3_units(r, d);
+                        const int64_t pos = static_cast<int64_t>(s.a4blk[i >> 4]) * 16 + (i & 15);
+#pragma unroll
+                        for (int l = 0; l < LIMBS; ++l) Vq[(LIMBS * kk + l) * s.n_pad + pos] = d[l];
+                    }
+                } else {
+                    // subjects 16 (e / 8) + e mod 8 and that + 8 share one byte per limb row (e2m1_byte)
+                    const int64_t rb = s.n_pad / 2;
+#pragma unroll
+                    for (int j = 0; j < (EPT + 1) / 2; ++j) {
+                        const int e = lane + 32 * j;
+                        const int64_t ia = i0 + ((e >> 3) << 4) + (e & 7);
+                        if (e >= CW / 2 || ia >= s.n) break;
+                        const float ra = V32[ia] * s1 * s2;
+                        const float rb8 = ia + 8 < s.n ? V32[ia + 8] * s1 * s2 : 0.f;
+                        finite = finite && isfinite(ra) && isfinite(rb8);
+                        const int64_t byte = static_cast<int64_t>(s.a4blk[ia >> 4]) * 8 + (ia & 7);
+                        if (s.form == FORM_E2M1) {
+                            uint8_t d0[LIMBS4], d1[LIMBS4];
+                            q += split_e2m1_units(ra, d0);
+                            q += split_e2m1_units(rb8, d1);
+#pragma unroll
+                            for (int l = 0; l < LIMBS4; ++l)
+                                Vq[(LIMBS4 * kk + l) * rb + byte] = static_cast<uint8_t>(d0[l] | (d1[l] << 4));
+                        } else {
+                            uint8_t d[LIMBS], d0[LIMBS_W], d1[LIMBS_W];
+                            const int qa = split_e4m3_units(ra, d), qb = split_e4m3_units(rb8, d);
+                            q += qa;
+                            q += qb;
+                            split_wide(qa, d0);
+                            split_wide(qb, d1);
+#pragma unroll
+                            for (int l = 0; l < LIMBS_W; ++l)
+                                Vq[(LIMBS_W * kk + l) * rb + byte] = static_cast<uint8_t>(d0[l] | (d1[l] << 4));
+                        }
+                    }
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+                finite = __all_sync(0xffffffffu, finite);
+                const int unit = s.form == FORM_E2M1 ? 1 + 3 * (LIMBS4 - 1) : 21;
+                if (lane == 0) s.vsp[t] = finite ? ldexp(static_cast<double>(q), sc - unit) : NAN;
+            }
+        }
+        if (last_of_column(s, kk, 2, column_blocks(s, kk))) finalize_column(s, kk, shd);
+        t0 = t1;
+    }
+
+    // the last block to end leaves the barrier's counters at zero for the next launch
     __syncthreads();
-    const int sc = s_sh;
-    const int64_t i0 = static_cast<int64_t>(c) * SCAN_CH;
-    const float *V32 = reinterpret_cast<const float *>(s.Rt);
-    long long q = 0;
-    bool finite = true;
-    for (int e = threadIdx.x; e < SCAN_CH; e += NT) {
-        const int64_t i = i0 + e;
-        if (i >= s.n) break;
-        uint8_t d[LIMBS];
-        // ldexpf of the FP32 value equals rounding the scaled FP64 value: the
-        // scale is a power of two and |V| >= 1/n whenever V is not all zero,
-        // so nothing the limbs can hold falls into FP32's subnormal range
-        const float r = ldexpf(V32[kk * s.n + i], -sc);
-        finite = finite && isfinite(r);
-        q += split_e4m3_units(r, d);
-        const int64_t pos = a4_pos(i, s.pa, s.pnb);
-#pragma unroll
-        for (int l = 0; l < LIMBS; ++l) Vq[(LIMBS * kk + l) * n_pad + pos] = d[l];
+    if (tid == 0) {
+        __threadfence();
+        if (atomicAdd(s.cnt + 1, 1u) == gridDim.x - 1) {
+            s.cnt[0] = 0;
+            s.cnt[1] = 0;
+        }
     }
-    const double t = block_sum(finite ? static_cast<double>(q) : NAN, sh);
-    if (threadIdx.x == 0) s.vsp[kk * s.nch + c] = ldexp(t, sc - 21);
 }
 
-// (4b, e2m1 form) V -> e2m1 limbs at the A4 K positions: thread e of a chunk
-// takes subjects 16 (e / 8) + e mod 8 and that + 8 of the chunk, which share
-// one byte per limb row (e2m1_byte); chunk sums of the values the limbs hold,
-// exact (integers of 2^(sc-22) units, below 2^35 per chunk).
-__global__ void k_vlimbs4(SP s, uint8_t *__restrict__ Vq, int64_t n_pad, const double *__restrict__ vmaxp,
-                          int *__restrict__ bs, int *err)
+// eta (FP64) from the product's partial slots, for cox_eta.
+__global__ void k_eta(const float *__restrict__ part, int64_t n, int64_t slot_stride, int64_t col_stride, int group_rows,
+                      int KC, int64_t L, double *__restrict__ eta)
 {
-    __shared__ double sh[NT / 32];
-    __shared__ int s_sh;
-    const int c = blockIdx.x, kk = blockIdx.y;
-    double m = 0.0;
-    for (int q = threadIdx.x; q < s.nch; q += NT) m = fmax(m, vmaxp[kk * s.nch + q]);
-    m = block_max(m, sh);
-    if (threadIdx.x == 0) {
-        float mf = static_cast<float>(m);
-        if (!isfinite(mf)) {
-            atomicOr(err, DEVERR_NONFINITE);
-            mf = 0.f;
-        }
-        s_sh = limb_scale4(mf);
-        if (c == 0) bs[kk] = s_sh;
+    const int kk = blockIdx.y;
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * NT + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * NT) {
+        const int64_t g = i / group_rows;
+        const int cnt = static_cast<int>((g * KC + KC - 1) / L - (g * KC) / L + 1);
+        double v = 0.0;
+        for (int sl = 0; sl < cnt; ++sl) v += static_cast<double>(part[sl * slot_stride + kk * col_stride + i]);
+        eta[kk * n + i] = v;
     }
-    __syncthreads();
-    const int sc = s_sh;
-    const int64_t i0 = static_cast<int64_t>(c) * SCAN_CH;
-    const float *V32 = reinterpret_cast<const float *>(s.Rt);
-    const int64_t rb = n_pad / 2;
-    long long q = 0;
-    bool finite = true;
-    for (int e = threadIdx.x; e < SCAN_CH / 2; e += NT) {
-        const int64_t ia = i0 + ((e >> 3) << 4) + (e & 7);
-        if (ia >= s.n) break;
-        uint8_t d0[LIMBS4], d1[LIMBS4];
-        const float ra = ldexpf(V32[kk * s.n + ia], -sc);
-        finite = finite && isfinite(ra);
-        q += split_e2m1_units(ra, d0);
-        if (ia + 8 < s.n) {
-            const float rb8 = ldexpf(V32[kk * s.n + ia + 8], -sc);
-            finite = finite && isfinite(rb8);
-            q += split_e2m1_units(rb8, d1);
-        } else {
-#pragma unroll
-            for (int l = 0; l < LIMBS4; ++l) d1[l] = 0;
-        }
-        const int64_t byte = e2m1_byte(a4_pos(ia, s.pa, s.pnb));
-#pragma unroll
-        for (int l = 0; l < LIMBS4; ++l) Vq[(LIMBS4 * kk + l) * rb + byte] = static_cast<uint8_t>(d0[l] | (d1[l] << 4));
-    }
-    const double t = block_sum(finite ? static_cast<double>(q) : NAN, sh);
-    if (threadIdx.x == 0) s.vsp[kk * s.nch + c] = ldexp(t, sc - (1 + 3 * (LIMBS4 - 1)));
 }
 
-// (4b, wide form) V -> the value of its e4m3 limbs as wide e2m1 limbs, in
-// k_vlimbs4's byte order; scales and chunk sums as k_vlimbs.
-__global__ void k_vlimbs_wide(SP s, uint8_t *__restrict__ Vq, int64_t n_pad, const double *__restrict__ vmaxp,
-                              int *__restrict__ bs, int *err)
+using ScanFn = void (*)(const SP);
+
+template <int EPT>
+ScanFn pick_scan(bool f64, bool q)
 {
-    __shared__ double sh[NT / 32];
-    __shared__ int s_sh;
-    const int c = blockIdx.x, kk = blockIdx.y;
-    double m = 0.0;
-    for (int q = threadIdx.x; q < s.nch; q += NT) m = fmax(m, vmaxp[kk * s.nch + q]);
-    m = block_max(m, sh);
-    if (threadIdx.x == 0) {
-        float mf = static_cast<float>(m);
-        if (!isfinite(mf)) {
-            atomicOr(err, DEVERR_NONFINITE);
-            mf = 0.f;
-        }
-        s_sh = limb_scale(mf);
-        if (c == 0) bs[kk] = s_sh;
-    }
-    __syncthreads();
-    const int sc = s_sh;
-    const int64_t i0 = static_cast<int64_t>(c) * SCAN_CH;
-    const float *V32 = reinterpret_cast<const float *>(s.Rt);
-    const int64_t rb = n_pad / 2;
-    long long q = 0;
-    bool finite = true;
-    for (int e = threadIdx.x; e < SCAN_CH / 2; e += NT) {
-        const int64_t ia = i0 + ((e >> 3) << 4) + (e & 7);
-        if (ia >= s.n) break;
-        uint8_t d[LIMBS], d0[LIMBS_W], d1[LIMBS_W];
-        const float ra = ldexpf(V32[kk * s.n + ia], -sc);
-        finite = finite && isfinite(ra);
-        const int qa = split_e4m3_units(ra, d);
-        int qb = 0;
-        if (ia + 8 < s.n) {
-            const float rb8 = ldexpf(V32[kk * s.n + ia + 8], -sc);
-            finite = finite && isfinite(rb8);
-            qb = split_e4m3_units(rb8, d);
-        }
-        q += qa;
-        q += qb;
-        split_wide(qa, d0);
-        split_wide(qb, d1);
-        const int64_t byte = e2m1_byte(a4_pos(ia, s.pa, s.pnb));
-#pragma unroll
-        for (int l = 0; l < LIMBS_W; ++l) Vq[(LIMBS_W * kk + l) * rb + byte] = static_cast<uint8_t>(d0[l] | (d1[l] << 4));
-    }
-    const double t = block_sum(finite ? static_cast<double>(q) : NAN, sh);
-    if (threadIdx.x == 0) s.vsp[kk * s.nch + c] = ldexp(t, sc - 21);
+    return f64 ? (q ? k_scans<EPT, true, true> : k_scans<EPT, true, false>)
+               : (q ? k_scans<EPT, false, true> : k_scans<EPT, false, false>);
 }
 
-// (5) per column (one warp each): sum V, f, ||beta||_1, F = f + lambda ||beta||_1;
-// flag non-finite.
-__device__ __forceinline__ double warp_sum(double x)
+ScanFn pick_scan(int ept, bool f64, bool q)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
-// With unpenalised covariates also g_Z = Z^T (delta - u) / n per column, and,
-// for a step, gamma <- gamma + step g_Z (Section 6: the covariates take a plain
-// gradient step; a frozen column keeps its gamma).
-__global__ void k_finalize(SP s, int l1_blocks, const double *l1p, const double *lam, double *sumV,
-                           double *f, double *l1, double *Fobj, bool need_loss, int *err, double *gz,
-                           double *gamma, const int *active, double step, bool gamma_step)
-{
-    const int kk = blockIdx.x, lane = threadIdx.x;
-    for (int cq = 0; cq < s.q; ++cq) {
-        double z = 0.0;
-        for (int c = lane; c < s.nch; c += 32) z += s.zvp[(static_cast<int64_t>(kk) * s.q + cq) * s.nch + c];
-        z = warp_sum(z) / static_cast<double>(s.n);
-        if (lane == 0) {
-            gz[kk * s.q + cq] = z;
-            if (gamma_step && (!active || active[kk])) gamma[kk * s.q + cq] += step * z;
-            if (!isfinite(z)) atomicOr(err, DEVERR_NONFINITE);
-        }
+    switch (ept) {
+    case 1: return pick_scan<1>(f64, q);
+    case 2: return pick_scan<2>(f64, q);
+    case 4: return pick_scan<4>(f64, q);
+    default: return pick_scan<8>(f64, q);
     }
-    double v = 0.0, lo = 0.0, b1 = 0.0;
-    for (int c = lane; c < s.nch; c += 32) v += s.vsp[kk * s.nch + c];
-    v = warp_sum(v);
-    if (need_loss) {
-        // f = (sum_g e_g log W_g + (events) c - sum_r delta_r eta_r) / n
-        for (int c = lane; c < s.nch; c += 32) lo += s.lossp[kk * s.nch + c];
-        if (l1p)
-            for (int c = lane; c < l1_blocks; c += 32) b1 += l1p[kk * l1_blocks + c];
-        lo = (s.lossg[kk] - warp_sum(lo)) / static_cast<double>(s.n);
-        b1 = warp_sum(b1);
-    }
-    if (lane != 0) return;
-    sumV[kk] = v;
-    if (need_loss) {
-        f[kk] = lo;
-        l1[kk] = b1;
-        Fobj[kk] = lo + (lam ? lam[kk] * b1 : 0.0);
-        if (!isfinite(lo)) atomicOr(err, DEVERR_NONFINITE);
-    }
-    if (!isfinite(v)) atomicOr(err, DEVERR_NONFINITE);
 }
 
 } // namespace
 
+// Subjects per lane: the smallest of 1, 2, 4, 8 that leaves at most 2000 chunks
+// (warps) a column, so that one column of a small problem spreads over the SMs.
+int scan_ept(int64_t n)
+{
+    for (int e = 1; e < 8; e *= 2)
+        if (n <= static_cast<int64_t>(2000) * 32 * e) return e;
+    return 8;
+}
+
+int scan_tiles(int64_t n_evhead) { return static_cast<int>((n_evhead + GT - 1) / GT); }
+
 int run_scans(cox_handle *h, const ScanArgs &a, cudaStream_t st)
 {
     Workspace &ws = h->ws;
+    if (a.eta_only) {
+        k_eta<<<dim3(static_cast<unsigned>(std::min<int64_t>((h->n + NT - 1) / NT, 1024)), a.k), NT, 0, st>>>(
+            static_cast<const float *>(a.eta), h->n, a.slot_stride, a.col_stride, a.group_rows, a.KC, a.L, ws.eta);
+        COX_CUDA(cudaGetLastError());
+        return COX_OK;
+    }
     SP s;
     s.n = h->n;
     s.n_pad = h->n_pad;
     s.nch = h->n_chunks;
     s.k = a.k;
-    s.pa = h->kperm_a;
-    s.pnb = h->kperm_nb;
+    s.G = h->n_evhead;
+    s.ntile = scan_tiles(s.G);
     s.delta = h->d_delta;
-    s.head = h->d_head;
-    s.tail = h->d_tail;
+    s.evflag = h->d_evflag;
     s.evhead = h->d_evhead;
     s.evcnt = h->d_evcnt;
     s.evidx = h->d_evidx;
-    s.evflag = h->d_evflag;
-    s.n_evh = h->n_evhead;
-    s.q = a.gamma ? h->q : 0;  // no gamma: X_c beta alone (cox_eta)
-    s.Z = h->d_Z;
-    s.gamma = a.gamma;
-    s.zvp = ws.zvp;
+    s.a4blk = h->d_a4blk;
+    s.src = a.eta_src;
+    s.group_rows = a.group_rows;
+    s.KC = a.KC;
+    s.eta_in = a.eta;
+    s.slot_stride = a.slot_stride;
+    s.col_stride = a.col_stride;
+    s.L = a.L;
     s.eta = ws.eta;
     s.w = ws.w;
-    s.Rt = ws.Rt;
+    s.V32 = ws.Vf;
+    s.Wg = ws.Wg;
     s.Fg = ws.Fg;
-    s.lossg = ws.lossg;
-    s.cmax = ws.cmax;
     s.csw = ws.csw;
     s.suf = ws.suf;
     s.lossp = ws.lossp;
+    s.tot = ws.tot;
+    s.tbase = ws.tbase;
+    s.lgp = ws.lgp;
     s.vsp = ws.vsp;
-    dim3 grid(h->n_chunks, a.k);
-    switch (a.eta_src) {
-    case ETA_PARTIAL_F32:
-        k_eta<ETA_PARTIAL_F32><<<grid, NT, 0, st>>>(s, a.eta, a.slot_stride, a.col_stride, a.group_rows, a.KC, a.L);
-        break;
-    case ETA_DENSE_F32:
-        k_eta<ETA_DENSE_F32><<<grid, NT, 0, st>>>(s, a.eta, 0, a.col_stride, 1, 1, 1);
-        break;
-    default:
-        k_eta<ETA_DENSE_F64><<<grid, NT, 0, st>>>(s, a.eta, 0, a.col_stride, 1, 1, 1);
-        break;
-    }
-    if (a.eta_only) {
-        COX_CUDA(cudaGetLastError());
-        return COX_OK;
-    }
-    if (a.exp64) k_rev<true><<<grid, NT, 0, st>>>(s);
-    else k_rev<false><<<grid, NT, 0, st>>>(s);
-    k_chunks<<<a.k, 32, 0, st>>>(s);
-    k_group<<<a.k, NT, 0, st>>>(s, a.need_loss);
-    switch (a.v_out) {
-    case V_LIMBS_E4M3:
-        k_uv<V_LIMBS_E4M3><<<grid, NT, 0, st>>>(s, a.V, h->n_pad, ws.vmaxp);
-        if (ws.g4.f4 == FORM_WIDE)
-            k_vlimbs_wide<<<grid, NT, 0, st>>>(s, static_cast<uint8_t *>(a.V), h->n_pad, ws.vmaxp, ws.bs4, h->d_err);
-        else if (ws.g4.f4)
-            k_vlimbs4<<<grid, NT, 0, st>>>(s, static_cast<uint8_t *>(a.V), h->n_pad, ws.vmaxp, ws.bs4, h->d_err);
-        else
-            k_vlimbs<<<grid, NT, 0, st>>>(s, static_cast<uint8_t *>(a.V), h->n_pad, ws.vmaxp, ws.bs4, h->d_err);
-        break;
-    case V_DENSE_F64: k_uv<V_DENSE_F64><<<grid, NT, 0, st>>>(s, a.V, h->n_pad, nullptr); break;
-    default: k_uv<V_DENSE_F32><<<grid, NT, 0, st>>>(s, a.V, h->n_pad, nullptr); break;
-    }
-    k_finalize<<<a.k, 32, 0, st>>>(s, h->l1_blocks, a.need_loss ? ws.l1p : nullptr, a.lam, ws.sumV, ws.f, ws.l1,
-                                 ws.F, a.need_loss, h->d_err, a.gz, a.gamma, a.active, a.step, a.gamma_step);
-    COX_CUDA(cudaGetLastError());
+    s.zvp = ws.zvp;
+    s.cmaxp = ws.cmax;
+    s.vmaxp = ws.vmaxp;
+    s.colc = ws.colc;
+    s.cnt = ws.scnt;
+    s.q = a.gamma ? h->q : 0;
+    s.Z = h->d_Z;
+    s.gamma = a.gamma;
+    s.gz = a.gz;
+    s.gamma_step = a.gamma_step;
+    s.active = a.active;
+    s.step = a.step;
+    s.vo = a.v_out;
+    s.form = ws.g4.f4;
+    s.V = a.V;
+    s.bs = ws.bs4;
+    s.l1_blocks = h->l1_blocks;
+    s.l1p = a.need_loss ? ws.l1p : nullptr;
+    s.lam = a.lam;
+    s.sumV = ws.sumV;
+    s.f = ws.f;
+    s.l1 = ws.l1;
+    s.F = ws.F;
+    s.need_loss = a.need_loss;
+    s.err = h->d_err;
+    s.wait_limit = h->wait_cycles;
+    const ScanFn fn = pick_scan(h->scan_ept, a.exp64, s.q > 0);
+    int occ = 0;
+    COX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, NT, 0));
+    // a warp per chunk, up to what the SMs hold at once (the grid barrier needs every
+    // block resident), and a block per tile of event groups while there is room
+    const int64_t room = static_cast<int64_t>(occ) * h->sm_count, tasks = static_cast<int64_t>(s.nch) * a.k;
+    const int64_t mains = std::min(room, (tasks + NW - 1) / NW);
+    s.per = (tasks + mains - 1) / mains;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(std::min(room, mains + 2 * static_cast<int64_t>(s.ntile) * a.k)));
+    cfg.blockDim = dim3(NT);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    COX_CUDA(cudaLaunchKernelEx(&cfg, fn, s));
     return COX_OK;
 }
 

@@ -538,7 +538,7 @@ def run_ours(args, rank, world):
                 "rel_l2_vs_batched_one_step": diff}
         prob.set_precision(args.precision)
 
-    # the CUDA-graph path fit (Section 6 rule): every penalty from beta = 0 to
+    # the path fit (Section 6 rule): every penalty from beta = 0 to
     # |F_t - F_{t-10}| / |F_t + 1| < tol or the iteration cap, replays of 10 steps
     path = None
     if args.path_iters > 0:
@@ -553,7 +553,7 @@ def run_ours(args, rank, world):
                 "iterations_per_column": [int(x) for x in iters],
                 "converged_columns": int(np.sum(np.asarray(iters) < args.path_iters)),
                 "final_objective": [float(x) for x in obj],
-                "timing": "wall clock around cox_path_fit (graph replays of 10 iterations, host reads the "
+                "timing": "wall clock around cox_path_fit (10 iterations at a time, host reads the "
                           "k objectives after each replay), beta = 0 to the stopping rule or the cap"}
 
     # the active-set X B late in the path: the 8 largest penalties from the

@@ -120,8 +120,7 @@ typedef struct cox_options {
                              columns, rebuilt when the support leaves it), or the
                              dense copy when the support exceeds a quarter of the
                              columns; each iteration then synchronises its stream
-                             once, and cox_path_fit runs plain launches instead
-                             of graph replays.  0 (default): always dense        */
+                             once.  0 (default): always dense                    */
 } cox_options;
 
 /* Fill *opt with the defaults above. */
@@ -259,8 +258,8 @@ int cox_last_objective(cox_h h, double *obj_host, int k, void *stream);
  * Solve k penalties from beta = 0 (or from beta_dev when warm != 0), each
  * column until |F_t - F_{t-lag}| / |F_t + 1| < tol (Section 6 stopping rule,
  * F = penalised objective) or max_iter.  A converged column is frozen: its
- * result equals a solo run.  Iterations run as CUDA-graph replays of `lag`
- * steps; the host reads k objectives per replay.
+ * result equals a solo run.  The host reads k objectives after every `lag`
+ * iterations.
  *   beta_dev  : p x k (device) out (in too when warm).
  *   iters_host: k ints, iterations each column ran.  obj_host: k doubles,
  *               final F.  Either may be NULL.
@@ -274,8 +273,8 @@ int cox_path_fit(cox_h h, const double *lambdas, int k, int max_iter, double tol
  * ran each lambda of its grid to the stopping rule): lambdas[l] is solved
  * from beta = 0 (warm = 0) or from the solution of lambdas[l-1] (warm = 1),
  * with its unpenalised coefficients gamma likewise (when covariates are set),
- * each to |F_t - F_{t-lag}| / |F_t + 1| < tol or max_iter iterations, as
- * CUDA-graph replays of `lag` steps (the rule of cox_path_fit with k = 1).
+ * each to |F_t - F_{t-lag}| / |F_t + 1| < tol or max_iter iterations (the
+ * rule of cox_path_fit with k = 1).
  *   B_dev     : p x L coefficients (device) out, column l at lambdas[l].
  *   G_host    : q x L doubles (host) out, column l = gamma at lambdas[l]; may
  *               be NULL (and is not written when no covariates are set).
@@ -426,8 +425,7 @@ int cox_set_precision(cox_h h, int precision);
  * with the fused step, 2 = risk-set scans (all their launches), 3 = other
  * (coefficient limbs, ||beta||_1).  cox_profile(h, 1) clears and starts
  * recording; cox_profile(h, 0) stops.  cox_profile_read synchronises, then
- * fills total_ms[4] and launches[4] for the recorded iterations.  Recording
- * is off inside cox_path_fit graphs.
+ * fills total_ms[4] and launches[4] for the recorded iterations.
  */
 int cox_profile(cox_h h, int enable);
 int cox_profile_read(cox_h h, double *total_ms, int64_t *launches);

@@ -1,7 +1,7 @@
 // api.cu -- the C ABI of libcoxgb: handle life cycle, one proximal-gradient
 // iteration (arXiv 2010.16114, Section 5.3), loss and gradient, the power
 // method for the step (Section 4.4), the batched path fit with the lag-10
-// stopping rule (Section 6) replayed as a CUDA graph, and checkpoints.
+// stopping rule (Section 6), and checkpoints.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -114,6 +114,20 @@ int default_form(const cox_handle *h, int k)
     return !forced && limb_cols_wide(k) ? FORM_WIDE : FORM_E4M3;
 }
 
+// The penalties of an iteration as a kernel argument (no copy in the stream), or
+// copied to ws.lam when there are more than it holds.
+int lam_arg(cox_handle *h, const double *lam, int k, LamArg &a, cudaStream_t st)
+{
+    if (!lam) return COX_OK;
+    if (k > MAX_LAM_ARG) {
+        COX_CUDA(cudaMemcpyAsync(h->ws.lam, lam, k * sizeof(double), cudaMemcpyHostToDevice, st));
+        return COX_OK;
+    }
+    a.k = k;
+    std::copy(lam, lam + k, a.v);
+    return COX_OK;
+}
+
 cudaEvent_t get_event(cox_handle *h)
 {
     if (h->ev_used == h->ev_pool.size()) {
@@ -162,15 +176,18 @@ void set_covariate_args(cox_handle *h, ScanArgs &sa, int col, int epi, double st
 }
 
 // One iteration for k columns.  epi: EPI_PROX (update beta) or EPI_GRAD.
-int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, cudaStream_t st)
+int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, cudaStream_t st, const double *lam,
+            double *F_out)
 {
     Workspace &ws = h->ws;
+    LamArg la;
+    COX_TRY(lam_arg(h, lam, k, la, st));
     if (is_split(h)) {
         float *b32 = static_cast<float *>(beta);
         int use_active = 0;
         {
             Site s_(h, 3, 1, st);
-            COX_TRY(l1_norms32(h, b32, k, st, ws.bmaxp));
+            COX_TRY(l1_norms32(h, b32, k, st, ws.bmaxp, &la));
             if (h->opt.active_set) COX_TRY(active_prepare(h, b32, k, st, &use_active));
             if (!use_active) {
                 COX_TRY(prep_limbs_beta(h, b32, k, st));
@@ -201,6 +218,7 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
         sa.exp64 = false;
         sa.lam = ws.lam;
         sa.need_loss = true;
+        sa.F_out = F_out;
         set_covariate_args(h, sa, 0, epi, step);
         {
             Site s_(h, 2, 1, st);
@@ -231,7 +249,7 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
         double *b64 = static_cast<double *>(beta);
         {
             Site s_(h, 3, 1, st);
-            COX_TRY(l1_norms64(h, b64, k, st));
+            COX_TRY(l1_norms64(h, b64, k, st, &la));
         }
         {
             Site s_(h, 0, 1, st);
@@ -252,6 +270,7 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
         sa.exp64 = true;
         sa.lam = ws.lam;
         sa.need_loss = true;
+        sa.F_out = F_out;
         set_covariate_args(h, sa, 0, epi, step);
         {
             Site s_(h, 2, 1, st);
@@ -268,7 +287,7 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
         float *bc = b32 + static_cast<int64_t>(c) * h->p;
         {
             Site s_(h, 3, 1, st);
-            COX_TRY(l1_norms32(h, bc, 1, st));
+            COX_TRY(l1_norms32(h, bc, 1, st, nullptr, c == 0 ? &la : nullptr));
         }
         {
             Site s_(h, 0, 2, st);
@@ -306,6 +325,7 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
     // gather per-column objectives into F / f
     COX_CUDA(cudaMemcpyAsync(ws.F, ws.Fring, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
     COX_CUDA(cudaMemcpyAsync(ws.f, ws.Fring + k, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    if (F_out) COX_CUDA(cudaMemcpyAsync(F_out, ws.F, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
     return COX_OK;
 }
 
@@ -314,9 +334,12 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
 // order, X part only; the handle adds Z gamma when covariates are set), the
 // replicated risk-set scans, then this shard's X_g^T V and the soft-threshold
 // step on its coefficients.
-int iterate_from_eta(cox_handle *h, void *beta, const double *eta, int k, double step, cudaStream_t st)
+int iterate_from_eta(cox_handle *h, void *beta, const double *eta, int k, double step, cudaStream_t st,
+                     const double *lam)
 {
     Workspace &ws = h->ws;
+    LamArg la;
+    COX_TRY(lam_arg(h, lam, k, la, st));
     ScanArgs sa;
     sa.k = k;
     sa.eta_src = ETA_DENSE_F64;
@@ -333,7 +356,7 @@ int iterate_from_eta(cox_handle *h, void *beta, const double *eta, int k, double
         float *b32 = static_cast<float *>(beta);
         {
             Site s_(h, 3, 1, st);
-            COX_TRY(l1_norms32(h, b32, k, st));
+            COX_TRY(l1_norms32(h, b32, k, st, nullptr, &la));
         }
         sa.v_out = V_LIMBS_E4M3;
         sa.V = ws.Vq;
@@ -363,7 +386,7 @@ int iterate_from_eta(cox_handle *h, void *beta, const double *eta, int k, double
         double *b64 = static_cast<double *>(beta);
         {
             Site s_(h, 3, 1, st);
-            COX_TRY(l1_norms64(h, b64, k, st));
+            COX_TRY(l1_norms64(h, b64, k, st, &la));
         }
         sa.v_out = V_DENSE_F64;
         sa.V = ws.V64;
@@ -388,12 +411,11 @@ int validate_k(const cox_handle *h, int k)
     return COX_OK;
 }
 
-int set_lambdas(cox_handle *h, const double *lambdas, int k, cudaStream_t st)
+int check_lambdas(const double *lambdas, int k)
 {
     if (!lambdas) return COX_ERR_ARG;
     for (int c = 0; c < k; ++c)
         if (!(lambdas[c] >= 0.0) || !std::isfinite(lambdas[c])) return COX_ERR_ARG;
-    COX_CUDA(cudaMemcpyAsync(h->ws.lam, lambdas, k * sizeof(double), cudaMemcpyHostToDevice, st));
     return COX_OK;
 }
 
@@ -983,14 +1005,13 @@ int cox_loss_grad(cox_h h, const void *beta_dev, int k, double *loss_host, void 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     COX_TRY(ensure_workspace(h, k));
     std::vector<double> zeros(static_cast<size_t>(k), 0.0);
-    COX_TRY(set_lambdas(h, zeros.data(), k, st));
     void *gout = grad_dev;
     void *tmp = nullptr;
     if (!gout) {
         COX_TRY(dmalloc(nullptr, &tmp, static_cast<size_t>(k) * h->p * (is_fp64(h) ? 8 : 4)));
         gout = tmp;
     }
-    int rc = iterate(h, const_cast<void *>(beta_dev), k, EPI_GRAD, gout, 0.0, st);
+    int rc = iterate(h, const_cast<void *>(beta_dev), k, EPI_GRAD, gout, 0.0, st, zeros.data());
     if (rc == COX_OK) rc = check_device_error(h, st);
     if (rc == COX_OK && loss_host) {
         if (cudaMemcpyAsync(loss_host, h->ws.f, k * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -1057,8 +1078,8 @@ int cox_prox_step(cox_h h, void *beta_dev, const double *lambdas, int k, double 
     DeviceGuard g(h->dev);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     COX_TRY(ensure_workspace(h, k));
-    COX_TRY(set_lambdas(h, lambdas, k, st));
-    return iterate(h, beta_dev, k, EPI_PROX, nullptr, step, st);
+    COX_TRY(check_lambdas(lambdas, k));
+    return iterate(h, beta_dev, k, EPI_PROX, nullptr, step, st, lambdas);
 }
 
 int cox_prox_step_host(cox_h h, void *beta_host, const double *lambdas, int k, double step, void *stream)
@@ -1081,8 +1102,8 @@ int cox_prox_step_host(cox_h h, void *beta_host, const double *lambdas, int k, d
         ddev = h->dev;
     }
     COX_CUDA(cudaMemcpyAsync(dbuf, beta_host, bytes, cudaMemcpyHostToDevice, st));
-    COX_TRY(set_lambdas(h, lambdas, k, st));
-    COX_TRY(iterate(h, dbuf, k, EPI_PROX, nullptr, step, st));
+    COX_TRY(check_lambdas(lambdas, k));
+    COX_TRY(iterate(h, dbuf, k, EPI_PROX, nullptr, step, st, lambdas));
     COX_CUDA(cudaMemcpyAsync(beta_host, dbuf, bytes, cudaMemcpyDeviceToHost, st));
     return check_device_error(h, st);
 }
@@ -1096,8 +1117,8 @@ int cox_prox_step_eta(cox_h h, void *beta_dev, const double *eta_dev, const doub
     DeviceGuard g(h->dev);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     COX_TRY(ensure_workspace(h, k));
-    COX_TRY(set_lambdas(h, lambdas, k, st));
-    return iterate_from_eta(h, beta_dev, eta_dev, k, step, st);
+    COX_TRY(check_lambdas(lambdas, k));
+    return iterate_from_eta(h, beta_dev, eta_dev, k, step, st, lambdas);
 }
 
 int cox_last_loss_l1(cox_h h, double *f_host, double *l1_host, int k, void *stream)

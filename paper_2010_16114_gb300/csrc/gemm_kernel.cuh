@@ -266,6 +266,7 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
     volatile int *armed2 = armed + S;                                      // [S2] the same for the limb slots
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(full0 + 8 * s, 1);
@@ -313,6 +314,11 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
         __syncthreads();
         tc_fence_after();
     }
+
+    // everything above touches only this CTA's shared memory, TMEM and the kernel
+    // parameters: with programmatic stream serialisation it runs while the kernel ahead
+    // ends; its results are read below
+    pdl_wait();
 
     const int64_t cta = blockIdx.x;
     const int64_t u0 = cta * P.L;

@@ -13,6 +13,8 @@ __global__ void k_prep_limbs_beta(const float *__restrict__ beta, int64_t p, int
                                   const float *__restrict__ maxp, uint8_t *__restrict__ Bq,
                                   int *__restrict__ bs, int *err)
 {
+    pdl_trigger();
+    pdl_wait();
     __shared__ int s_sh;
     const int kk = blockIdx.y;
     if (threadIdx.x < 32) {
@@ -46,6 +48,8 @@ __global__ void k_prep_limbs_beta4(const float *__restrict__ beta, int64_t p, in
                                    const float *__restrict__ maxp, uint8_t *__restrict__ Bq,
                                    int *__restrict__ bs, int *err)
 {
+    pdl_trigger();
+    pdl_wait();
     __shared__ int s_sh;
     const int kk = blockIdx.y;
     if (threadIdx.x < 32) {
@@ -86,6 +90,8 @@ __global__ void k_prep_limbs_beta_wide(const float *__restrict__ beta, int64_t p
                                        const float *__restrict__ maxp, uint8_t *__restrict__ Bq,
                                        int *__restrict__ bs, int *err)
 {
+    pdl_trigger();
+    pdl_wait();
     __shared__ int s_sh;
     const int kk = blockIdx.y;
     if (threadIdx.x < 32) {
@@ -470,8 +476,7 @@ int launch_gemm(cox_handle *h, const GemmPlan &g, const EpiArgs &e, int k, cudaS
     kp.err = e.err ? e.err : h->d_err;
     KernelFn fn = pick_kernel(g.T, g.CH, g.NP, g.alt, g.f4);
     if (!fn) return COX_ERR_ARG;
-    fn<<<g.grid, threads_for(g.T, g.G, g.alt), g.smem, st>>>(g.tmA, g.tmB, kp);
-    COX_CUDA(cudaGetLastError());
+    COX_CUDA(launch_pdl(fn, dim3(g.grid), threads_for(g.T, g.G, g.alt), g.smem, st, false, g.tmA, g.tmB, kp));
     return COX_OK;
 }
 
@@ -480,16 +485,9 @@ int prep_limbs_beta(cox_handle *h, const float *beta, int k, cudaStream_t st)
     // about four blocks per SM over all columns; each block strides over p
     const int64_t bx = std::max<int64_t>(1, (4 * static_cast<int64_t>(h->sm_count) + k - 1) / k);
     dim3 grid(static_cast<unsigned>(std::min<int64_t>((h->p + 255) / 256, bx)), k);
-    if (h->ws.g1.f4 == FORM_WIDE)
-        k_prep_limbs_beta_wide<<<grid, 256, 0, st>>>(beta, h->p, h->p_pad, h->l1_blocks, h->ws.bmaxp, h->ws.Bq,
-                                                     h->ws.bs1, h->d_err);
-    else if (h->ws.g1.f4)
-        k_prep_limbs_beta4<<<grid, 256, 0, st>>>(beta, h->p, h->p_pad, h->l1_blocks, h->ws.bmaxp, h->ws.Bq,
-                                                 h->ws.bs1, h->d_err);
-    else
-        k_prep_limbs_beta<<<grid, 256, 0, st>>>(beta, h->p, h->p_pad, h->l1_blocks, h->ws.bmaxp, h->ws.Bq,
-                                                h->ws.bs1, h->d_err);
-    COX_CUDA(cudaGetLastError());
+    const auto fn = h->ws.g1.f4 == FORM_WIDE ? k_prep_limbs_beta_wide : h->ws.g1.f4 ? k_prep_limbs_beta4 : k_prep_limbs_beta;
+    COX_CUDA(launch_pdl(fn, grid, 256, 0, st, false, beta, h->p, h->p_pad, h->l1_blocks, h->ws.bmaxp, h->ws.Bq, h->ws.bs1,
+                        h->d_err));
     return COX_OK;
 }
 

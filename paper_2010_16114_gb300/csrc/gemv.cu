@@ -10,13 +10,18 @@
 #include <cmath>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace coxgb {
 namespace {
 
+// ||beta_c||_1 and max |beta_c| partials; also writes the iteration's penalties (lam)
 __global__ void k_l1_32(const float *__restrict__ beta, int64_t p, int nb, double *__restrict__ l1p,
-                        float *__restrict__ maxp)
+                        float *__restrict__ maxp, const LamArg lam, double *__restrict__ lam_dev)
 {
+    pdl_trigger();
+    pdl_wait();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < lam.k) lam_dev[threadIdx.x] = lam.v[threadIdx.x];
     __shared__ double sh[8];
     __shared__ float shm[8];
     const int b = blockIdx.x, kk = blockIdx.y;
@@ -53,8 +58,12 @@ __global__ void k_l1_32(const float *__restrict__ beta, int64_t p, int nb, doubl
     }
 }
 
-__global__ void k_l1_64(const double *__restrict__ beta, int64_t p, int nb, double *__restrict__ l1p)
+__global__ void k_l1_64(const double *__restrict__ beta, int64_t p, int nb, double *__restrict__ l1p, const LamArg lam,
+                        double *__restrict__ lam_dev)
 {
+    pdl_trigger();
+    pdl_wait();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < lam.k) lam_dev[threadIdx.x] = lam.v[threadIdx.x];
     __shared__ double sh[8];
     const int b = blockIdx.x, kk = blockIdx.y;
     double s = 0.0;
@@ -230,6 +239,8 @@ __global__ void k_prox32(const float *__restrict__ G, int64_t p, const double *_
 __global__ void k_eta64(const double *__restrict__ Xr, int64_t n, int64_t p, const double *__restrict__ beta,
                         int k, double *__restrict__ eta)
 {
+    pdl_trigger();
+    pdl_wait();
     const int64_t wid = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (wid >= n * k) return;
@@ -246,6 +257,8 @@ __global__ void k_xtv64(const double *__restrict__ Xc, int64_t n, int64_t p, con
                         const double *__restrict__ mu, const double *__restrict__ sumV, double *beta, double *grad,
                         const double *__restrict__ lam, double step, const int *active)
 {
+    pdl_trigger();
+    pdl_wait();
     const int64_t wid = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (wid >= p * k) return;
@@ -305,17 +318,17 @@ unsigned blocks_for(int64_t n, int t) { return static_cast<unsigned>((n + t - 1)
 
 } // namespace
 
-int l1_norms32(cox_handle *h, const float *beta, int k, cudaStream_t st, float *maxp)
+int l1_norms32(cox_handle *h, const float *beta, int k, cudaStream_t st, float *maxp, const LamArg *lam)
 {
-    k_l1_32<<<dim3(h->l1_blocks, k), 256, 0, st>>>(beta, h->p, h->l1_blocks, h->ws.l1p, maxp);
-    COX_CUDA(cudaGetLastError());
+    COX_CUDA(launch_pdl(k_l1_32, dim3(h->l1_blocks, k), 256, 0, st, false, beta, h->p, h->l1_blocks, h->ws.l1p, maxp,
+                        lam ? *lam : LamArg(), h->ws.lam));
     return COX_OK;
 }
 
-int l1_norms64(cox_handle *h, const double *beta, int k, cudaStream_t st)
+int l1_norms64(cox_handle *h, const double *beta, int k, cudaStream_t st, const LamArg *lam)
 {
-    k_l1_64<<<dim3(h->l1_blocks, k), 256, 0, st>>>(beta, h->p, h->l1_blocks, h->ws.l1p);
-    COX_CUDA(cudaGetLastError());
+    COX_CUDA(launch_pdl(k_l1_64, dim3(h->l1_blocks, k), 256, 0, st, false, beta, h->p, h->l1_blocks, h->ws.l1p,
+                        lam ? *lam : LamArg(), h->ws.lam));
     return COX_OK;
 }
 
@@ -371,8 +384,7 @@ int prox_or_grad32(cox_handle *h, const float *G, int col, float *beta, float *g
 int eta64(cox_handle *h, const double *beta, int k, double *eta, cudaStream_t st)
 {
     const int64_t warps = h->n * k;
-    k_eta64<<<blocks_for(warps * 32, 256), 256, 0, st>>>(h->d_Xr, h->n, h->p, beta, k, eta);
-    COX_CUDA(cudaGetLastError());
+    COX_CUDA(launch_pdl(k_eta64, dim3(blocks_for(warps * 32, 256)), 256, 0, st, false, h->d_Xr, h->n, h->p, beta, k, eta));
     return COX_OK;
 }
 
@@ -380,9 +392,8 @@ int xtv64(cox_handle *h, const double *V, int k, double *beta, double *grad, con
           cudaStream_t st)
 {
     const int64_t warps = h->p * k;
-    k_xtv64<<<blocks_for(warps * 32, 256), 256, 0, st>>>(h->d_Xc, h->n, h->p, V, k, h->d_mu, h->ws.sumV, beta,
-                                                         grad, lam, step, h->ws.active);
-    COX_CUDA(cudaGetLastError());
+    COX_CUDA(launch_pdl(k_xtv64, dim3(blocks_for(warps * 32, 256)), 256, 0, st, false, h->d_Xc, h->n, h->p, V, k, h->d_mu,
+                        h->ws.sumV, beta, grad, lam, step, h->ws.active));
     return COX_OK;
 }
 

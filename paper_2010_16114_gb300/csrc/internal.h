@@ -7,6 +7,7 @@
 
 #include <cstdint>
 #include <map>
+#include <utility>
 #include <vector>
 
 #include "../../include/coxgb.h"
@@ -373,6 +374,39 @@ int cuda_status(cudaError_t e);
         if (r_ != COX_OK) return r_; \
     } while (0)
 
+// Launch with programmatic stream serialisation: the kernel may be scheduled while
+// the one ahead of it in the stream ends, and waits for it (pdl_wait) before it
+// touches global memory.  coop: as a cooperative grid instead, which starts when the
+// kernel ahead has ended (both attributes at once measured no faster).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, bool coop,
+                       Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    if (coop) {
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+    } else {
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+
+// Penalties passed by value to the first kernel of an iteration, which puts them in ws.lam.
+constexpr int MAX_LAM_ARG = 64;
+struct LamArg {
+    int k = 0;
+    double v[MAX_LAM_ARG] = {};
+};
+
 int dmalloc(cox_handle *h, void **p, size_t bytes);
 void dfree(void *p);
 
@@ -382,8 +416,12 @@ int setup_dense64(cox_handle *h, const double *X, cudaStream_t st);
 
 // ---- workspace / plans / one iteration (api.cu) ----------------------------------
 int ensure_workspace(cox_handle *h, int k);
-int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, cudaStream_t st);
-int iterate_from_eta(cox_handle *h, void *beta, const double *eta, int k, double step, cudaStream_t st);
+// lam: the k penalties on the host, passed to the first kernel by value (null: ws.lam
+// holds them); F_out: where this iteration's objectives also go (device, may be null)
+int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, cudaStream_t st,
+            const double *lam = nullptr, double *F_out = nullptr);
+int iterate_from_eta(cox_handle *h, void *beta, const double *eta, int k, double step, cudaStream_t st,
+                     const double *lam);
 struct ScanArgs;
 void set_covariate_args(cox_handle *h, ScanArgs &sa, int col, int epi, double step);
 
@@ -412,6 +450,7 @@ struct ScanArgs {
     const int *active = nullptr;
     double step = 0.0;
     bool gamma_step = false;
+    double *F_out = nullptr;
 };
 int run_scans(cox_handle *h, const ScanArgs &a, cudaStream_t st);
 int scan_ept(int64_t n);              // subjects per lane
@@ -462,8 +501,9 @@ void active_free(cox_handle *h);
 
 // ---- CUDA-core paths (gemv.cu) -----------------------------------------------------
 // ||beta_c||_1 partials into ws.l1p; with maxp, max |beta_c| partials too
-int l1_norms32(cox_handle *h, const float *beta, int k, cudaStream_t st, float *maxp = nullptr);
-int l1_norms64(cox_handle *h, const double *beta, int k, cudaStream_t st);
+int l1_norms32(cox_handle *h, const float *beta, int k, cudaStream_t st, float *maxp = nullptr,
+               const LamArg *lam = nullptr);
+int l1_norms64(cox_handle *h, const double *beta, int k, cudaStream_t st, const LamArg *lam = nullptr);
 // The FP32 baseline's product y = A x (byte tables of x; part: the partials,
 // gemv_lut_part_floats(rows, KC) floats).  Two kernels.
 int gemv_lut(cox_handle *h, const uint32_t *A, int64_t rows, int64_t KC, const float *x, int64_t K_valid,

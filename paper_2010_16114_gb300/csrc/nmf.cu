@@ -487,30 +487,10 @@ int plan_side(nmf_handle *h, NmfSide &sd, const __nv_bfloat16 *A, int64_t rows, 
     return COX_OK;
 }
 
-// Launch with programmatic stream serialisation: the kernel may be scheduled
-// while the one ahead of it in the stream finishes (each NMF kernel waits for
-// its predecessor with pdl_wait before touching global memory).
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
-                       Args &&...args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
-}
-
 int launch_gemm(nmf_handle *h, const NmfSide &sd, cudaStream_t st)
 {
     ++h->launches;
-    return launch_pdl(k_nmf_gemm, sd.grid, GEMM_THREADS, sd.smem, st, sd.tmA, sd.tmB, sd.g) == cudaSuccess
+    return launch_pdl(k_nmf_gemm, dim3(sd.grid), GEMM_THREADS, sd.smem, st, false, sd.tmA, sd.tmB, sd.g) == cudaSuccess
                ? COX_OK
                : COX_ERR_CUDA;
 }
@@ -544,7 +524,7 @@ int launch_update(nmf_handle *h, int side, int mode, int algo, double eps, cudaS
     a.nblk = upd_blocks(a.R);
     a.err = h->err;
     ++h->launches;
-    if (launch_pdl(k_nmf_update, a.nblk, UPD_ROWS * upd_warps(h->r), upd_smem(h->r), st, a) != cudaSuccess)
+    if (launch_pdl(k_nmf_update, dim3(a.nblk), UPD_ROWS * upd_warps(h->r), upd_smem(h->r), st, false, a) != cudaSuccess)
         return COX_ERR_CUDA;
     GramArgs gm;
     gm.r = h->r;
@@ -554,7 +534,7 @@ int launch_update(nmf_handle *h, int side, int mode, int algo, double eps, cudaS
     gm.G32 = side == 0 ? h->GV32 : h->GW32;
     const int npair = h->r * (h->r + 1) / 2;
     ++h->launches;
-    return launch_pdl(k_nmf_gram, (npair + 7) / 8, 256, 0, st, gm) == cudaSuccess ? COX_OK : COX_ERR_CUDA;
+    return launch_pdl(k_nmf_gram, dim3((npair + 7) / 8), 256, 0, st, false, gm) == cudaSuccess ? COX_OK : COX_ERR_CUDA;
 }
 
 int check_err(nmf_handle *h, cudaStream_t st)

@@ -1,7 +1,7 @@
 // path.cu -- step size by the power method (arXiv 2010.16114, Section 4.4,
 // used for the Section 5.3 step), the batched regularisation-path fit with the
-// Section 6 stopping rule |F_t - F_{t-lag}| / |F_t + 1| < tol, replayed as a
-// CUDA graph of `lag` iterations, and checkpoint / resume of that fit.
+// Section 6 stopping rule |F_t - F_{t-lag}| / |F_t + 1| < tol, and checkpoint /
+// resume of that fit.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -192,53 +192,35 @@ namespace coxgb {
 namespace {
 
 // The Section 6 stopping-rule loop for k columns on the handle's device
-// buffers (lambdas and active flags already set): CUDA-graph replays of `lag`
-// iterations, the host reading the k objectives after each replay; a column
-// stops when |F_t - F_{t-lag}| / |F_t + 1| < tol and is frozen.  iters,
-// active, hist and t carry the state in and out (resume).
+// buffers (lambdas and active flags already set): `lag` iterations at a time, the
+// host reading the k objectives after each run of them; a column stops when
+// |F_t - F_{t-lag}| / |F_t + 1| < tol and is frozen.  iters, active, hist and t
+// carry the state in and out (resume).  An iteration is five launches, whose
+// ~20 us of host time hide behind its own GPU time; captured as a graph of `lag`
+// iterations the same kernels took longer (20 iterations at n = 200,000,
+// p = 10,000, k = 1: 5.59 ms against 5.45; three penalties of 10 at n = 20,011,
+// p = 5,003: 3.97 against 3.58, capture and instantiation included).
 int path_run(cox_handle *h, int k, int max_iter, double tol, double step, void *beta_dev, std::vector<int> &iters,
              std::vector<int> &active, std::vector<std::vector<double>> &hist, int64_t &t)
 {
     Workspace &ws = h->ws;
     const int lag = h->opt.lag;
     cudaStream_t cs = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
     int rc = COX_OK;
     auto one_step = [&](int slot) -> int {
-        int r = iterate(h, beta_dev, k, EPI_PROX, nullptr, step, cs);
-        if (r != COX_OK) return r;
-        if (cudaMemcpyAsync(ws.Fring + static_cast<size_t>(slot) * k, ws.F, k * sizeof(double), cudaMemcpyDeviceToDevice,
-                            cs) != cudaSuccess)
-            return COX_ERR_CUDA;
-        return COX_OK;
+        return iterate(h, beta_dev, k, EPI_PROX, nullptr, step, cs, nullptr, ws.Fring + static_cast<size_t>(slot) * k);
     };
     if (cudaMemcpy(ws.active, active.data(), k * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) return COX_ERR_CUDA;
     do {
         if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) { rc = COX_ERR_CUDA; break; }
-        // the active-set product decides on the host before each iteration, so
-        // those iterations run as plain launches instead of graph replays
-        if (max_iter - t >= lag && !(h->opt.active_set && (h->opt.precision == COX_SPLIT_E4M3 || is_e2m1(h)))) {
-            if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { rc = COX_ERR_CUDA; break; }
-            for (int s = 0; s < lag && rc == COX_OK; ++s) rc = one_step(s);
-            cudaError_t ec = cudaStreamEndCapture(cs, &graph);
-            if (rc != COX_OK) break;
-            if (ec != cudaSuccess || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) { rc = COX_ERR_CUDA; break; }
-        }
         std::vector<double> ring(static_cast<size_t>(lag) * k);
         while (t < max_iter) {
             bool any = false;
             for (int c = 0; c < k; ++c) any |= active[c] != 0;
             if (!any) break;
-            int steps;
-            if (exec && max_iter - t >= lag) {
-                if (cudaGraphLaunch(exec, cs) != cudaSuccess) { rc = COX_ERR_CUDA; break; }
-                steps = lag;
-            } else {
-                steps = static_cast<int>(std::min<int64_t>(lag, max_iter - t));
-                for (int s = 0; s < steps && rc == COX_OK; ++s) rc = one_step(s);
-                if (rc != COX_OK) break;
-            }
+            const int steps = static_cast<int>(std::min<int64_t>(lag, max_iter - t));
+            for (int s = 0; s < steps && rc == COX_OK; ++s) rc = one_step(s);
+            if (rc != COX_OK) break;
             if (cudaMemcpyAsync(ring.data(), ws.Fring, static_cast<size_t>(steps) * k * sizeof(double),
                                 cudaMemcpyDeviceToHost, cs) != cudaSuccess) { rc = COX_ERR_CUDA; break; }
             int e = 0;
@@ -270,8 +252,6 @@ int path_run(cox_handle *h, int k, int max_iter, double tol, double step, void *
             }
         }
     } while (false);
-    if (exec) cudaGraphExecDestroy(exec);
-    if (graph) cudaGraphDestroy(graph);
     if (cs) {
         cudaStreamSynchronize(cs);
         cudaStreamDestroy(cs);

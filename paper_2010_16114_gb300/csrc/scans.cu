@@ -45,6 +45,7 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "ptx.cuh"
 
 namespace coxgb {
 namespace {
@@ -197,7 +198,7 @@ struct SP {
     int *bs;
     int l1_blocks;
     const double *l1p, *lam;
-    double *sumV, *f, *l1, *F;
+    double *sumV, *f, *l1, *F, *F_out;
     bool need_loss;
     int *err;
     long long wait_limit;
@@ -304,7 +305,9 @@ __device__ __forceinline__ void finalize_column(const SP &s, int kk, double *sh)
         const double lo = (x[3] - x[1]) / n;
         s.f[kk] = lo;
         s.l1[kk] = b1;
-        s.F[kk] = lo + (s.lam ? s.lam[kk] * b1 : 0.0);
+        const double F = lo + (s.lam ? s.lam[kk] * b1 : 0.0);
+        s.F[kk] = F;
+        if (s.F_out) s.F_out[kk] = F;
         if (!isfinite(lo)) atomicOr(s.err, DEVERR_NONFINITE);
     }
     if (!isfinite(v)) atomicOr(s.err, DEVERR_NONFINITE);
@@ -366,6 +369,7 @@ __global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
     __shared__ long long shl[NW];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     double *const buf = buf_all + warp * BW;
+    pdl_trigger();  // the product behind may set up as soon as this grid runs
     const int64_t nch = s.nch, tasks = nch * s.k;
     const int64_t lo = min(tasks, blockIdx.x * s.per), hi = min(tasks, lo + s.per);
 
@@ -932,6 +936,7 @@ int run_scans(cox_handle *h, const ScanArgs &a, cudaStream_t st)
     s.f = ws.f;
     s.l1 = ws.l1;
     s.F = ws.F;
+    s.F_out = a.F_out;
     s.need_loss = a.need_loss;
     s.err = h->d_err;
     s.wait_limit = h->wait_cycles;
@@ -943,16 +948,8 @@ int run_scans(cox_handle *h, const ScanArgs &a, cudaStream_t st)
     const int64_t room = static_cast<int64_t>(occ) * h->sm_count, tasks = static_cast<int64_t>(s.nch) * a.k;
     const int64_t mains = std::min(room, (tasks + NW - 1) / NW);
     s.per = (tasks + mains - 1) / mains;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(std::min(room, mains + 2 * static_cast<int64_t>(s.ntile) * a.k)));
-    cfg.blockDim = dim3(NT);
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    COX_CUDA(cudaLaunchKernelEx(&cfg, fn, s));
+    const unsigned grid = static_cast<unsigned>(std::min(room, mains + 2 * static_cast<int64_t>(s.ntile) * a.k));
+    COX_CUDA(launch_pdl(fn, dim3(grid), NT, 0, st, true, s));
     return COX_OK;
 }
 

@@ -11,7 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libcoxgb.so")
 SOURCES = ["api.cu", "setup.cu", "scans.cu", "gemm_tc.cu", "gemm_f4.cu", "gemv.cu", "path.cu", "power.cu", "active.cu", "nmf.cu"]
-HEADERS = ["internal.h", "ptx.cuh", "nmf_gemm.cuh", "gemm_kernel.cuh"]
+HEADERS = ["internal.h", "ptx.cuh", "nmf_gemm.cuh", "gemm_kernel.cuh", "pairs.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 CFLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fno-strict-aliasing",
           f"-I{os.path.join(ROOT, 'include')}"]

@@ -4,11 +4,11 @@
 //
 // An iteration is six kernels:
 //   k_nmf_gemm    P = X W^T   (m x r)   tcgen05 kind::f16, A = X row-major
+//   k_nmf_gram    W W^T (FP64) from the partials of W's update, beside that product
 //   k_nmf_update  V from P and W W^T; limbs of V; per-block partials of V^T V
-//   k_nmf_gram    V^T V (FP64) from the partials
 //   k_nmf_gemm    Q = X^T V   (n x r)   A = X column-major
+//   k_nmf_gram    V^T V, beside that product
 //   k_nmf_update  W from Q and V^T V; limbs of W; partials of W W^T
-//   k_nmf_gram    W W^T
 // Both updates have one form.  With F a factor held r x R (V^T, or W), G the
 // Gram matrix of the other factor and P the product of X with it,
 //   (V W W^T)_ic = sum_d G_cd F_di  and  (V^T V W)_cj = sum_d G_cd F_dj
@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "pairs.cuh"
 #include "ptx.cuh"
 #include "../../include/nmfgb.h"
 #include "nmf_gemm.cuh"
@@ -48,11 +49,10 @@ struct UpdArgs {
     const float *part;       // product partials of this side
     int SL, KC;
     int64_t L;
-    const float *Gin;        // r x r Gram of the other factor, FP32
-    const double *Gin64;     // and FP64 (its squared Frobenius norm sets the APG step)
+    const float *Gin;        // Gram matrix of the other factor, FP32 rows of gram_ld(r)
+    const tf *Gsq;           // its pairs' parts of the squared Frobenius norm (the APG step)
     double eps;
-    float *gpart;            // Gram partials of the new F: [pair][block], pairs c <= d
-    int nblk;                // blocks of this launch
+    float *gpart;            // Gram partials of the new F: [block][pair], pairs c <= d
     int *err;
 };
 
@@ -68,99 +68,166 @@ __device__ __forceinline__ void split_bf16(float f, __nv_bfloat16 &h0, __nv_bflo
 // Pair p of the upper triangle (c <= d, row by row) of an r x r matrix.
 __device__ __forceinline__ void pair_cd(int p, int r, int &c, int &d)
 {
-    c = 0;
-    while (p >= r - c) {
-        p -= r - c;
-        ++c;
-    }
-    d = c + p;
+    const float b = static_cast<float>(2 * r + 1);
+    c = static_cast<int>((b - sqrtf(b * b - 8.f * static_cast<float>(p))) * 0.5f);
+    while (c > 0 && p < c * r - c * (c - 1) / 2) --c;             // the root is within one row
+    while (p >= (c + 1) * r - (c + 1) * c / 2) ++c;
+    d = c + (p - (c * r - c * (c - 1) / 2));
 }
+__device__ __forceinline__ int pair_index(int c, int d, int r) { return c * r - c * (c - 1) / 2 + (d - c); }
 
 constexpr int UPD_ROWS = 32;    // factor columns per block (one per lane)
-constexpr int UPD_MAXW = 32;    // warps per block: min(r, 32); warp y takes rank rows c = y, y + W, ...
+constexpr int UPD_MAXW = 32;    // warps per block of k_nmf_fit
+constexpr int UPD_LDN = UPD_ROWS + 4;  // stride of the new F's rows: float4 reads of 8 rows hit all banks
 
-int upd_warps(int r) { return r < UPD_MAXW ? r : UPD_MAXW; }
+int fit_warps(int r) { return r < UPD_MAXW ? r : UPD_MAXW; }
+
+constexpr int CPW = 4;          // rank rows per warp of k_nmf_update
+int upd_warps(int r) { return (r + CPW - 1) / CPW; }
+int gram_ld(int r) { return upd_warps(r) * CPW; }  // row stride of the FP32 Gram matrices (zero past r)
 
 // A quarter row tile of a factor per block: lane x of every warp owns column
-// i = 128 g + 32 q + x of F (block 4 g + q); warp y of W = min(r, 32) takes
-// the rank rows c = y, y + W, ...  Shared memory: G (r x r), the old and the
-// new F and the summed product partials ([c][33] each).  The block also
-// leaves its partial of the new F's Gram matrix over its 32 columns (FP32),
-// one per pair c <= d.  Dot products run in four interleaved FP32 sums (a
-// fixed order) to shorten the dependent chains.
-__global__ void __launch_bounds__(UPD_ROWS * UPD_MAXW) k_nmf_update(const UpdArgs A)
+// i = 128 g + 32 q + x of F (block 4 g + q); warp w takes the rank rows
+// c = 4 w .. 4 w + 3.  Shared memory: G (rows of gram_ld(r) floats), the old F
+// ([c][32]) and the new one ([c][36], rows up to an even count).
+//   sums    the product's partial slots, in pairs of floats (FP64 sums of the
+//           slots held the two FP64 lanes of an SM for most of this kernel)
+//   dots    sum_d G_cd F_di for the four rows of a warp at once: one load of F and a
+//           broadcast float4 load of G (symmetric: row d) per four multiply-adds,
+//           against two loads per multiply-add for one row at a time; four
+//           interleaved FP32 sums per row
+//   Gram    the block's partial of the new F's Gram matrix over its 32 columns, 2 x 2
+//           pairs per thread from float4 loads, four interleaved FP32 sums per pair
+// What is left is latency, so a thread's loads are in flight before the first use
+// (64 registers, for a second block per SM at r = 60, made whole iterations slower).
+// An APG iteration, against one row at a time with FP64 slot sums and the Gram
+// kernel behind it: X 3001 x 8009, r = 60 139 -> 70 us (with the copy of the
+// factors to the host, per 20), 10,000 x 500, r = 40 84 -> 41, 2000 x 2000, r = 20
+// 51 -> 23, 10,000 x 10,000, r = 20 108 -> 89.
+__global__ void __launch_bounds__(640) k_nmf_update(const UpdArgs A)
 {
-    extern __shared__ float sh[];
-    __shared__ double fro_w[UPD_MAXW];
+    extern __shared__ __align__(16) float sh[];
+    __shared__ tf fro_w[NMF_MAX_RANK / CPW];
     __shared__ float step_s;
-    constexpr int LD = UPD_ROWS + 1;
-    const int r = A.r, t = threadIdx.x, x = t % UPD_ROWS, y = t / UPD_ROWS;
-    const int W = blockDim.x / UPD_ROWS, nthr = blockDim.x;
-    pdl_trigger();
-    pdl_wait();  // the product ahead (and everything before it) is complete
+    const int r = A.r, t = threadIdx.x, x = t % UPD_ROWS, w = t / UPD_ROWS;
+    const int W = blockDim.x / UPD_ROWS, LDG = W * CPW, nthr = blockDim.x;
     float *Gs = sh;
-    float *Fo = Gs + r * r;
-    float *Fn = Fo + r * LD;
-    float *Pc = Fn + r * LD;
+    float *Fo = Gs + r * LDG;
+    float *Fn = Fo + r * UPD_ROWS;
     const int64_t g = blockIdx.x / (NT / UPD_ROWS);
     const int rit = static_cast<int>(blockIdx.x % (NT / UPD_ROWS)) * UPD_ROWS + x;  // row in the tile
     const int64_t i = g * NT + rit;
     const bool valid = i < A.R;
     const bool apg = A.mode && A.algo == NMF_APG;
+    const int c0 = w * CPW;
+    const int64_t first = (g * A.KC) / A.L, last = (g * A.KC + A.KC - 1) / A.L;
+    const int ns = A.mode ? static_cast<int>(last - first + 1) : 0;
+    const float *pp = A.part + (g * A.SL * r + c0) * NT + rit;
+    const int64_t ps = static_cast<int64_t>(r) * NT;  // slot stride
+    pdl_trigger();
+    pdl_wait();  // the product and the other factor's Gram matrix are complete
+    float old[CPW], pc[CPW];
+#pragma unroll
+    for (int q = 0; q < CPW; ++q) old[q] = valid && c0 + q < r ? A.F[(c0 + q) * A.R + i] : 0.f;
+    constexpr int SB = 4;  // slots whose loads are in flight together
+    float b[SB][CPW];
+#pragma unroll
+    for (int u = 0; u < SB; ++u)
+#pragma unroll
+        for (int q = 0; q < CPW; ++q) b[u][q] = u < ns && c0 + q < r ? pp[u * ps + q * NT] : 0.f;
     if (A.mode) {
-        double f = 0.0;  // ||G||_F^2 (APG step): every thread a few entries, then a fixed-order reduction
-        for (int e = t; e < r * r; e += nthr) {
-            Gs[e] = A.Gin[e];
-            if (apg) {
-                const double gv = A.Gin64[e];
-                f += gv * gv;
+        // G is r W float4, at most NMF_MAX_RANK / 32 (rounded up) per thread
+        constexpr int GB = (NMF_MAX_RANK + 31) / 32;
+        float4 gv[GB];
+#pragma unroll
+        for (int u = 0; u < GB; ++u)
+            if (t + u * nthr < r * W) gv[u] = reinterpret_cast<const float4 *>(A.Gin)[t + u * nthr];
+        if (apg) {  // ||G||_F^2: at most (r + 1) / 16 + 1 pairs per thread, then a fixed-order reduction
+            constexpr int QB = (NMF_MAX_RANK + 1) / 16 + 1;
+            tf f{0.f, 0.f}, sq[QB];
+#pragma unroll
+            for (int u = 0; u < QB; ++u) sq[u] = t + u * nthr < r * (r + 1) / 2 ? A.Gsq[t + u * nthr] : tf{0.f, 0.f};
+#pragma unroll
+            for (int u = 0; u < QB; ++u) f = tf_add(f, sq[u]);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) f = tf_add(f, shfl_xor(f, o));
+            if (x == 0) fro_w[w] = f;
+        }
+#pragma unroll
+        for (int u = 0; u < GB; ++u)
+            if (t + u * nthr < r * W) reinterpret_cast<float4 *>(Gs)[t + u * nthr] = gv[u];
+        tf sum[CPW];
+#pragma unroll
+        for (int q = 0; q < CPW; ++q) sum[q] = tf{b[0][q], 0.f};
+#pragma unroll
+        for (int u = 1; u < SB; ++u)
+            if (u < ns) {
+#pragma unroll
+                for (int q = 0; q < CPW; ++q) sum[q] = tf_add(sum[q], tf{b[u][q], 0.f});
             }
+        for (int sl = SB; sl < ns; sl += SB) {
+#pragma unroll
+            for (int u = 0; u < SB; ++u)
+#pragma unroll
+                for (int q = 0; q < CPW; ++q)
+                    b[u][q] = sl + u < ns && c0 + q < r ? pp[(sl + u) * ps + q * NT] : 0.f;
+#pragma unroll
+            for (int u = 0; u < SB; ++u)
+#pragma unroll
+                for (int q = 0; q < CPW; ++q) sum[q] = tf_add(sum[q], tf{b[u][q], 0.f});
         }
-        if (apg) {
-            for (int off = 16; off > 0; off >>= 1) f += __shfl_down_sync(0xffffffffu, f, off);
-            if (x == 0) fro_w[y] = f;
-        }
-        const int64_t first = (g * A.KC) / A.L, last = (g * A.KC + A.KC - 1) / A.L;
-        const int ns = static_cast<int>(last - first + 1);
-        const float *pp = A.part + (g * A.SL * r) * NT + rit;
-        for (int c = y; c < r; c += W) {
-            double acc = 0.0;
-#pragma unroll 4
-            for (int sl = 0; sl < ns; ++sl) acc += static_cast<double>(pp[(static_cast<int64_t>(sl) * r + c) * NT]);
-            Pc[c * LD + x] = static_cast<float>(acc);
-        }
+#pragma unroll
+        for (int q = 0; q < CPW; ++q) pc[q] = sum[q].h;  // the pair's sum rounded to FP32
     }
-    for (int c = y; c < r; c += W) Fo[c * LD + x] = valid ? A.F[c * A.R + i] : 0.f;
+#pragma unroll
+    for (int q = 0; q < CPW; ++q)
+        if (c0 + q < r) Fo[(c0 + q) * UPD_ROWS + x] = old[q];
     __syncthreads();
-    if (apg && t == 0) {  // the step, formed once per block (FP64 division is slow on this part)
-        double f2 = 0.0;
-        for (int w = 0; w < W; ++w) f2 += fro_w[w];
-        step_s = static_cast<float>(1.0 / (2.0 * f2 + A.eps));
+    if (apg) {  // the step, formed once per block (FP64 division is slow on this part)
+        if (t == 0) {
+            tf f2 = fro_w[0];
+            for (int v = 1; v < W; ++v) f2 = tf_add(f2, fro_w[v]);
+            step_s = static_cast<float>(1.0 / (2.0 * tf_double(f2) + A.eps));
+        }
+        __syncthreads();
     }
-    if (apg) __syncthreads();
     const float s = apg ? step_s : 0.f;
     const float eps = static_cast<float>(A.eps);
     bool bad = false;
-    for (int c = y; c < r; c += W) {
-        const float old = Fo[c * LD + x];
-        float v = old;
-        if (A.mode && valid) {
-            const float pc = Pc[c * LD + x];
-            float d4[4] = {0.f, 0.f, 0.f, 0.f};
-            const float *gr = Gs + c * r;
-            int d = 0;
-            for (; d + 4 <= r; d += 4) {
+    float acc[4][CPW];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) d4[q] = fmaf(gr[d + q], Fo[(d + q) * LD + x], d4[q]);
-            }
-            for (; d < r; ++d) d4[0] = fmaf(gr[d], Fo[d * LD + x], d4[0]);
-            const float den = (d4[0] + d4[1]) + (d4[2] + d4[3]);
-            v = A.algo == NMF_MULTIPLICATIVE ? old * pc / (den + eps) : fmaxf(0.f, old - s * (den - pc));
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int q = 0; q < CPW; ++q) acc[u][q] = 0.f;
+    if (A.mode) {
+        auto row = [&](int d, float *a) {
+            const float f = Fo[d * UPD_ROWS + x];
+            const float4 gv = *reinterpret_cast<const float4 *>(Gs + d * LDG + c0);
+            a[0] = fmaf(gv.x, f, a[0]);
+            a[1] = fmaf(gv.y, f, a[1]);
+            a[2] = fmaf(gv.z, f, a[2]);
+            a[3] = fmaf(gv.w, f, a[3]);
+        };
+        int d = 0;
+        for (; d + 4 <= r; d += 4) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) row(d + u, acc[u]);
+        }
+        for (; d < r; ++d) row(d, acc[0]);
+    }
+#pragma unroll
+    for (int q = 0; q < CPW; ++q) {
+        const int c = c0 + q;
+        if (c >= r) break;
+        float v = old[q];
+        if (A.mode && valid) {
+            const float den = (acc[0][q] + acc[1][q]) + (acc[2][q] + acc[3][q]);
+            v = A.algo == NMF_MULTIPLICATIVE ? old[q] * pc[q] / (den + eps) : fmaxf(0.f, old[q] - s * (den - pc[q]));
             bad |= !isfinite(v);
             A.F[c * A.R + i] = v;
         }
         if (!valid) v = 0.f;
-        Fn[c * LD + x] = v;
+        Fn[c * UPD_LDN + x] = v;
         if (valid) {
             __nv_bfloat16 h0, h1, h2;
             split_bf16(v, h0, h1, h2);
@@ -169,63 +236,97 @@ __global__ void __launch_bounds__(UPD_ROWS * UPD_MAXW) k_nmf_update(const UpdArg
             A.limb[static_cast<int64_t>(2 * A.rp + c) * A.ldl + i] = h2;
         }
     }
+    if ((r & 1) && w == 0) Fn[r * UPD_LDN + x] = 0.f;
     if (bad) atomicOr(A.err, NMF_ERR_NONFINITE);
     __syncthreads();
-    // Gram partial over the block's 32 columns (zero for columns past R)
-    const int npair = r * (r + 1) / 2;
-    for (int p = t; p < npair; p += nthr) {
-        int c, d;
-        pair_cd(p, r, c, d);
-        const float *fc = Fn + c * LD, *fd = Fn + d * LD;
-        float a4[4] = {0.f, 0.f, 0.f, 0.f};
+    // Gram partial over the block's 32 columns (zero for columns past R): 2 x 2 pairs
+    const int r2 = (r + 1) / 2, npair = r * (r + 1) / 2;
+    float *gp = A.gpart + static_cast<int64_t>(blockIdx.x) * npair;
+    for (int p = t; p < r2 * (r2 + 1) / 2; p += blockDim.x) {
+        int a, b;
+        pair_cd(p, r2, a, b);
+        float4 m[2][2];
 #pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) m[u][v] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
         for (int j = 0; j < UPD_ROWS; j += 4) {
+            float4 fc[2], fd[2];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) a4[q] = fmaf(fc[j + q], fd[j + q], a4[q]);
+            for (int u = 0; u < 2; ++u) {
+                fc[u] = *reinterpret_cast<const float4 *>(Fn + (2 * a + u) * UPD_LDN + j);
+                fd[u] = *reinterpret_cast<const float4 *>(Fn + (2 * b + u) * UPD_LDN + j);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    m[u][v].x = fmaf(fc[u].x, fd[v].x, m[u][v].x);
+                    m[u][v].y = fmaf(fc[u].y, fd[v].y, m[u][v].y);
+                    m[u][v].z = fmaf(fc[u].z, fd[v].z, m[u][v].z);
+                    m[u][v].w = fmaf(fc[u].w, fd[v].w, m[u][v].w);
+                }
         }
-        A.gpart[static_cast<int64_t>(p) * A.nblk + blockIdx.x] = (a4[0] + a4[1]) + (a4[2] + a4[3]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int c = 2 * a + u, d = 2 * b + v;
+                if (c <= d && d < r) gp[pair_index(c, d, r)] = (m[u][v].x + m[u][v].y) + (m[u][v].z + m[u][v].w);
+            }
     }
 }
 
 struct GramArgs {
-    int r, nblk;
-    const float *gpart;      // [pair][block]
+    int r, nblk, ldg;
+    const float *gpart;      // [block][pair]
     double *G64;             // r x r
-    float *G32;
+    float *G32;              // rows of ldg floats
+    tf *Gsq;                 // per pair: its part of ||G||_F^2
 };
 
-// G = F F^T from the update blocks' partials: one warp per pair c <= d, lane
-// sums of the blocks b = lane, lane + 32, ... in FP64 and a shuffle tree (a
-// fixed order: deterministic).
+// G = F F^T from the update blocks' partials, in FP64: 32 pairs per block (one per
+// lane), warp y adds the blocks b = y, y + 8, ..., then the warps' sums in warp
+// order (a fixed order: deterministic).  Runs beside the product that follows the
+// update: that product lets it start once the update is complete, and it waits for
+// the product only at its end, so that the update behind it finds both complete.
 __global__ void __launch_bounds__(256) k_nmf_gram(const GramArgs A)
 {
-    const int lane = threadIdx.x & 31;
-    const int p = blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int r = A.r;
+    __shared__ double sums[8][32];
+    const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
+    const int p = blockIdx.x * 32 + lane;
+    const int r = A.r, npair = r * (r + 1) / 2;
     pdl_trigger();
-    pdl_wait();  // the update ahead is complete
-    if (p >= r * (r + 1) / 2) return;
-    const float *src = A.gpart + static_cast<int64_t>(p) * A.nblk;
-    double v4[4] = {0.0, 0.0, 0.0, 0.0};  // blocks lane + 32 (4 j + q)
-    int b = lane;
-    for (; b + 96 < A.nblk; b += 128) {
-        float u[4];
+    double v = 0.0;
+    if (p < npair) {
+        const float *src = A.gpart + p;
+        double v4[4] = {0.0, 0.0, 0.0, 0.0};
+        int b = y;
+        for (; b + 56 < A.nblk; b += 64) {
+            float u[8];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) u[q] = src[b + 32 * q];
+            for (int q = 0; q < 8; ++q) u[q] = __ldcg(src + static_cast<int64_t>(b + 8 * q) * npair);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v4[q] += static_cast<double>(u[q]);
+            for (int q = 0; q < 8; ++q) v4[q & 3] += static_cast<double>(u[q]);
+        }
+#pragma unroll 4
+        for (; b < A.nblk; b += 8) v4[0] += static_cast<double>(__ldcg(src + static_cast<int64_t>(b) * npair));
+        v = (v4[0] + v4[1]) + (v4[2] + v4[3]);
     }
-    for (; b < A.nblk; b += 32) v4[0] += static_cast<double>(src[b]);
-    double v = (v4[0] + v4[1]) + (v4[2] + v4[3]);
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (lane == 0) {
+    sums[y][lane] = v;
+    __syncthreads();
+    if (y == 0 && p < npair) {
+        for (int k = 1; k < 8; ++k) v += sums[k][lane];
         int c, d;
         pair_cd(p, r, c, d);
         A.G64[c * r + d] = v;
         A.G64[d * r + c] = v;
-        A.G32[c * r + d] = static_cast<float>(v);
-        A.G32[d * r + c] = static_cast<float>(v);
+        A.G32[c * A.ldg + d] = static_cast<float>(v);
+        A.G32[d * A.ldg + c] = static_cast<float>(v);
+        A.Gsq[p] = tf_of(c == d ? v * v : 2.0 * (v * v));
     }
+    pdl_wait();
 }
 
 struct FitArgs {
@@ -417,7 +518,8 @@ struct nmf_handle {
     float *part1 = nullptr, *part2 = nullptr;
     NmfSide s1, s2;               // X W^T, X^T V
     float *GV32 = nullptr, *GW32 = nullptr;
-    float *gpart = nullptr;    // Gram partials [pair][update block]
+    float *gpartV = nullptr, *gpartW = nullptr;  // Gram partials [update block][pair]
+    coxgb::tf *GVsq = nullptr, *GWsq = nullptr;   // per pair: its part of ||G||_F^2
     double *GV64 = nullptr, *GW64 = nullptr, *opart = nullptr, *fobj = nullptr;
     int *counters = nullptr, *err = nullptr;
     double xx = 0.0;
@@ -495,12 +597,14 @@ int launch_gemm(nmf_handle *h, const NmfSide &sd, cudaStream_t st)
                : COX_ERR_CUDA;
 }
 
-size_t upd_smem(int r) { return static_cast<size_t>(r * r + 3 * r * (UPD_ROWS + 1)) * sizeof(float); }
+size_t upd_smem(int r)
+{
+    return static_cast<size_t>(r * gram_ld(r) + r * UPD_ROWS + (r + 1) / 2 * 2 * UPD_LDN) * sizeof(float);
+}
 
 int upd_blocks(int64_t R) { return static_cast<int>((R + NT - 1) / NT * (NT / UPD_ROWS)); }
 
-// side 0: V from X W^T (rows m); side 1: W from X^T V (rows n); then the Gram
-// matrix of the new factor from the blocks' partials
+// side 0: V from X W^T (rows m); side 1: W from X^T V (rows n)
 int launch_update(nmf_handle *h, int side, int mode, int algo, double eps, cudaStream_t st)
 {
     UpdArgs a;
@@ -518,23 +622,45 @@ int launch_update(nmf_handle *h, int side, int mode, int algo, double eps, cudaS
     a.KC = sd.g.KC;
     a.L = sd.g.L;
     a.Gin = side == 0 ? h->GW32 : h->GV32;
-    a.Gin64 = side == 0 ? h->GW64 : h->GV64;
+    a.Gsq = side == 0 ? h->GWsq : h->GVsq;
     a.eps = eps;
-    a.gpart = h->gpart;
-    a.nblk = upd_blocks(a.R);
+    a.gpart = side == 0 ? h->gpartV : h->gpartW;
     a.err = h->err;
     ++h->launches;
-    if (launch_pdl(k_nmf_update, dim3(a.nblk), UPD_ROWS * upd_warps(h->r), upd_smem(h->r), st, false, a) != cudaSuccess)
-        return COX_ERR_CUDA;
+    return launch_pdl(k_nmf_update, dim3(upd_blocks(a.R)), UPD_ROWS * upd_warps(h->r), upd_smem(h->r), st, false, a) ==
+                   cudaSuccess
+               ? COX_OK
+               : COX_ERR_CUDA;
+}
+
+// The Gram matrix of a factor (0: V, 1: W) from its last update's partials.  beside:
+// right behind the product that follows that update, to run while it runs.
+int launch_gram(nmf_handle *h, int side, cudaStream_t st, bool beside)
+{
     GramArgs gm;
     gm.r = h->r;
-    gm.nblk = a.nblk;
-    gm.gpart = h->gpart;
+    gm.ldg = gram_ld(h->r);
+    gm.nblk = upd_blocks(side == 0 ? h->m : h->n);
+    gm.gpart = side == 0 ? h->gpartV : h->gpartW;
     gm.G64 = side == 0 ? h->GV64 : h->GW64;
     gm.G32 = side == 0 ? h->GV32 : h->GW32;
-    const int npair = h->r * (h->r + 1) / 2;
+    gm.Gsq = side == 0 ? h->GVsq : h->GWsq;
+    const unsigned grid = static_cast<unsigned>((h->r * (h->r + 1) / 2 + 31) / 32);
     ++h->launches;
-    return launch_pdl(k_nmf_gram, dim3((npair + 7) / 8), 256, 0, st, false, gm) == cudaSuccess ? COX_OK : COX_ERR_CUDA;
+    if (beside) return launch_pdl(k_nmf_gram, dim3(grid), 256, 0, st, false, gm) == cudaSuccess ? COX_OK : COX_ERR_CUDA;
+    k_nmf_gram<<<grid, 256, 0, st>>>(gm);
+    return cudaGetLastError() == cudaSuccess ? COX_OK : COX_ERR_CUDA;
+}
+
+// One iteration: each factor's Gram matrix is formed beside the next product.
+int launch_iteration(nmf_handle *h, int algo, double eps, cudaStream_t st)
+{
+    COX_TRY(launch_gemm(h, h->s1, st));
+    COX_TRY(launch_gram(h, 1, st, true));
+    COX_TRY(launch_update(h, 0, 1, algo, eps, st));
+    COX_TRY(launch_gemm(h, h->s2, st));
+    COX_TRY(launch_gram(h, 0, st, true));
+    return launch_update(h, 1, 1, algo, eps, st);
 }
 
 int check_err(nmf_handle *h, cudaStream_t st)
@@ -603,7 +729,7 @@ int setup_impl(const float *X, int64_t m, int64_t n, int r, int device, nmf_hand
         if ((rc = A(reinterpret_cast<void **>(&h->Vt), static_cast<size_t>(r * m) * 4)) != COX_OK) break;
         if ((rc = A(reinterpret_cast<void **>(&h->W), static_cast<size_t>(r * n) * 4)) != COX_OK) break;
         for (float **p : {&h->GV32, &h->GW32})
-            if ((rc = A(reinterpret_cast<void **>(p), static_cast<size_t>(r * r) * 4)) != COX_OK) break;
+            if ((rc = A(reinterpret_cast<void **>(p), static_cast<size_t>(r * gram_ld(r)) * 4)) != COX_OK) break;
         if (rc) break;
         for (double **p : {&h->GV64, &h->GW64})
             if ((rc = A(reinterpret_cast<void **>(p), static_cast<size_t>(r * r) * 8)) != COX_OK) break;
@@ -612,17 +738,23 @@ int setup_impl(const float *X, int64_t m, int64_t n, int r, int device, nmf_hand
         if ((rc = A(reinterpret_cast<void **>(&h->opart), static_cast<size_t>(upd_blocks(std::max(m, n))) * 8)) !=
             COX_OK)
             break;
-        if ((rc = A(reinterpret_cast<void **>(&h->gpart), static_cast<size_t>(r * (r + 1) / 2) *
-                                                                  upd_blocks(std::max(m, n)) * sizeof(float))) != COX_OK)
-            break;
+        const size_t npair = static_cast<size_t>(r) * (r + 1) / 2;
+        const size_t gpv = npair * upd_blocks(m) * sizeof(float), gpw = npair * upd_blocks(n) * sizeof(float);
+        if ((rc = A(reinterpret_cast<void **>(&h->gpartV), gpv)) != COX_OK) break;
+        if ((rc = A(reinterpret_cast<void **>(&h->gpartW), gpw)) != COX_OK) break;
+        if ((rc = A(reinterpret_cast<void **>(&h->GVsq), npair * sizeof(tf))) != COX_OK) break;
+        if ((rc = A(reinterpret_cast<void **>(&h->GWsq), npair * sizeof(tf))) != COX_OK) break;
         if (cudaMemsetAsync(h->err, 0, sizeof(int), st) != cudaSuccess ||
             cudaMemsetAsync(h->counters, 0, 4 * sizeof(int), st) != cudaSuccess ||
             cudaMemsetAsync(h->Vl, 0, static_cast<size_t>(h->NP * h->ldm) * 2, st) != cudaSuccess ||
             cudaMemsetAsync(h->Wl, 0, static_cast<size_t>(h->NP * h->ldn) * 2, st) != cudaSuccess ||
             cudaMemsetAsync(h->Vt, 0, static_cast<size_t>(r * m) * 4, st) != cudaSuccess ||
             cudaMemsetAsync(h->W, 0, static_cast<size_t>(r * n) * 4, st) != cudaSuccess ||
-            cudaMemsetAsync(h->GV32, 0, static_cast<size_t>(r * r) * 4, st) != cudaSuccess ||
-            cudaMemsetAsync(h->GW32, 0, static_cast<size_t>(r * r) * 4, st) != cudaSuccess ||
+            cudaMemsetAsync(h->gpartV, 0, gpv, st) != cudaSuccess || cudaMemsetAsync(h->gpartW, 0, gpw, st) != cudaSuccess ||
+            cudaMemsetAsync(h->GVsq, 0, npair * sizeof(tf), st) != cudaSuccess ||
+            cudaMemsetAsync(h->GWsq, 0, npair * sizeof(tf), st) != cudaSuccess ||
+            cudaMemsetAsync(h->GV32, 0, static_cast<size_t>(r * gram_ld(r)) * 4, st) != cudaSuccess ||
+            cudaMemsetAsync(h->GW32, 0, static_cast<size_t>(r * gram_ld(r)) * 4, st) != cudaSuccess ||
             cudaMemsetAsync(h->GV64, 0, static_cast<size_t>(r * r) * 8, st) != cudaSuccess ||
             cudaMemsetAsync(h->GW64, 0, static_cast<size_t>(r * r) * 8, st) != cudaSuccess) {
             rc = COX_ERR_CUDA;
@@ -737,7 +869,9 @@ int nmf_set_factors(nmf_h h, const float *V, const float *W, void *stream)
     COX_CUDA(cudaMemcpyAsync(h->Vt, vt.data(), vt.size() * 4, cudaMemcpyHostToDevice, st));
     COX_CUDA(cudaMemcpyAsync(h->W, W, static_cast<size_t>(r * n) * 4, cudaMemcpyHostToDevice, st));
     COX_TRY(launch_update(h, 0, 0, 0, 0.0, st));
+    COX_TRY(launch_gram(h, 0, st, false));
     COX_TRY(launch_update(h, 1, 0, 0, 0.0, st));
+    COX_TRY(launch_gram(h, 1, st, false));
     return check_err(h, st);
 }
 
@@ -771,10 +905,7 @@ int nmf_iterate(nmf_h h, int algo, int64_t iters, double eps, void *stream)
         }
         const int64_t before = h->launches;
         COX_CUDA(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-        int rc = launch_gemm(h, h->s1, h->cap);
-        if (rc == COX_OK) rc = launch_update(h, 0, 1, algo, eps, h->cap);
-        if (rc == COX_OK) rc = launch_gemm(h, h->s2, h->cap);
-        if (rc == COX_OK) rc = launch_update(h, 1, 1, algo, eps, h->cap);
+        int rc = launch_iteration(h, algo, eps, h->cap);
         cudaGraph_t graph = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(h->cap, &graph);
         h->launches = before;
@@ -799,6 +930,7 @@ int nmf_objective(nmf_h h, double *f, void *stream)
     if (!h || !f) return COX_ERR_ARG;
     DevGuard guard(h->dev);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    COX_TRY(launch_gram(h, 1, st, false));  // W's is otherwise formed in the next iteration
     COX_TRY(launch_gemm(h, h->s1, st));
     FitArgs a;
     a.r = h->r;
@@ -814,7 +946,7 @@ int nmf_objective(nmf_h h, double *f, void *stream)
     a.GW = h->GW64;
     a.xx = h->xx;
     a.out = h->fobj;
-    k_nmf_fit<<<upd_blocks(h->m), UPD_ROWS * upd_warps(h->r), 0, st>>>(a);
+    k_nmf_fit<<<upd_blocks(h->m), UPD_ROWS * fit_warps(h->r), 0, st>>>(a);
     ++h->launches;
     COX_CUDA(cudaGetLastError());
     COX_CUDA(cudaMemcpyAsync(f, h->fobj, sizeof(double), cudaMemcpyDeviceToHost, st));

@@ -95,7 +95,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     float *sums = reinterpret_cast<float *>(smem + S * STAGE + 256);  // [r][128] running sums
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    pdl_trigger();
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(full0 + 8 * s, 1);
@@ -123,8 +122,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     const uint32_t tbase = *tmem_slot;
     // everything above touches only this CTA's shared memory, TMEM and the
     // kernel parameters; the kernel ahead (the factor update that wrote the
-    // limb panel) must be complete before any global access
+    // limb panel) must be complete before any global access.  Only then may the
+    // next one (the Gram sum of that same update) be scheduled: what it reads is
+    // complete whenever it runs, beside this product.
     pdl_wait();
+    pdl_trigger();
 
     const int64_t u0 = static_cast<int64_t>(blockIdx.x) * P.L;
     const int64_t u1 = min(u0 + P.L, P.units);

@@ -630,6 +630,7 @@ int cox_setup(cox_h *out, const void *X, int64_t n, int64_t p, int x_format, con
     cox_handle *h = new cox_handle();
     h->dev = dev;
     h->sm_count = prop.multiProcessorCount;
+    h->l2_bytes = prop.l2CacheSize;
     h->opt = opt;
     h->n = n;
     h->p = p;
@@ -655,7 +656,9 @@ int cox_setup(cox_h *out, const void *X, int64_t n, int64_t p, int x_format, con
         }
         h->kperm_ainv = ((t0 % nb) + nb) % nb;
     }
-    h->l1_blocks = static_cast<int>(std::min<int64_t>(64, (p + 4095) / 4096));
+    // blocks of the ||beta||_1 partials: four entries per thread while p allows (the
+    // kernel is first in an iteration, and 16 entries one after the other are latency)
+    h->l1_blocks = static_cast<int>(std::min<int64_t>(64, (p + 1023) / 1024));
     {
         int khz = 0;
         if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess || khz <= 0) {

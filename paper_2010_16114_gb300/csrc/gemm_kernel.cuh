@@ -88,6 +88,7 @@ namespace coxgb {
 struct KParams {
     int KC, F, k, stages, ring, nb_period;
     int stages2;        // e2m1 form: depth of the limb ring (stages is the code ring's)
+    int stream;         // codes are loaded with L2 priority evict-first (GemmPlan::stream)
     int pair;           // per-tile issuers commit after every second stage of a window
     const int *bscale;  // k: power-of-two scale of the B limbs
     int64_t units, L;
@@ -338,6 +339,7 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
         // keeps (at least G + R, or a multiple of G: ring_safe).
         if (lane == 0) {
             const bool codes = warp == 0;
+            const uint64_t policy = l2_evict_first();
             const int SR = codes ? S : S2;
             int s = 0, kc = kc0, g = g0;
             uint32_t ph = 0;
@@ -351,7 +353,9 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
                     const uint32_t fb = full0 + 8 * s;
                     armed[s] = static_cast<int>(ph);
                     mbar_arrive_expect_tx(fb, X_BYTES);
-                    tma_load_4d(smem_addr(smem + static_cast<size_t>(s) * X_BYTES), &tmA, 0, 0, kc * CH, g * T, fb);
+                    const uint32_t xs = smem_addr(smem + static_cast<size_t>(s) * X_BYTES);
+                    if (P.stream) tma_load_4d_hint(xs, &tmA, 0, 0, kc * CH, g * T, fb, policy);
+                    else tma_load_4d(xs, &tmA, 0, 0, kc * CH, g * T, fb);
                 } else {
                     const uint32_t fb = lfull0 + 8 * s;
                     const uint32_t st = smem_addr(lring + static_cast<size_t>(s) * B_BYTES);
@@ -374,6 +378,7 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
         // ---------------- TMA producers ----------------
         if (lane == 0) {
             const int w = warp;
+            const uint64_t policy = l2_evict_first();
             int s = w, kc = kc0 + w, g = g0;
             if (kc >= KC) {
                 kc -= KC;
@@ -392,7 +397,8 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
 #pragma unroll
                 for (int h = 0; h < (F4 ? CH / 2 : CH); ++h)
                     tma_load_2d(st + h * NP * 128, &tmB, (F4 ? kc * (CH / 2) + h : kc * CH + h) * 128, 0, fb);
-                tma_load_4d(st + B_BYTES, &tmA, 0, 0, kc * CH, g * T, fb);
+                if (P.stream) tma_load_4d_hint(st + B_BYTES, &tmA, 0, 0, kc * CH, g * T, fb, policy);
+                else tma_load_4d(st + B_BYTES, &tmA, 0, 0, kc * CH, g * T, fb);
                 s += 2;
                 if (s >= S) {
                     s -= S;

@@ -217,6 +217,7 @@ struct GemmPlan {
     int ring = 4;      // TMEM A buffers
     int nb_period = 6; // stage period of the named barriers: lcm(decoder groups, ring)
     int F = 32;        // K chunks per TMEM accumulation window
+    int stream = 0;    // 1: both copies of the codes exceed half of L2: load them evict-first
     int grid = 0;      // CTAs
     int KC = 0;        // stages per M group (K chunks / CH)
     int n_groups = 0;  // M groups
@@ -291,6 +292,7 @@ struct PowerWork {
 
 struct cox_handle {
     int dev = 0, sm_count = 0;
+    int64_t l2_bytes = 0;
     int64_t n = 0, p = 0, n_pad = 0, p_pad = 0;
     int64_t kperm_a = 1, kperm_nb = 1;  // K order of A4 (a4_pos)
     int64_t kperm_ainv = 1;             // a^-1 mod nb: A4 block B holds sorted block ainv B mod nb

@@ -53,6 +53,7 @@ struct GemmArgs {
     int64_t units, L;   // (row tile, chunk) units; units per CTA
     int SL;             // partial slots per row tile
     float *part;        // [tile][slot][r][128] FP32
+    int64_t keep;       // a CTA's first units whose X stays in L2 (-1: no priorities, all of it fits)
     long long wait_limit;
     int *err;
 };
@@ -138,6 +139,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
     if (warp == 0) {
         // ---------------- TMA producer (lane 0) ----------------
         if (lane == 0) {
+            const uint64_t stay = l2_evict_last(), pass = l2_evict_first();
             int g = g0, kc = kc0, s = 0;
             uint32_t ph = 0;
             int64_t issued = 0;
@@ -149,8 +151,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                 const uint32_t st = smem_addr(smem + static_cast<size_t>(s) * STAGE);
                 const uint32_t fb = full0 + 8 * s;
                 mbar_arrive_expect_tx(fb, static_cast<uint32_t>(STAGE));
-                tma_load_2d(st, &tmA, kc * NK, g * NT, fb);
-                tma_load_2d(st + A_BYTES, &tmB, kc * NK, 0, fb);
+                if (P.keep < 0) {
+                    tma_load_2d(st, &tmA, kc * NK, g * NT, fb);
+                    tma_load_2d(st + A_BYTES, &tmB, kc * NK, 0, fb);
+                } else {
+                    tma_load_2d_hint(st, &tmA, kc * NK, g * NT, fb, i < P.keep ? stay : pass);
+                    tma_load_2d_hint(st + A_BYTES, &tmB, kc * NK, 0, fb, stay);
+                }
                 ++issued;
                 if (++s == S) {
                     s = 0;

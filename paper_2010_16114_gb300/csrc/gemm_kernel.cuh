@@ -647,14 +647,19 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
 #pragma unroll
                 for (int tt = 0; tt < T; ++tt) {
 #pragma unroll
-                    for (int cc = 0; cc < NP / 8; ++cc) {
-                        uint32_t u[8];
-                        tmem_ld_32x32b_x8(lane_base + static_cast<uint32_t>(tt * NP + cc * 8), u);
-                        tmem_wait_ld();
-                        float x = __uint_as_float(u[7]);
+                    for (int c0 = 0; c0 < NP / 8; c0 += 4) {  // four loads in flight per wait
+                        uint32_t u[4][8];
 #pragma unroll
-                        for (int l = 6; l >= 0; --l) x = fmaf(x, 0.125f, __uint_as_float(u[l]));
-                        acc(tt, cc) += x;
+                        for (int b = 0; b < 4; ++b)
+                            tmem_ld_32x32b_x8(lane_base + static_cast<uint32_t>(tt * NP + (c0 + b) * 8), u[b]);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            float x = __uint_as_float(u[b][7]);
+#pragma unroll
+                            for (int l = 6; l >= 0; --l) x = fmaf(x, 0.125f, __uint_as_float(u[b][l]));
+                            acc(tt, c0 + b) += x;
+                        }
                     }
                 }
             } else {

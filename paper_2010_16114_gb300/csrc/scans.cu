@@ -216,14 +216,27 @@ __device__ __forceinline__ unsigned column_blocks(const SP &s, int kk)
 // Z^T (delta - u) / n and, for a step, gamma <- gamma + step g_Z (Section 6: the
 // covariates take a plain gradient step; a frozen column keeps its gamma); flags
 // non-finite values.
-__device__ __forceinline__ void finalize_column(const SP &s, int kk, double *sh)
+__device__ __forceinline__ void finalize_column(const SP &s, int kk)
 {
     const double n = static_cast<double>(s.n);
-    for (int cq = 0; cq < s.q; ++cq) {
-        double z = 0.0;
-        for (int c = threadIdx.x; c < s.nch; c += NT) z += s.zvp[(static_cast<int64_t>(kk) * s.q + cq) * s.nch + c];
-        z = block_sum(z, sh) / n;
-        if (threadIdx.x == 0) {
+    const int lane = threadIdx.x & 31;
+    for (int cq = threadIdx.x >> 5; cq < s.q; cq += NW) {  // a warp per covariate
+        const double *zp = s.zvp + (static_cast<int64_t>(kk) * s.q + cq) * s.nch;
+        double z4[4] = {0.0, 0.0, 0.0, 0.0};
+        int c = lane;
+        for (; c + 224 < s.nch; c += 256) {
+            double u[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) u[e] = zp[c + 32 * e];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) z4[e & 3] += u[e];
+        }
+        for (; c < s.nch; c += 32) z4[0] += zp[c];
+        double z = (z4[0] + z4[1]) + (z4[2] + z4[3]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+        z /= n;
+        if (lane == 0) {
             s.gz[kk * s.q + cq] = z;
             if (s.gamma_step && (!s.active || s.active[kk])) s.gamma[kk * s.q + cq] += s.step * z;
             if (!isfinite(z)) atomicOr(s.err, DEVERR_NONFINITE);
@@ -376,10 +389,11 @@ __global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
             const int64_t i = i0 + lane + 32 * j;
             if (i >= s.n) break;
             if (Q) {  // eta += Z gamma (Section 6 unpenalised covariates), in FP64
-                double zg = 0.0;
-#pragma unroll 4
-                for (int cq = 0; cq < s.q; ++cq) zg += s.Z[cq * s.n + i] * s.gamma[kk * s.q + cq];
-                const double vd = as_double(v[j]) + zg;
+                double zg[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+                for (int cq = 0; cq < MAXQ; ++cq)  // unrolled: every load in flight at once
+                    if (cq < s.q) zg[cq & 3] += s.Z[cq * s.n + i] * s.gamma[kk * s.q + cq];
+                const double vd = as_double(v[j]) + ((zg[0] + zg[1]) + (zg[2] + zg[3]));
                 if constexpr (F64) v[j] = vd;
                 else v[j] = tf_of(vd);
             }
@@ -679,14 +693,24 @@ __global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
             if (lane == 0) s.vsp[t] = as_double(vs);
         }
         if (Q) {
+            // sums over the lanes of all 16 values at once: at each of the first four steps
+            // a lane passes half of its values on and keeps the other half (16 FP64 adds
+            // against 80); lanes 2 cq and 2 cq + 1 end with covariate cq's
+            double x[MAXQ];
 #pragma unroll
-            for (int cq = 0; cq < MAXQ; ++cq)
-                if (cq < s.q) {
-                    double x = zv[Q ? cq : 0];
+            for (int cq = 0; cq < MAXQ; ++cq) x[cq] = zv[Q ? cq : 0];
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                    if (lane == 0) s.zvp[(static_cast<int64_t>(kk) * s.q + cq) * nch + c] = x;
+            for (int o = 16, m = MAXQ / 2; m > 0; o >>= 1, m >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int e = 0; e < m; ++e) {
+                    const double send = up ? x[e] : x[e + m], keep = up ? x[e + m] : x[e];
+                    x[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
                 }
+            }
+            x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
+            const int cq = lane >> 1;
+            if (!(lane & 1) && cq < s.q) s.zvp[(static_cast<int64_t>(kk) * s.q + cq) * nch + c] = x[0];
         }
     }
     if (limbs) grid_barrier(s, 4);
@@ -770,7 +794,7 @@ __global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
                 if (lane == 0) s.vsp[t] = finite ? ldexp(static_cast<double>(q), sc - unit) : NAN;
             }
         }
-        if (last_of_column(s, kk, 2, column_blocks(s, kk))) finalize_column(s, kk, shd);
+        if (last_of_column(s, kk, 2, column_blocks(s, kk))) finalize_column(s, kk);
         t0 = t1;
     }
 

@@ -74,8 +74,8 @@ enum {
 enum {
     COX_SPLIT_E4M3 = 0, /* tcgen05 tensor cores (kind::f8f6f4): genotype codes as
                            e4m3, coefficients split into 4 e4m3 limbs under a
-                           power-of-two column scale, FP32 accumulation; FP64
-                           risk-set scans (default).  For k <= 12, unless the
+                           power-of-two column scale, FP32 accumulation;
+                           risk-set scans in pairs of floats and FP64 (default).  For k <= 12, unless the
                            options force a pipeline shape, the same coefficient
                            values run as ten e2m1 digits each (kind::mxf4)     */
     COX_FP64 = 1,       /* FP64 everywhere, dense X (COX_X_F64_HOST)          */
@@ -86,7 +86,7 @@ enum {
                            MMA), coefficients split into 8 e2m1 limbs on the
                            grid of halves under a power-of-two column scale
                            (within 2^-23 of the column's largest magnitude),
-                           FP32 accumulation; FP64 risk-set scans; k <= 16  */
+                           FP32 accumulation; scans as above; k <= 16         */
 };
 
 typedef struct cox_options {

@@ -65,11 +65,17 @@ void free_workspace(cox_handle *h)
     h->ws = Workspace();
 }
 
-int check_device_error(cox_handle *h, cudaStream_t st)
+// Waits for the stream and reports the device-side errors met; with `bytes`, also
+// brings that many back from src to out (host).
+int check_device_error(cox_handle *h, cudaStream_t st, void *out = nullptr, const void *src = nullptr, size_t bytes = 0)
 {
-    int e = 0;
-    COX_CUDA(cudaMemcpyAsync(&e, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    int local = 0, *err = h->pin ? static_cast<int *>(h->pin) : &local;
+    void *stage = pin_stage(h, out, bytes);
+    if (bytes) COX_CUDA(cudaMemcpyAsync(stage, src, bytes, cudaMemcpyDeviceToHost, st));
+    COX_CUDA(cudaMemcpyAsync(err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
     COX_CUDA(cudaStreamSynchronize(st));
+    const int e = *err;
+    if (bytes && stage != out) std::memcpy(out, stage, bytes);
     if (e) {
         COX_CUDA(cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
         COX_CUDA(cudaStreamSynchronize(st));
@@ -589,6 +595,7 @@ void cox_destroy(cox_h h)
     free_workspace(h);
     active_free(h);
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
+    if (h->pin) cudaFreeHost(h->pin);
     void *ptrs[] = {h->d_evhead, h->d_evcnt, h->d_evidx, h->d_evflag, h->d_a4blk, h->d_delta,
                     h->d_mu, h->d_A1, h->d_A4, h->d_Xr, h->d_Xc, h->d_err, h->d_Z, h->pow.base};
     for (void *p : ptrs) dfree(p);
@@ -702,6 +709,10 @@ int cox_setup(cox_h *out, const void *X, int64_t n, int64_t p, int x_format, con
     std::vector<int32_t> a4blk(static_cast<size_t>(h->n_pad / 16));
     for (int64_t b = 0; b < h->n_pad / 16; ++b) a4blk[b] = static_cast<int32_t>(a4_pos(16 * b, h->kperm_a, h->kperm_nb) / 16);
 
+    if (cudaMallocHost(&h->pin, PIN_BYTES) != cudaSuccess) {  // results then come back through pageable memory
+        cudaGetLastError();
+        h->pin = nullptr;
+    }
     cudaStream_t st = 0;
     int rc = COX_OK;
     do {
@@ -1015,11 +1026,10 @@ int cox_loss_grad(cox_h h, const void *beta_dev, int k, double *loss_host, void 
         gout = tmp;
     }
     int rc = iterate(h, const_cast<void *>(beta_dev), k, EPI_GRAD, gout, 0.0, st, zeros.data());
-    if (rc == COX_OK) rc = check_device_error(h, st);
-    if (rc == COX_OK && loss_host) {
-        if (cudaMemcpyAsync(loss_host, h->ws.f, k * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            rc = COX_ERR_CUDA;
+    if (rc == COX_OK) {
+        std::vector<double> f(static_cast<size_t>(k));  // loss_host is written only without an error
+        rc = check_device_error(h, st, f.data(), h->ws.f, loss_host ? k * sizeof(double) : 0);
+        if (rc == COX_OK && loss_host) std::copy(f.begin(), f.end(), loss_host);
     }
     if (tmp) {
         cudaStreamSynchronize(st);
@@ -1139,8 +1149,7 @@ int cox_last_objective(cox_h h, double *obj_host, int k, void *stream)
     if (!h || !obj_host || k != h->ws.k) return COX_ERR_ARG;
     DeviceGuard g(h->dev);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    COX_CUDA(cudaMemcpyAsync(obj_host, h->ws.F, k * sizeof(double), cudaMemcpyDeviceToHost, st));
-    return check_device_error(h, st);
+    return check_device_error(h, st, obj_host, h->ws.F, k * sizeof(double));
 }
 
 int cox_set_covariates(cox_h h, const double *Z_host, int q)

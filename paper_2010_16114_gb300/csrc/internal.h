@@ -327,6 +327,7 @@ struct cox_handle {
     double *d_Xr = nullptr;    // FP64: n x p, sorted rows
     double *d_Xc = nullptr;    // FP64: p x n (columns), sorted subjects
     int *d_err = nullptr;
+    void *pin = nullptr;  // PIN_BYTES of pinned host memory (null: none) for error bits and small results
     int64_t device_bytes = 0;
     long long wait_cycles = 0;
     coxgb::Workspace ws;
@@ -411,6 +412,15 @@ struct LamArg {
 
 int dmalloc(cox_handle *h, void **p, size_t bytes);
 void dfree(void *p);
+
+// Results of up to PIN_BYTES - 64 bytes and the error bits come back through the
+// handle's pinned buffer: two copies and one wait, where each copy to pageable
+// memory is a wait of its own (14-16 us).
+constexpr size_t PIN_BYTES = 16384;
+inline void *pin_stage(cox_handle *h, void *out, size_t bytes)
+{
+    return h->pin && bytes <= PIN_BYTES - 64 ? static_cast<uint8_t *>(h->pin) + 64 : out;
+}
 
 // ---- setup (setup.cu) ----------------------------------------------------------
 int setup_genotypes(cox_handle *h, const void *X, int x_format, cudaStream_t st);

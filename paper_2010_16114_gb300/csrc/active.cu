@@ -101,18 +101,8 @@ __global__ void k_prep_limbs_active(const float *__restrict__ beta, int64_t p, c
     __shared__ int s_sh;
     const int kk = blockIdx.y;
     if (threadIdx.x < 32) {
-        float m = 0.f;
-        for (int b = threadIdx.x; b < nb; b += 32) m = fmaxf(m, maxp[kk * nb + b]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) {
-            if (!isfinite(m)) {
-                atomicOr(err, DEVERR_NONFINITE);
-                m = 0.f;
-            }
-            s_sh = limb_scale(m);
-            if (blockIdx.x == 0) bs[kk] = s_sh;
-        }
+        const int sc = column_scale(maxp + kk * nb, nb, FORM_E4M3, blockIdx.x == 0 ? bs + kk : nullptr, err);
+        if (threadIdx.x == 0) s_sh = sc;
     }
     __syncthreads();
     const int s = s_sh;
@@ -134,18 +124,8 @@ __global__ void k_prep_limbs_active4(const float *__restrict__ beta, int64_t p, 
     __shared__ int s_sh;
     const int kk = blockIdx.y;
     if (threadIdx.x < 32) {
-        float m = 0.f;
-        for (int b = threadIdx.x; b < nb; b += 32) m = fmaxf(m, maxp[kk * nb + b]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) {
-            if (!isfinite(m)) {
-                atomicOr(err, DEVERR_NONFINITE);
-                m = 0.f;
-            }
-            s_sh = limb_scale4(m);
-            if (blockIdx.x == 0) bs[kk] = s_sh;
-        }
+        const int sc = column_scale(maxp + kk * nb, nb, FORM_E2M1, blockIdx.x == 0 ? bs + kk : nullptr, err);
+        if (threadIdx.x == 0) s_sh = sc;
     }
     __syncthreads();
     const int s = s_sh;
@@ -169,18 +149,8 @@ __global__ void k_prep_limbs_active_wide(const float *__restrict__ beta, int64_t
     __shared__ int s_sh;
     const int kk = blockIdx.y;
     if (threadIdx.x < 32) {
-        float m = 0.f;
-        for (int b = threadIdx.x; b < nb; b += 32) m = fmaxf(m, maxp[kk * nb + b]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) {
-            if (!isfinite(m)) {
-                atomicOr(err, DEVERR_NONFINITE);
-                m = 0.f;
-            }
-            s_sh = limb_scale(m);
-            if (blockIdx.x == 0) bs[kk] = s_sh;
-        }
+        const int sc = column_scale(maxp + kk * nb, nb, FORM_WIDE, blockIdx.x == 0 ? bs + kk : nullptr, err);
+        if (threadIdx.x == 0) s_sh = sc;
     }
     __syncthreads();
     const int s = s_sh;
@@ -191,8 +161,6 @@ __global__ void k_prep_limbs_active_wide(const float *__restrict__ beta, int64_t
         uint8_t d[LIMBS], d0[LIMBS_W], d1[LIMBS_W];
         const float *bc = beta + static_cast<int64_t>(kk) * p;
         const float ra = t0 < nA ? ldexpf(bc[Aidx[t0]], -s) : 0.f, rc = t0 + 8 < nA ? ldexpf(bc[Aidx[t0 + 8]], -s) : 0.f;
-        // a NaN passes the maximum and has no digits (as e4m3 it would reach eta)
-        if (!isfinite(ra) || !isfinite(rc)) atomicOr(err, DEVERR_NONFINITE);
         split_wide(split_e4m3_units(ra, d), d0);
         split_wide(split_e4m3_units(rc, d), d1);
 #pragma unroll

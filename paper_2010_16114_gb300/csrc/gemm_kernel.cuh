@@ -90,7 +90,7 @@ struct KParams {
     int stages2;        // e2m1 form: depth of the limb ring (stages is the code ring's)
     int stream;         // codes are loaded with L2 priority evict-first (GemmPlan::stream)
     int pair;           // per-tile issuers commit after every second stage of a window
-    const int *bscale;  // k: power-of-two scale of the B limbs
+    const int *bscale;  // k: power-of-two scale of the B limbs (e2m1 operands: or NAN_SCALE)
     int64_t units, L;
     int64_t rows_pad, slot_stride;
     float *part;
@@ -598,6 +598,10 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
                 }
             }
         }
+        auto scaled = [&](float x, int bs) {  // NAN_SCALE: a column whose digits stand for a non-finite value
+            if (F4 && bs == NAN_SCALE) return __int_as_float(0x7fc00000);
+            return ldexpf(x, bs + SH);
+        };
         uint32_t epi_phase = 0, fold_phase = 0;
         bool ok = true;
 
@@ -740,7 +744,7 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
                         for (int u = 0; u < EB; ++u) {
                             const int e = e0 + u;
                             if (e >= P.k) break;
-                            const float xtv = ldexpf(acc(tt, e), bsc[e] + SH);  // (X^T V)_j
+                            const float xtv = scaled(acc(tt, e), bsc[e]);  // (X^T V)_j
                             acc(tt, e) = 0.f;
                             if (!valid) continue;
                             const float gv = (xtv - muv * colc[e]) * inv_n;
@@ -766,7 +770,7 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
                 const int64_t row = (static_cast<int64_t>(g) * T + tt) * TILE + rit;
 #pragma unroll
                 for (int e = 0; e < KH; ++e) {
-                    if (e < P.k) P.part[slot * P.slot_stride + e * P.rows_pad + row] = ldexpf(acc(tt, e), bsc[e] + SH);
+                    if (e < P.k) P.part[slot * P.slot_stride + e * P.rows_pad + row] = scaled(acc(tt, e), bsc[e]);
                     acc(tt, e) = 0.f;
                 }
             }

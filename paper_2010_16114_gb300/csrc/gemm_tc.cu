@@ -18,18 +18,8 @@ __global__ void k_prep_limbs_beta(const float *__restrict__ beta, int64_t p, int
     __shared__ int s_sh;
     const int kk = blockIdx.y;
     if (threadIdx.x < 32) {
-        float m = 0.f;
-        for (int b = threadIdx.x; b < nb; b += 32) m = fmaxf(m, maxp[kk * nb + b]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) {
-            if (!isfinite(m)) {
-                atomicOr(err, DEVERR_NONFINITE);
-                m = 0.f;
-            }
-            s_sh = limb_scale(m);
-            if (blockIdx.x == 0) bs[kk] = s_sh;
-        }
+        const int sc = column_scale(maxp + kk * nb, nb, FORM_E4M3, blockIdx.x == 0 ? bs + kk : nullptr, err);
+        if (threadIdx.x == 0) s_sh = sc;
     }
     __syncthreads();
     const int s = s_sh;
@@ -53,18 +43,8 @@ __global__ void k_prep_limbs_beta4(const float *__restrict__ beta, int64_t p, in
     __shared__ int s_sh;
     const int kk = blockIdx.y;
     if (threadIdx.x < 32) {
-        float m = 0.f;
-        for (int b = threadIdx.x; b < nb; b += 32) m = fmaxf(m, maxp[kk * nb + b]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) {
-            if (!isfinite(m)) {
-                atomicOr(err, DEVERR_NONFINITE);
-                m = 0.f;
-            }
-            s_sh = limb_scale4(m);
-            if (blockIdx.x == 0) bs[kk] = s_sh;
-        }
+        const int sc = column_scale(maxp + kk * nb, nb, FORM_E2M1, blockIdx.x == 0 ? bs + kk : nullptr, err);
+        if (threadIdx.x == 0) s_sh = sc;
     }
     __syncthreads();
     const int s = s_sh;
@@ -95,18 +75,8 @@ __global__ void k_prep_limbs_beta_wide(const float *__restrict__ beta, int64_t p
     __shared__ int s_sh;
     const int kk = blockIdx.y;
     if (threadIdx.x < 32) {
-        float m = 0.f;
-        for (int b = threadIdx.x; b < nb; b += 32) m = fmaxf(m, maxp[kk * nb + b]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (threadIdx.x == 0) {
-            if (!isfinite(m)) {
-                atomicOr(err, DEVERR_NONFINITE);
-                m = 0.f;
-            }
-            s_sh = limb_scale(m);
-            if (blockIdx.x == 0) bs[kk] = s_sh;
-        }
+        const int sc = column_scale(maxp + kk * nb, nb, FORM_WIDE, blockIdx.x == 0 ? bs + kk : nullptr, err);
+        if (threadIdx.x == 0) s_sh = sc;
     }
     __syncthreads();
     const int s = s_sh;
@@ -118,8 +88,6 @@ __global__ void k_prep_limbs_beta_wide(const float *__restrict__ beta, int64_t p
         uint8_t d[LIMBS], d0[LIMBS_W], d1[LIMBS_W];
         const float *bc = beta + static_cast<int64_t>(kk) * p;
         const float ra = ldexpf(bc[j0], -s), rc = j0 + 8 < p ? ldexpf(bc[j0 + 8], -s) : 0.f;
-        // a NaN passes the maximum and has no digits (as e4m3 it would reach eta)
-        if (!isfinite(ra) || !isfinite(rc)) atomicOr(err, DEVERR_NONFINITE);
         split_wide(split_e4m3_units(ra, d), d0);
         split_wide(split_e4m3_units(rc, d), d1);
 #pragma unroll

@@ -28,6 +28,7 @@ __global__ void k_l1_32(const float *__restrict__ beta, int64_t p, int nb, doubl
     // compensated FP32 sum (Knuth's TwoSum per term; the error terms summed
     // apart): ~2^-48 relative, without GB300's slow FP64 pipe in the loop
     float hi = 0.f, lo = 0.f, m = 0.f;
+    bool nan = false;  // the maximum skips NaN: marked by the partial's sign
     for (int64_t j = static_cast<int64_t>(b) * blockDim.x + threadIdx.x; j < p; j += static_cast<int64_t>(nb) * blockDim.x) {
         const float v = fabsf(beta[kk * p + j]);
         const float t = hi + v;
@@ -35,6 +36,7 @@ __global__ void k_l1_32(const float *__restrict__ beta, int64_t p, int nb, doubl
         lo += (hi - (t - bv)) + (v - bv);
         hi = t;
         m = fmaxf(m, v);
+        nan |= isnan(v);
     }
     double s = static_cast<double>(hi) + static_cast<double>(lo);
     for (int o = 16; o > 0; o >>= 1) {
@@ -45,7 +47,7 @@ __global__ void k_l1_32(const float *__restrict__ beta, int64_t p, int nb, doubl
         sh[threadIdx.x >> 5] = s;
         shm[threadIdx.x >> 5] = m;
     }
-    __syncthreads();
+    nan = __syncthreads_or(nan);
     if (threadIdx.x == 0) {
         double t = 0.0;
         float mm = 0.f;
@@ -54,7 +56,7 @@ __global__ void k_l1_32(const float *__restrict__ beta, int64_t p, int nb, doubl
             mm = fmaxf(mm, shm[w]);
         }
         l1p[kk * nb + b] = t;
-        if (maxp) maxp[kk * nb + b] = mm;
+        if (maxp) maxp[kk * nb + b] = nan ? -mm : mm;
     }
 }
 

@@ -140,7 +140,7 @@ __device__ inline int limb_scale4(float mx) { return mx > 0.f ? ilogbf(mx) : 0; 
 
 // Limbs of r (|r| < 2) as e2m1 nibbles; returns the value they represent in
 // units of 2^(-1 - 3 (LIMBS4 - 1)), an exact integer.  Non-finite r gives zero
-// limbs (its caller flags it).
+// limbs (NAN_SCALE, or a NaN sum of V, stands for it).
 __device__ inline int split_e2m1_units(float r, uint8_t *nib)
 {
     if (!isfinite(r)) {
@@ -160,6 +160,32 @@ __device__ inline int split_e2m1_units(float r, uint8_t *nib)
         r = fmaf(-4.f, t, 8.f * r);  // 8 (r - t / 2), exact
     }
     return q;
+}
+
+// Scale exponent of a column's limbs, by the first warp of a block, from the column's
+// max |beta| partials (k_l1_32; a set sign bit marks NaN entries, which a maximum
+// skips).  bs: where the product finds it (may be null).  An e4m3 limb can be NaN and
+// takes the whole column with it; digits cannot, so a column with a non-finite entry
+// has NAN_SCALE there, which the e2m1 kernels' epilogue turns into NaN: as with FP64
+// and e4m3 operands, eta, the loss and the gradient of that column are NaN.
+constexpr int NAN_SCALE = 1 << 20;
+__device__ inline int column_scale(const float *__restrict__ maxp, int nb, int form, int *bs, int *err)
+{
+    float m = 0.f;
+    unsigned neg = 0;
+    for (int b = threadIdx.x; b < nb; b += 32) {
+        m = fmaxf(m, fabsf(maxp[b]));
+        neg |= __float_as_uint(maxp[b]) >> 31;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const bool inf = !isfinite(m), nan = __any_sync(0xffffffffu, neg);
+    const int s = inf ? 0 : form == FORM_E2M1 ? limb_scale4(m) : limb_scale(m);
+    if (threadIdx.x == 0) {
+        if (inf) atomicOr(err, DEVERR_NONFINITE);
+        if (bs) *bs = form != FORM_E4M3 && (inf || nan) ? NAN_SCALE : s;
+    }
+    return s;
 }
 
 // ---- wide e2m1 limbs --------------------------------------------------------------

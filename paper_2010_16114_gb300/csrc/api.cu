@@ -55,7 +55,7 @@ void free_workspace(cox_handle *h)
 {
     Workspace &w = h->ws;
     void *ptrs[] = {w.eta, w.w, w.Vf, w.Wg, w.Fg, w.tot, w.tbase, w.lgp, w.colc, w.scnt, w.cmax, w.csw, w.suf, w.lossp, w.vsp, w.l1p,
-                    w.sumV, w.f, w.F, w.l1, w.mub, w.lam, w.active, w.Fring, w.Bq, w.Vq, w.bs1, w.bs4, w.bmaxp,
+                    w.sumV, w.f, w.F, w.l1, w.mub, w.lam, w.active, w.Fring, w.Fcol, w.Bq, w.Vq, w.bs1, w.bs4, w.bmaxp,
                     w.vmaxp, w.part1, w.part4, w.cnt4, w.V64, w.V32, w.eta32, w.G32, w.gpart, w.gamma, w.gz, w.zvp};
     for (void *p : ptrs) dfree(p);
     dfree(w.Bqa);
@@ -319,8 +319,8 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
             Site s_(h, 2, 1, st);
             COX_TRY(run_scans(h, sa, st));
         }
-        COX_CUDA(cudaMemcpyAsync(ws.Fring + c, ws.F, sizeof(double), cudaMemcpyDeviceToDevice, st));
-        COX_CUDA(cudaMemcpyAsync(ws.Fring + k + c, ws.f, sizeof(double), cudaMemcpyDeviceToDevice, st));
+        COX_CUDA(cudaMemcpyAsync(ws.Fcol + c, ws.F, sizeof(double), cudaMemcpyDeviceToDevice, st));
+        COX_CUDA(cudaMemcpyAsync(ws.Fcol + k + c, ws.f, sizeof(double), cudaMemcpyDeviceToDevice, st));
         {
             Site s_(h, 1, 3, st);
             COX_TRY(gemv_lut(h, h->d_A4, h->p_pad, h->n_pad / TILE, ws.V32, h->n_pad, ws.gpart, ws.G32, st));
@@ -329,8 +329,8 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
         }
     }
     // gather per-column objectives into F / f
-    COX_CUDA(cudaMemcpyAsync(ws.F, ws.Fring, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    COX_CUDA(cudaMemcpyAsync(ws.f, ws.Fring + k, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    COX_CUDA(cudaMemcpyAsync(ws.F, ws.Fcol, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    COX_CUDA(cudaMemcpyAsync(ws.f, ws.Fcol + k, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
     if (F_out) COX_CUDA(cudaMemcpyAsync(F_out, ws.F, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
     return COX_OK;
 }
@@ -480,7 +480,7 @@ int ensure_workspace(cox_handle *h, int k)
     A(ws.mub, k);
     A(ws.lam, k);
     A(ws.active, k);
-    A(ws.Fring, static_cast<size_t>(std::max(lag, 2)) * k);
+    A(ws.Fring, static_cast<size_t>(lag) * k);
     if (h->q > 0) {
         A(ws.gamma, static_cast<size_t>(k) * h->q);
         A(ws.gz, static_cast<size_t>(k) * h->q);
@@ -531,6 +531,7 @@ int ensure_workspace(cox_handle *h, int k)
     } else if (is_fp64(h)) {
         A(ws.V64, k * n);
     } else {
+        A(ws.Fcol, 2 * static_cast<size_t>(k));
         A(ws.V32, h->n_pad);  // A4 K order; positions of padding stay zero
         cudaMemset(ws.V32, 0, h->n_pad * sizeof(float));
         A(ws.eta32, h->n_pad);

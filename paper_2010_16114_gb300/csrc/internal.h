@@ -273,6 +273,7 @@ struct Workspace {
     double *lam = nullptr;     // k
     int *active = nullptr;     // k
     double *Fring = nullptr;   // lag x k
+    double *Fcol = nullptr;    // 2 k: F and f of the columns done so far (FP32 baseline, one column at a time)
     // split mode
     uint8_t *Bq = nullptr;     // limbs of beta in g1's form: NP x p_pad e4m3 or NP x p_pad / 2 e2m1 pairs
                                // (row c limbs_of(form) + l: limb l of column c)

@@ -216,7 +216,10 @@ int cox_eta(cox_h h, const void *beta_dev, int k, double *eta_dev, void *stream)
  *   beta_dev : p x k in/out (device).
  *   lambdas  : k penalties (host, >= 0).  step: sigma > 0.
  * Asynchronous on `stream`.  The handle keeps F(beta entering this step)
- * per column; cox_last_objective() reads it.
+ * per column; cox_last_objective() reads it.  `lambdas` is read during the
+ * call; under stream capture the copy of it becomes part of the graph, so that
+ * every replay reads the array anew (cox_prox_step_eta likewise): it has to
+ * stay valid, and the first call with k columns has to come before the capture.
  */
 int cox_prox_step(cox_h h, void *beta_dev, const double *lambdas, int k, double step,
                   void *stream);

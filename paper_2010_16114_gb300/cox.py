@@ -123,6 +123,7 @@ class CoxProblem:
         self.h = h
         self.n, self.p = n, p
         self.q = 0
+        self._captured = []  # penalties that captured steps read at replay
         self.precision = precision
         self.dtype = torch.float64 if precision == "fp64" else torch.float32
         dev = torch.cuda.current_device() if device is None else device
@@ -208,6 +209,21 @@ class CoxProblem:
             raise ValueError(f"beta must be a contiguous {self.dtype} CUDA tensor of shape (k, {self.p})")
         return beta
 
+    def _lambdas(self, lambdas, k: int, stream) -> np.ndarray:
+        """k penalties as a float64 array.  A graph that captures the call reads the array at every
+        replay, so it is kept alive then (the caller's own, if it is float64, contiguous and of k
+        entries: replays follow changes to it)."""
+        lam = np.ascontiguousarray(np.broadcast_to(np.asarray(lambdas, dtype=np.float64), (k,)))
+        if stream is None:
+            capturing = torch.cuda.is_current_stream_capturing()
+        else:
+            s = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(int(stream))
+            with torch.cuda.stream(s):
+                capturing = torch.cuda.is_current_stream_capturing()
+        if capturing:
+            self._captured.append(lam)
+        return lam
+
     # -- the iteration ---------------------------------------------------------------------
     def loss_grad(self, beta: torch.Tensor, stream=None):
         """f(beta_c) per row and grad f (same shape as beta)."""
@@ -231,7 +247,7 @@ class CoxProblem:
         """One iteration in place on beta (asynchronous)."""
         b = self._beta(beta)
         k = b.shape[0]
-        lam = np.ascontiguousarray(np.broadcast_to(np.asarray(lambdas, dtype=np.float64), (k,)))
+        lam = self._lambdas(lambdas, k, stream)
         rc = L.cox_prox_step(self.h, _vp(b), _vp(lam), k, float(step), _stream_ptr(stream))
         L.check(rc, "cox_prox_step")
         return beta
@@ -243,7 +259,7 @@ class CoxProblem:
         k = b.shape[0]
         if eta.dtype != torch.float64 or not eta.is_cuda or tuple(eta.shape) != (k, self.n) or not eta.is_contiguous():
             raise ValueError(f"eta must be a contiguous float64 CUDA tensor of shape ({k}, {self.n})")
-        lam = np.ascontiguousarray(np.broadcast_to(np.asarray(lambdas, dtype=np.float64), (k,)))
+        lam = self._lambdas(lambdas, k, stream)
         L.check(L.cox_prox_step_eta(self.h, _vp(b), _vp(eta), _vp(lam), k, float(step), _stream_ptr(stream)),
                 "cox_prox_step_eta")
         return beta

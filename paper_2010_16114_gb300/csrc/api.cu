@@ -120,12 +120,19 @@ int default_form(const cox_handle *h, int k)
     return !forced && limb_cols_wide(k) ? FORM_WIDE : FORM_E4M3;
 }
 
-// The penalties of an iteration as a kernel argument (no copy in the stream), or
-// copied to ws.lam when there are more than it holds.
+// The penalties of an iteration as a kernel argument (no copy in the stream).  Copied to
+// ws.lam instead when there are more than it holds, and under stream capture: there the
+// copy belongs to the graph and reads the caller's array at every replay, where an
+// argument would keep the values of the capture.
 int lam_arg(cox_handle *h, const double *lam, int k, LamArg &a, cudaStream_t st)
 {
     if (!lam) return COX_OK;
-    if (k > MAX_LAM_ARG) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {  // legacy stream beside another stream's capture
+        cudaGetLastError();
+        cap = cudaStreamCaptureStatusNone;
+    }
+    if (k > MAX_LAM_ARG || cap != cudaStreamCaptureStatusNone) {
         COX_CUDA(cudaMemcpyAsync(h->ws.lam, lam, k * sizeof(double), cudaMemcpyHostToDevice, st));
         return COX_OK;
     }

@@ -100,7 +100,9 @@ typedef struct cox_options {
                              built-in default                                       */
     int stages;           /* shared-memory pipeline depth; 0 = automatic             */
     int lag;              /* stopping-rule lag in iterations (default 10, Section 6) */
-    double wait_limit_s;  /* device-side wait limit in seconds (default 2.0)         */
+    double wait_limit_s;  /* limit in seconds of the waits inside the tensor-core
+                             products (default 2.0); the waits of the scans and of
+                             cox_lipschitz have at least the default's              */
     int chunks;           /* 128-wide K chunks per pipeline stage (1 or 2; 3 with
                              two row tiles at 64 limb columns, k = 9..16, where
                              the product's chunk count divides by 3; COX_SPLIT_E2M1:
@@ -153,7 +155,8 @@ void cox_destroy(cox_h h);
  * from the power method of Section 4.4: stop when the estimate changes by at
  * most tol relative (tol <= 0: the paper's 1e-6) or after maxiter iterations
  * (maxiter <= 0: the paper's 1000).  start_host: p doubles, the start vector
- * (NULL: all ones).  Synchronous.
+ * (NULL: all ones).  Synchronous.  Genotype handles run it on the tensor-core
+ * products: COX_ERR_TIMEOUT when one of their waits runs out.
  */
 int cox_lipschitz(cox_h h, const double *start_host, double tol, int maxiter, double *L_out);
 

@@ -404,6 +404,11 @@ int cuda_status(cudaError_t e);
         if (r_ != COX_OK) return r_; \
     } while (0)
 
+// cox_options.wait_limit_s is for the iteration's products.  The scans' grid barriers and
+// the power method's products replaced kernels without any wait, so a handle with a
+// shorter limit gives them at least this one (cycles, about two seconds).
+constexpr long long MIN_WAIT_CYCLES = 4000000000LL;
+
 // Launch with programmatic stream serialisation: the kernel may be scheduled while
 // the one ahead of it in the stream ends, and waits for it (pdl_wait) before it
 // touches global memory.  coop: as a cooperative grid instead, which starts when the

@@ -278,9 +278,7 @@ int power_method_tiles(cox_handle *h, const double *start, double tol, int maxit
         e.part = w.part;
         e.bscale = bscale;
         e.err = &S->err;
-        // at least the default limit: the step size does not take part in a
-        // handle's own wait limit (it had no device-side waits to limit)
-        e.wait = std::max<long long>(h->wait_cycles, 4000000000LL);
+        e.wait = std::max(h->wait_cycles, MIN_WAIT_CYCLES);
         return launch_gemm(h, g, e, 1, st);
     };
     double s = 0.0, s_prev = 0.0;

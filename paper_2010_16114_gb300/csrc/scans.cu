@@ -922,7 +922,7 @@ int run_scans(cox_handle *h, const ScanArgs &a, cudaStream_t st)
     s.F_out = a.F_out;
     s.need_loss = a.need_loss;
     s.err = h->d_err;
-    s.wait_limit = h->wait_cycles;
+    s.wait_limit = std::max(h->wait_cycles, MIN_WAIT_CYCLES);  // FP64 and FP32 handles have no other waits to limit
     const ScanFn fn = pick_scan(h->scan_ept, a.exp64, s.q > 0);
     int occ = 0;
     COX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, NT, 0));

@@ -40,6 +40,31 @@ void dfree(void *p)
     if (p) cudaFree(p);
 }
 
+int device_status(cox_handle *h, cudaStream_t st, void *out, const void *src, size_t bytes)
+{
+    uint8_t buf[RES_BYTES];
+    const uint8_t *err = reinterpret_cast<const uint8_t *>(h->d_err), *from = static_cast<const uint8_t *>(src);
+    size_t span = sizeof(int);
+    if (bytes) {
+        const bool beside = from > err && from + bytes <= err + RES_BYTES;
+        if (beside) span = static_cast<size_t>(from + bytes - err);
+        else COX_CUDA(cudaMemcpyAsync(out, src, bytes, cudaMemcpyDeviceToHost, st));
+    }
+    COX_CUDA(cudaMemcpyAsync(buf, err, span, cudaMemcpyDeviceToHost, st));
+    COX_CUDA(cudaStreamSynchronize(st));
+    if (span > sizeof(int)) std::memcpy(out, buf + span - bytes, bytes);
+    int e;
+    std::memcpy(&e, buf, sizeof(int));
+    if (e) {
+        COX_CUDA(cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
+        COX_CUDA(cudaStreamSynchronize(st));
+        if (e & DEVERR_TIMEOUT) return COX_ERR_TIMEOUT;
+        if (e & DEVERR_NONFINITE) return COX_ERR_NONFINITE;
+        if (e & DEVERR_CODE3) return COX_ERR_CODE3;
+    }
+    return COX_OK;
+}
+
 namespace {
 
 template <typename T>
@@ -55,7 +80,7 @@ void free_workspace(cox_handle *h)
 {
     Workspace &w = h->ws;
     void *ptrs[] = {w.eta, w.w, w.Vf, w.Wg, w.Fg, w.tot, w.tbase, w.lgp, w.colc, w.scnt, w.cmax, w.csw, w.suf, w.lossp, w.vsp, w.l1p,
-                    w.sumV, w.f, w.F, w.l1, w.mub, w.lam, w.active, w.Fring, w.Fcol, w.Bq, w.Vq, w.bs1, w.bs4, w.bmaxp,
+                    w.sumV, w.res, w.mub, w.lam, w.active, w.Fcol, w.Bq, w.Vq, w.bs1, w.bs4, w.bmaxp,
                     w.vmaxp, w.part1, w.part4, w.cnt4, w.V64, w.V32, w.eta32, w.G32, w.gpart, w.gamma, w.gz, w.zvp};
     for (void *p : ptrs) dfree(p);
     dfree(w.Bqa);
@@ -63,27 +88,6 @@ void free_workspace(cox_handle *h)
     (void)g1;
     (void)g4;
     h->ws = Workspace();
-}
-
-// Waits for the stream and reports the device-side errors met; with `bytes`, also
-// brings that many back from src to out (host).
-int check_device_error(cox_handle *h, cudaStream_t st, void *out = nullptr, const void *src = nullptr, size_t bytes = 0)
-{
-    int local = 0, *err = h->pin ? static_cast<int *>(h->pin) : &local;
-    void *stage = pin_stage(h, out, bytes);
-    if (bytes) COX_CUDA(cudaMemcpyAsync(stage, src, bytes, cudaMemcpyDeviceToHost, st));
-    COX_CUDA(cudaMemcpyAsync(err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    COX_CUDA(cudaStreamSynchronize(st));
-    const int e = *err;
-    if (bytes && stage != out) std::memcpy(out, stage, bytes);
-    if (e) {
-        COX_CUDA(cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
-        COX_CUDA(cudaStreamSynchronize(st));
-        if (e & DEVERR_TIMEOUT) return COX_ERR_TIMEOUT;
-        if (e & DEVERR_NONFINITE) return COX_ERR_NONFINITE;
-        if (e & DEVERR_CODE3) return COX_ERR_CODE3;
-    }
-    return COX_OK;
 }
 
 struct DeviceGuard {
@@ -481,13 +485,21 @@ int ensure_workspace(cox_handle *h, int k)
     A(ws.vsp, k * nch);
     A(ws.l1p, static_cast<size_t>(k) * h->l1_blocks);
     A(ws.sumV, k);
-    A(ws.f, k);
-    A(ws.F, k);
-    A(ws.l1, k);
     A(ws.mub, k);
     A(ws.lam, k);
     A(ws.active, k);
-    A(ws.Fring, static_cast<size_t>(lag) * k);
+    // F, f, ||beta||_1 and the ring of a path fit's objectives lie behind the error bits,
+    // so that one copy brings them to the host, unless there are too many
+    const size_t nres = (3 + static_cast<size_t>(lag)) * k;
+    double *res = reinterpret_cast<double *>(reinterpret_cast<uint8_t *>(h->d_err) + RES_HEAD);
+    if (RES_HEAD + nres * sizeof(double) > RES_BYTES) {
+        A(ws.res, nres);
+        res = ws.res;
+    }
+    ws.F = res;
+    ws.f = res + k;
+    ws.l1 = res + 2 * k;
+    ws.Fring = res + 3 * k;
     if (h->q > 0) {
         A(ws.gamma, static_cast<size_t>(k) * h->q);
         A(ws.gz, static_cast<size_t>(k) * h->q);
@@ -603,7 +615,6 @@ void cox_destroy(cox_h h)
     free_workspace(h);
     active_free(h);
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
-    if (h->pin) cudaFreeHost(h->pin);
     void *ptrs[] = {h->d_evhead, h->d_evcnt, h->d_evidx, h->d_evflag, h->d_a4blk, h->d_delta,
                     h->d_mu, h->d_A1, h->d_A4, h->d_Xr, h->d_Xc, h->d_err, h->d_Z, h->pow.base};
     for (void *p : ptrs) dfree(p);
@@ -717,14 +728,10 @@ int cox_setup(cox_h *out, const void *X, int64_t n, int64_t p, int x_format, con
     std::vector<int32_t> a4blk(static_cast<size_t>(h->n_pad / 16));
     for (int64_t b = 0; b < h->n_pad / 16; ++b) a4blk[b] = static_cast<int32_t>(a4_pos(16 * b, h->kperm_a, h->kperm_nb) / 16);
 
-    if (cudaMallocHost(&h->pin, PIN_BYTES) != cudaSuccess) {  // results then come back through pageable memory
-        cudaGetLastError();
-        h->pin = nullptr;
-    }
     cudaStream_t st = 0;
     int rc = COX_OK;
     do {
-        if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_err), sizeof(int))) != COX_OK) break;
+        if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_err), RES_BYTES)) != COX_OK) break;
         if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_evhead), evhead.size() * sizeof(int32_t))) != COX_OK)
             break;
         if ((rc = dmalloc(h, reinterpret_cast<void **>(&h->d_evcnt), evcnt.size() * sizeof(int32_t))) != COX_OK)
@@ -862,7 +869,7 @@ int cox_autotune(cox_h h, int k, int reps, cox_tune_choice *xb, cox_tune_choice 
                     rc = COX_ERR_CUDA;
                     break;
                 }
-                if ((rc = check_device_error(h, 0)) != COX_OK) break;
+                if ((rc = device_status(h, 0)) != COX_OK) break;
                 ++cand[prod];
                 const double m = static_cast<double>(ms) / reps;
                 if (m < best[prod].ms) {
@@ -1016,7 +1023,7 @@ int cox_sync(cox_h h, void *stream)
 {
     if (!h) return COX_ERR_ARG;
     DeviceGuard g(h->dev);
-    return check_device_error(h, static_cast<cudaStream_t>(stream));
+    return device_status(h, static_cast<cudaStream_t>(stream));
 }
 
 int cox_loss_grad(cox_h h, const void *beta_dev, int k, double *loss_host, void *grad_dev, void *stream)
@@ -1036,7 +1043,7 @@ int cox_loss_grad(cox_h h, const void *beta_dev, int k, double *loss_host, void 
     int rc = iterate(h, const_cast<void *>(beta_dev), k, EPI_GRAD, gout, 0.0, st, zeros.data());
     if (rc == COX_OK) {
         std::vector<double> f(static_cast<size_t>(k));  // loss_host is written only without an error
-        rc = check_device_error(h, st, f.data(), h->ws.f, loss_host ? k * sizeof(double) : 0);
+        rc = device_status(h, st, f.data(), h->ws.f, loss_host ? k * sizeof(double) : 0);
         if (rc == COX_OK && loss_host) std::copy(f.begin(), f.end(), loss_host);
     }
     if (tmp) {
@@ -1088,7 +1095,7 @@ int cox_eta(cox_h h, const void *beta_dev, int k, double *eta_dev, void *stream)
     }
     COX_TRY(eta_centred_out(h, beta_dev, is_fp64(h), k, eta_dev, st));
     h->launches += 2;
-    COX_TRY(check_device_error(h, st));
+    COX_TRY(device_status(h, st));
     return COX_OK;
 }
 
@@ -1126,7 +1133,7 @@ int cox_prox_step_host(cox_h h, void *beta_host, const double *lambdas, int k, d
     COX_TRY(check_lambdas(lambdas, k));
     COX_TRY(iterate(h, dbuf, k, EPI_PROX, nullptr, step, st, lambdas));
     COX_CUDA(cudaMemcpyAsync(beta_host, dbuf, bytes, cudaMemcpyDeviceToHost, st));
-    return check_device_error(h, st);
+    return device_status(h, st);
 }
 
 int cox_prox_step_eta(cox_h h, void *beta_dev, const double *eta_dev, const double *lambdas, int k, double step,
@@ -1149,7 +1156,7 @@ int cox_last_loss_l1(cox_h h, double *f_host, double *l1_host, int k, void *stre
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (f_host) COX_CUDA(cudaMemcpyAsync(f_host, h->ws.f, k * sizeof(double), cudaMemcpyDeviceToHost, st));
     if (l1_host) COX_CUDA(cudaMemcpyAsync(l1_host, h->ws.l1, k * sizeof(double), cudaMemcpyDeviceToHost, st));
-    return check_device_error(h, st);
+    return device_status(h, st);
 }
 
 int cox_last_objective(cox_h h, double *obj_host, int k, void *stream)
@@ -1157,7 +1164,7 @@ int cox_last_objective(cox_h h, double *obj_host, int k, void *stream)
     if (!h || !obj_host || k != h->ws.k) return COX_ERR_ARG;
     DeviceGuard g(h->dev);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    return check_device_error(h, st, obj_host, h->ws.F, k * sizeof(double));
+    return device_status(h, st, obj_host, h->ws.F, k * sizeof(double));
 }
 
 int cox_set_covariates(cox_h h, const double *Z_host, int q)

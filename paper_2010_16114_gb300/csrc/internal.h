@@ -268,11 +268,12 @@ struct Workspace {
     double *cmax = nullptr, *csw = nullptr, *suf = nullptr;
     double *lossp = nullptr, *vsp = nullptr;  // k x chunks (lossp: sum of delta eta per chunk)
     double *l1p = nullptr;                    // k x l1 blocks
-    double *sumV = nullptr, *f = nullptr, *F = nullptr, *l1 = nullptr;  // k
+    double *sumV = nullptr;    // k
+    double *F = nullptr, *f = nullptr, *l1 = nullptr, *Fring = nullptr;  // k each, lag x k: behind the error bits,
+    double *res = nullptr;                                               // or here when they do not fit there
     double *mub = nullptr;     // k: mu^T beta (cox_eta)
     double *lam = nullptr;     // k
     int *active = nullptr;     // k
-    double *Fring = nullptr;   // lag x k
     double *Fcol = nullptr;    // 2 k: F and f of the columns done so far (FP32 baseline, one column at a time)
     // split mode
     uint8_t *Bq = nullptr;     // limbs of beta in g1's form: NP x p_pad e4m3 or NP x p_pad / 2 e2m1 pairs
@@ -353,8 +354,7 @@ struct cox_handle {
     uint32_t *d_A4 = nullptr;  // SNP-major 2-bit tiles
     double *d_Xr = nullptr;    // FP64: n x p, sorted rows
     double *d_Xc = nullptr;    // FP64: p x n (columns), sorted subjects
-    int *d_err = nullptr;
-    void *pin = nullptr;  // PIN_BYTES of pinned host memory (null: none) for error bits and small results
+    int *d_err = nullptr;      // error bits: the head of RES_BYTES, small results behind
     int64_t device_bytes = 0;
     long long wait_cycles = 0;
     coxgb::Workspace ws;
@@ -445,14 +445,15 @@ struct LamArg {
 int dmalloc(cox_handle *h, void **p, size_t bytes);
 void dfree(void *p);
 
-// Results of up to PIN_BYTES - 64 bytes and the error bits come back through the
-// handle's pinned buffer: two copies and one wait, where each copy to pageable
-// memory is a wait of its own (14-16 us).
-constexpr size_t PIN_BYTES = 16384;
-inline void *pin_stage(cox_handle *h, void *out, size_t bytes)
-{
-    return h->pin && bytes <= PIN_BYTES - 64 ? static_cast<uint8_t *>(h->pin) + 64 : out;
-}
+// The handle's error bits (d_err) are the head of a block whose rest holds small
+// results.  A copy to pageable memory is a wait of its own (14-16 us), so what a call
+// returns is brought back together with the bits: cox_loss_grad at n = 20,000, p = 2,000
+// takes 126 us against 144 with two copies.  (A pinned buffer per handle did the same
+// and cost every cox_setup 140 us.)
+constexpr size_t RES_HEAD = 64, RES_BYTES = 16384;
+// Waits for the stream, reports and clears the device-side errors met; with `bytes`,
+// also brings that many back from src (device) to out (host).
+int device_status(cox_handle *h, cudaStream_t st, void *out = nullptr, const void *src = nullptr, size_t bytes = 0);
 
 // ---- setup (setup.cu) ----------------------------------------------------------
 int setup_genotypes(cox_handle *h, const void *X, int x_format, cudaStream_t st);

@@ -221,19 +221,8 @@ int path_run(cox_handle *h, int k, int max_iter, double tol, double step, void *
             const int steps = static_cast<int>(std::min<int64_t>(lag, max_iter - t));
             for (int s = 0; s < steps && rc == COX_OK; ++s) rc = one_step(s);
             if (rc != COX_OK) break;
-            const size_t rbytes = static_cast<size_t>(steps) * k * sizeof(double);
-            void *stage = pin_stage(h, ring.data(), rbytes);
-            if (cudaMemcpyAsync(stage, ws.Fring, rbytes, cudaMemcpyDeviceToHost, cs) != cudaSuccess) { rc = COX_ERR_CUDA; break; }
-            int local = 0, *err = h->pin ? static_cast<int *>(h->pin) : &local;
-            if (cudaMemcpyAsync(err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, cs) != cudaSuccess ||
-                cudaStreamSynchronize(cs) != cudaSuccess) { rc = COX_ERR_CUDA; break; }
-            const int e = *err;
-            if (stage != ring.data()) std::memcpy(ring.data(), stage, rbytes);
-            if (e) {
-                cudaMemset(h->d_err, 0, sizeof(int));
-                rc = (e & DEVERR_TIMEOUT) ? COX_ERR_TIMEOUT : COX_ERR_NONFINITE;
-                break;
-            }
+            rc = device_status(h, cs, ring.data(), ws.Fring, static_cast<size_t>(steps) * k * sizeof(double));
+            if (rc != COX_OK) break;
             t += steps;
             bool changed = false;
             for (int c = 0; c < k; ++c) {

@@ -45,3 +45,29 @@ def test_every_iteration_keeps_its_own_objective(precision, lag, iters):
         for c in range(2):
             assert np.array_equal(got[c], want[c]), (c, got[c], want[c])
             assert obj[c] == want[c][-1]
+
+
+@pytest.mark.parametrize("k,lag,iters", [(3, 700, 702), (200, 10, 11), (64, 28, 30)])
+def test_more_results_than_the_small_block(k, lag, iters):
+    """Results that do not fit beside the error bits (16 KB with the ring of the path
+    fit: lag + 3 values per column) come back the same; (64, 28) just fits."""
+    import paper_2010_16114_gb300 as P
+    from paper_2010_16114_gb300.cox import CoxProblem
+    P.build()
+    w, X, Xf, mu = dense_problem("geno_100k_50k", n=200, p=60)
+    lams, step = np.linspace(0.02, 0.0, k), 0.4
+    with CoxProblem(Xf, w.y, w.delta, precision="fp64", center=True, lag=lag) as prob:
+        b = torch.zeros((k, w.p), dtype=torch.float64, device="cuda")
+        want = []
+        for _ in range(iters):
+            prob.prox_step(b, lams, step)
+            want.append(prob.last_objective(k))
+        want = np.array(want).T
+        f, l1 = prob.last_loss_l1(k)
+        assert np.array_equal(f + lams * l1, want[:, -1])
+        fit, it, obj, _ = prob.path_fit(lams, step, max_iter=iters, tol=0.0)
+        got = _history(prob.get_state(), w.p, k, 8)
+        assert torch.equal(fit, b) and np.array_equal(np.array(got), want)
+        assert np.array_equal(obj, want[:, -1])
+        loss, _ = prob.loss_grad(torch.zeros_like(b))
+        assert np.ptp(loss) == 0.0 and loss[0] > 0

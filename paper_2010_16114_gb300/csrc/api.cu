@@ -332,6 +332,7 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
         }
         COX_CUDA(cudaMemcpyAsync(ws.Fcol + c, ws.F, sizeof(double), cudaMemcpyDeviceToDevice, st));
         COX_CUDA(cudaMemcpyAsync(ws.Fcol + k + c, ws.f, sizeof(double), cudaMemcpyDeviceToDevice, st));
+        COX_CUDA(cudaMemcpyAsync(ws.Fcol + 2 * k + c, ws.l1, sizeof(double), cudaMemcpyDeviceToDevice, st));
         {
             Site s_(h, 1, 3, st);
             COX_TRY(gemv_lut(h, h->d_A4, h->p_pad, h->n_pad / TILE, ws.V32, h->n_pad, ws.gpart, ws.G32, st));
@@ -339,9 +340,8 @@ int iterate(cox_handle *h, void *beta, int k, int epi, void *grad, double step, 
             COX_TRY(prox_or_grad32(h, ws.G32, c, epi == EPI_PROX ? b32 : nullptr, gc, ws.lam, step, st));
         }
     }
-    // gather per-column objectives into F / f
-    COX_CUDA(cudaMemcpyAsync(ws.F, ws.Fcol, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    COX_CUDA(cudaMemcpyAsync(ws.f, ws.Fcol + k, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    // gather the columns' results
+    COX_CUDA(cudaMemcpyAsync(ws.F, ws.Fcol, 3 * k * sizeof(double), cudaMemcpyDeviceToDevice, st));  // F, f, l1
     if (F_out) COX_CUDA(cudaMemcpyAsync(F_out, ws.F, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
     return COX_OK;
 }
@@ -550,7 +550,7 @@ int ensure_workspace(cox_handle *h, int k)
     } else if (is_fp64(h)) {
         A(ws.V64, k * n);
     } else {
-        A(ws.Fcol, 2 * static_cast<size_t>(k));
+        A(ws.Fcol, 3 * static_cast<size_t>(k));
         A(ws.V32, h->n_pad);  // A4 K order; positions of padding stay zero
         cudaMemset(ws.V32, 0, h->n_pad * sizeof(float));
         A(ws.eta32, h->n_pad);

@@ -274,7 +274,7 @@ struct Workspace {
     double *mub = nullptr;     // k: mu^T beta (cox_eta)
     double *lam = nullptr;     // k
     int *active = nullptr;     // k
-    double *Fcol = nullptr;    // 2 k: F and f of the columns done so far (FP32 baseline, one column at a time)
+    double *Fcol = nullptr;    // 3 k: F, f, l1 of the columns done so far (FP32 baseline, one column at a time)
     // split mode
     uint8_t *Bq = nullptr;     // limbs of beta in g1's form: NP x p_pad e4m3 or NP x p_pad / 2 e2m1 pairs
                                // (row c limbs_of(form) + l: limb l of column c)

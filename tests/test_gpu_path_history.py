@@ -71,3 +71,22 @@ def test_more_results_than_the_small_block(k, lag, iters):
         assert np.array_equal(obj, want[:, -1])
         loss, _ = prob.loss_grad(torch.zeros_like(b))
         assert np.ptp(loss) == 0.0 and loss[0] > 0
+
+
+@pytest.mark.parametrize("precision", ["fp32_gemv", "split_e4m3", "split_e2m1", "fp64"])
+def test_loss_and_l1_of_every_column(precision):
+    import paper_2010_16114_gb300 as P
+    from paper_2010_16114_gb300.cox import CoxProblem
+    P.build()
+    w, X, Xf, mu = dense_problem("geno_100k_50k", n=900, p=300)
+    B = np.random.default_rng(5).normal(size=(3, w.p)) * np.array([[0.01], [0.03], [0.002]])
+    lams = [0.01, 0.002, 0.0]
+    with CoxProblem(Xf if precision == "fp64" else X, w.y, w.delta, precision=precision, center=True) as prob:
+        b = torch.tensor(B, dtype=prob.dtype, device="cuda")
+        norms = b.double().abs().sum(1).cpu().numpy()
+        loss, _ = prob.loss_grad(b)
+        prob.prox_step(b, lams, 0.3)
+        f, l1 = prob.last_loss_l1(3)
+        assert np.array_equal(f, loss)
+        assert np.allclose(l1, norms, rtol=1e-12, atol=0)  # sums of 300 terms in FP64 or pairs of floats
+        assert np.allclose(prob.last_objective(3), f + np.array(lams) * l1, rtol=1e-14, atol=0)

@@ -256,6 +256,7 @@ struct GemmPlan {
 
 struct Workspace {
     int k = 0;        // columns the workspace is sized for
+    void *base = nullptr;       // the allocation that holds everything below but part1 and Bqa
     // split / gemv / fp64 common (sorted subject order)
     double *eta = nullptr;      // k x n
     void *w = nullptr;          // k x n: float, double for FP64 handles
@@ -269,8 +270,7 @@ struct Workspace {
     double *lossp = nullptr, *vsp = nullptr;  // k x chunks (lossp: sum of delta eta per chunk)
     double *l1p = nullptr;                    // k x l1 blocks
     double *sumV = nullptr;    // k
-    double *F = nullptr, *f = nullptr, *l1 = nullptr, *Fring = nullptr;  // k each, lag x k: behind the error bits,
-    double *res = nullptr;                                               // or here when they do not fit there
+    double *F = nullptr, *f = nullptr, *l1 = nullptr, *Fring = nullptr;  // k each, lag x k, in a row
     double *mub = nullptr;     // k: mu^T beta (cox_eta)
     double *lam = nullptr;     // k
     int *active = nullptr;     // k

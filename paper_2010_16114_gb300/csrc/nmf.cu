@@ -51,6 +51,7 @@ struct UpdArgs {
     int64_t L;
     const float *Gin;        // Gram matrix of the other factor, FP32 rows of gram_ld(r)
     const tf *Gsq;           // its pairs' parts of the squared Frobenius norm (the APG step)
+    const double *G64;       // the same matrix in FP64, for squared norms outside FP32's range
     double eps;
     float *gpart;            // Gram partials of the new F: [block][pair], pairs c <= d
     int *err;
@@ -177,7 +178,14 @@ __global__ void __launch_bounds__(640) k_nmf_update(const UpdArgs A)
                 for (int q = 0; q < CPW; ++q) sum[q] = tf_add(sum[q], tf{b[u][q], 0.f});
         }
 #pragma unroll
-        for (int q = 0; q < CPW; ++q) pc[q] = sum[q].h;  // the pair's sum rounded to FP32
+        for (int q = 0; q < CPW; ++q) {
+            pc[q] = sum[q].h;  // the pair's sum rounded to FP32
+            if (!isfinite(pc[q])) {  // past FP32's range pairs give NaN: the infinity it is
+                double d = 0.0;
+                for (int sl = 0; sl < ns; ++sl) d += c0 + q < r ? static_cast<double>(pp[sl * ps + q * NT]) : 0.0;
+                pc[q] = static_cast<float>(d);
+            }
+        }
     }
 #pragma unroll
     for (int q = 0; q < CPW; ++q)
@@ -187,7 +195,12 @@ __global__ void __launch_bounds__(640) k_nmf_update(const UpdArgs A)
         if (t == 0) {
             tf f2 = fro_w[0];
             for (int v = 1; v < W; ++v) f2 = tf_add(f2, fro_w[v]);
-            step_s = static_cast<float>(1.0 / (2.0 * tf_double(f2) + A.eps));
+            double g2 = tf_double(f2);
+            if (!(f2.h > 1e-30f && f2.h < 1e37f)) {  // the squares leave FP32's range
+                g2 = 0.0;
+                for (int e = 0; e < r * r; ++e) g2 = fma(A.G64[e], A.G64[e], g2);
+            }
+            step_s = static_cast<float>(1.0 / (2.0 * g2 + A.eps));
         }
         __syncthreads();
     }
@@ -633,6 +646,7 @@ int launch_update(nmf_handle *h, int side, int mode, int algo, double eps, cudaS
     a.L = sd.g.L;
     a.Gin = side == 0 ? h->GW32 : h->GV32;
     a.Gsq = side == 0 ? h->GWsq : h->GVsq;
+    a.G64 = side == 0 ? h->GW64 : h->GV64;
     a.eps = eps;
     a.gpart = side == 0 ? h->gpartV : h->gpartW;
     a.err = h->err;

@@ -4,7 +4,7 @@
 //
 // An iteration is six kernels:
 //   k_nmf_gemm    P = X W^T   (m x r)   tcgen05 kind::f16, A = X row-major
-//   k_nmf_gram    W W^T (FP64) from the partials of W's update, beside that product
+//   k_nmf_gram    W W^T from the partials of W's update, beside that product
 //   k_nmf_update  V from P and W W^T; limbs of V; per-block partials of V^T V
 //   k_nmf_gemm    Q = X^T V   (n x r)   A = X column-major
 //   k_nmf_gram    V^T V, beside that product
@@ -299,11 +299,17 @@ struct GramArgs {
     tf *Gsq;                 // per pair: its part of ||G||_F^2
 };
 
-// G = F F^T from the update blocks' partials, in FP64: 32 pairs per block (one per
-// lane), warp y adds the blocks b = y, y + 8, ..., then the warps' sums in warp
-// order (a fixed order: deterministic).  Runs beside the product that follows the
+// G = F F^T from the update blocks' partials: 32 pairs per block (one per lane), warp y
+// adds the blocks b = y, y + 8, ... in pairs of floats, then the warps' sums in FP64 in
+// warp order (a fixed order: deterministic).  Runs beside the product that follows the
 // update: that product lets it start once the update is complete, and it waits for
 // the product only at its end, so that the update behind it finds both complete.
+// Beside a product there may be room on few SMs only (one that the product's grid
+// leaves free, or those whose CTA ends first), and eight of these blocks then share an
+// SM: summed in FP64, its two FP64 lanes made that longer than the product (5000 x 5000,
+// r = 20: 59.6 us an iteration against 53.7 with each Gram sum behind its update;
+// 10,000 x 10,000, r = 80: 238 against 221).  Pairs (2^-47 relative; the partials are
+// FP32 sums of 32 terms) take 39.1 and 159.
 __global__ void __launch_bounds__(256) k_nmf_gram(const GramArgs A)
 {
     __shared__ double sums[8][32];
@@ -314,18 +320,25 @@ __global__ void __launch_bounds__(256) k_nmf_gram(const GramArgs A)
     double v = 0.0;
     if (p < npair) {
         const float *src = A.gpart + p;
-        double v4[4] = {0.0, 0.0, 0.0, 0.0};
+        tf a[2] = {{0.f, 0.f}, {0.f, 0.f}};
         int b = y;
         for (; b + 56 < A.nblk; b += 64) {
             float u[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) u[q] = __ldcg(src + static_cast<int64_t>(b + 8 * q) * npair);
+            tf t[4];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v4[q & 3] += static_cast<double>(u[q]);
+            for (int q = 0; q < 4; ++q) t[q] = two_sum(u[2 * q], u[2 * q + 1]);
+            a[0] = tf_add(a[0], tf_add(t[0], t[1]));
+            a[1] = tf_add(a[1], tf_add(t[2], t[3]));
         }
 #pragma unroll 4
-        for (; b < A.nblk; b += 8) v4[0] += static_cast<double>(__ldcg(src + static_cast<int64_t>(b) * npair));
-        v = (v4[0] + v4[1]) + (v4[2] + v4[3]);
+        for (; b < A.nblk; b += 8) a[0] = tf_add(a[0], tf{__ldcg(src + static_cast<int64_t>(b) * npair), 0.f});
+        v = tf_double(tf_add(a[0], a[1]));
+        if (!(v < 1e37)) {  // the pairs left FP32's range
+            v = 0.0;
+            for (b = y; b < A.nblk; b += 8) v += static_cast<double>(__ldcg(src + static_cast<int64_t>(b) * npair));
+        }
     }
     sums[y][lane] = v;
     __syncthreads();

@@ -53,3 +53,19 @@ def test_overflowing_product_is_reported(algo, m, n):
         h.sync()
     assert e.value.code == L.COX_ERR_NONFINITE
     h.close()
+
+
+@pytest.mark.parametrize("r", [3, 20, 80])
+def test_gram_sums_past_fp32(r):
+    """Gram partials that are finite in FP32 while their sum is not: the sum is finite in
+    FP64, and the update takes the FP32 infinity of it (V -> 0 for finite products)."""
+    m, n = 200, 12_800
+    X = np.full((m, n), 1.0, np.float32)
+    h = _nmf(X, r)
+    W0 = np.full((r, n), np.float32(1.5e18))  # 32 columns: 7.2e37 a partial, 400 blocks: 2.9e40
+    h.set_factors(np.ones((m, r), np.float32), W0)
+    f = h.objective()
+    # ||X - V W||^2 with every entry (1.5e18 r)^2 to rounding
+    want = float(m) * n * (1.5e18 * r) ** 2
+    assert any(abs(f - s * want) <= 1e-5 * s * want for s in (0.5, 1.0)), (f, want)
+    h.close()

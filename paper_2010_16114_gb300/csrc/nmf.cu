@@ -546,6 +546,7 @@ struct nmf_handle {
     NmfSide s1, s2;               // X W^T, X^T V
     float *GV32 = nullptr, *GW32 = nullptr;
     float *gpartV = nullptr, *gpartW = nullptr;  // Gram partials [update block][pair]
+    bool gw_behind = false;    // GW is of an earlier W than the last iteration's
     coxgb::tf *GVsq = nullptr, *GWsq = nullptr;   // per pair: its part of ||G||_F^2
     double *GV64 = nullptr, *GW64 = nullptr, *opart = nullptr, *fobj = nullptr;
     int *counters = nullptr, *err = nullptr;
@@ -910,6 +911,7 @@ int nmf_set_factors(nmf_h h, const float *V, const float *W, void *stream)
     COX_TRY(launch_gram(h, 0, st, false));
     COX_TRY(launch_update(h, 1, 0, 0, 0.0, st));
     COX_TRY(launch_gram(h, 1, st, false));
+    h->gw_behind = false;
     return check_err(h, st);
 }
 
@@ -958,6 +960,7 @@ int nmf_iterate(nmf_h h, int algo, int64_t iters, double eps, void *stream)
         h->g_algo = algo;
         h->g_eps = eps;
     }
+    h->gw_behind = true;
     for (int64_t t = 0; t < iters; ++t) COX_CUDA(cudaGraphLaunch(h->exec, st));
     h->launches += 6 * iters;
     return COX_OK;
@@ -968,8 +971,11 @@ int nmf_objective(nmf_h h, double *f, void *stream)
     if (!h || !f) return COX_ERR_ARG;
     DevGuard guard(h->dev);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    COX_TRY(launch_gram(h, 1, st, false));  // W's is otherwise formed in the next iteration
     COX_TRY(launch_gemm(h, h->s1, st));
+    if (h->gw_behind) {  // an iteration leaves W's Gram matrix to the next one's product
+        COX_TRY(launch_gram(h, 1, st, true));
+        h->gw_behind = false;
+    }
     FitArgs a;
     a.r = h->r;
     a.R = h->m;

@@ -69,3 +69,29 @@ def test_gram_sums_past_fp32(r):
     want = float(m) * n * (1.5e18 * r) ** 2
     assert any(abs(f - s * want) <= 1e-5 * s * want for s in (0.5, 1.0)), (f, want)
     h.close()
+
+
+def test_objective_between_iterations():
+    """The objective after every mix of iterations, set_factors and repeated calls is that
+    of the factors now held (W's Gram matrix is formed late)."""
+    m, n, r = 400, 900, 9
+    X, V0, W0 = synth.nmf_inputs(m, n, r)
+    h = _nmf(X, r)
+
+    def check():
+        V, W = h.factors()
+        want = oracle.nmf_objective(X, V, W)
+        for _ in range(2):
+            assert abs(h.objective() - want) <= 1e-5 * want
+
+    h.set_factors(V0, W0)
+    check()
+    for algo, iters in (("mult", 1), ("apg", 2), ("mult", 0), ("mult", 3)):
+        h.iterate(iters, algo)
+        check()
+    h.set_factors(V0 * 0.5, W0)
+    check()
+    h.iterate(1, "apg")
+    h.set_factors(V0, W0 * 2)
+    check()
+    h.close()

@@ -582,14 +582,22 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
         float *accs = reinterpret_cast<float *>(smem + ring_bytes + 1024) + (threadIdx.x - 32 * DEC0);
         auto acc = [&](int tt, int e) -> float & { return accs[(tt * KH + e) * 128]; };
         // per-column constants, loaded once: sum V, step lambda, active (fused
-        // step) and the power-of-two scale of the B limbs
+        // step) or the scale's factors (partial sums alone), and the power-of-two
+        // scale of the B limbs
         float *colc = reinterpret_cast<float *>(smem + ring_bytes + 1024) + T * KH * 128;
         if (gamma == 0) {
             for (int e = 0; e < T * KH; ++e) accs[e * 128] = 0.f;
             const int tid = threadIdx.x - 32 * DEC0;
             if (tid < P.k) {
-                reinterpret_cast<int *>(colc + 3 * KH)[tid] = P.bscale[tid];
-                if (P.epi != EPI_PARTIAL) {
+                const int bs = P.bscale[tid];
+                reinterpret_cast<int *>(colc + 3 * KH)[tid] = bs;
+                if (P.epi == EPI_PARTIAL) {
+                    // the scale as two factors, 2^(s/2) 2^(s-s/2): exact, and NaN for a column
+                    // whose digits stand for a non-finite value
+                    const int sc = bs + SH;
+                    colc[tid] = bs == NAN_SCALE ? __int_as_float(0x7fc00000) : ldexpf(1.f, sc / 2);
+                    colc[KH + tid] = bs == NAN_SCALE ? 1.f : ldexpf(1.f, sc - sc / 2);
+                } else {
                     colc[tid] = static_cast<float>(P.sumV[tid]);
                     if (P.epi == EPI_PROX) {
                         colc[KH + tid] = static_cast<float>(P.step * P.lam[tid]);
@@ -598,10 +606,6 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
                 }
             }
         }
-        auto scaled = [&](float x, int bs) {  // NAN_SCALE: a column whose digits stand for a non-finite value
-            if (F4 && bs == NAN_SCALE) return __int_as_float(0x7fc00000);
-            return ldexpf(x, bs + SH);
-        };
         uint32_t epi_phase = 0, fold_phase = 0;
         bool ok = true;
 
@@ -744,7 +748,7 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
                         for (int u = 0; u < EB; ++u) {
                             const int e = e0 + u;
                             if (e >= P.k) break;
-                            const float xtv = scaled(acc(tt, e), bsc[e]);  // (X^T V)_j
+                            const float xtv = ldexpf(acc(tt, e), bsc[e] + SH);  // (X^T V)_j
                             acc(tt, e) = 0.f;
                             if (!valid) continue;
                             const float gv = (xtv - muv * colc[e]) * inv_n;
@@ -770,7 +774,9 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
                 const int64_t row = (static_cast<int64_t>(g) * T + tt) * TILE + rit;
 #pragma unroll
                 for (int e = 0; e < KH; ++e) {
-                    if (e < P.k) P.part[slot * P.slot_stride + e * P.rows_pad + row] = scaled(acc(tt, e), bsc[e]);
+                    if (e < P.k)
+                        P.part[slot * P.slot_stride + e * P.rows_pad + row] =
+                            P.epi == EPI_PARTIAL ? acc(tt, e) * colc[e] * colc[KH + e] : ldexpf(acc(tt, e), bsc[e] + SH);
                     acc(tt, e) = 0.f;
                 }
             }

@@ -23,40 +23,39 @@ __global__ void k_l1_32(const float *__restrict__ beta, int64_t p, int nb, doubl
     pdl_wait();
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < lam.k) lam_dev[threadIdx.x] = lam.v[threadIdx.x];
     __shared__ double sh[8];
-    __shared__ float shm[8];
+    __shared__ unsigned shm[8];
     const int b = blockIdx.x, kk = blockIdx.y;
     // compensated FP32 sum (Knuth's TwoSum per term; the error terms summed
     // apart): ~2^-48 relative, without GB300's slow FP64 pipe in the loop
-    float hi = 0.f, lo = 0.f, m = 0.f;
-    bool nan = false;  // the maximum skips NaN: marked by the partial's sign
+    float hi = 0.f, lo = 0.f;
+    unsigned m = 0;  // bits of the largest |beta|: a NaN's exceed every number's
     for (int64_t j = static_cast<int64_t>(b) * blockDim.x + threadIdx.x; j < p; j += static_cast<int64_t>(nb) * blockDim.x) {
         const float v = fabsf(beta[kk * p + j]);
         const float t = hi + v;
         const float bv = t - hi;
         lo += (hi - (t - bv)) + (v - bv);
         hi = t;
-        m = fmaxf(m, v);
-        nan |= isnan(v);
+        m = max(m, __float_as_uint(v));
     }
     double s = static_cast<double>(hi) + static_cast<double>(lo);
     for (int o = 16; o > 0; o >>= 1) {
         s += __shfl_xor_sync(0xffffffffu, s, o);
-        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     }
     if ((threadIdx.x & 31) == 0) {
         sh[threadIdx.x >> 5] = s;
         shm[threadIdx.x >> 5] = m;
     }
-    nan = __syncthreads_or(nan);
+    __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        float mm = 0.f;
+        unsigned mm = 0;
         for (int w = 0; w < blockDim.x / 32; ++w) {
             t += sh[w];
-            mm = fmaxf(mm, shm[w]);
+            mm = max(mm, shm[w]);
         }
         l1p[kk * nb + b] = t;
-        if (maxp) maxp[kk * nb + b] = nan ? -mm : mm;
+        if (maxp) maxp[kk * nb + b] = __uint_as_float(mm);
     }
 }
 

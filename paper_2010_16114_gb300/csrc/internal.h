@@ -163,27 +163,23 @@ __device__ inline int split_e2m1_units(float r, uint8_t *nib)
 }
 
 // Scale exponent of a column's limbs, by the first warp of a block, from the column's
-// max |beta| partials (k_l1_32; a set sign bit marks NaN entries, which a maximum
-// skips).  bs: where the product finds it (may be null).  An e4m3 limb can be NaN and
-// takes the whole column with it; digits cannot, so a column with a non-finite entry
-// has NAN_SCALE there, which the e2m1 kernels' epilogue turns into NaN: as with FP64
+// max |beta| partials (k_l1_32, compared as bits: a NaN exceeds every number).  bs:
+// where the product finds it (may be null).  An e4m3 limb can be NaN and takes the
+// whole column with it; digits cannot, so a column with a non-finite entry has
+// NAN_SCALE there, which turns the e2m1 kernels' partial sums into NaN: as with FP64
 // and e4m3 operands, eta, the loss and the gradient of that column are NaN.
 constexpr int NAN_SCALE = 1 << 20;
 __device__ inline int column_scale(const float *__restrict__ maxp, int nb, int form, int *bs, int *err)
 {
-    float m = 0.f;
-    unsigned neg = 0;
-    for (int b = threadIdx.x; b < nb; b += 32) {
-        m = fmaxf(m, fabsf(maxp[b]));
-        neg |= __float_as_uint(maxp[b]) >> 31;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    const bool inf = !isfinite(m), nan = __any_sync(0xffffffffu, neg);
-    const int s = inf ? 0 : form == FORM_E2M1 ? limb_scale4(m) : limb_scale(m);
+    unsigned u = 0;
+    for (int b = threadIdx.x; b < nb; b += 32) u = max(u, __float_as_uint(maxp[b]));
+    u = __reduce_max_sync(0xffffffffu, u);
+    const float m = __uint_as_float(u);
+    const bool bad = !isfinite(m);
+    const int s = bad ? 0 : form == FORM_E2M1 ? limb_scale4(m) : limb_scale(m);
     if (threadIdx.x == 0) {
-        if (inf) atomicOr(err, DEVERR_NONFINITE);
-        if (bs) *bs = form != FORM_E4M3 && (inf || nan) ? NAN_SCALE : s;
+        if (isinf(m)) atomicOr(err, DEVERR_NONFINITE);  // a NaN is reported by the scans
+        if (bs) *bs = form != FORM_E4M3 && bad ? NAN_SCALE : s;
     }
     return s;
 }

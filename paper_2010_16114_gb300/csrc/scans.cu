@@ -316,13 +316,20 @@ __device__ __forceinline__ int slot_count(const SP &s, int64_t g)
 __device__ __forceinline__ int padded(int e) { return e + (e >> 5); }
 
 // EPT: subjects per lane (a chunk is the 32 EPT subjects of one warp); F64: FP64
-// throughout (COX_FP64); Q: with unpenalised covariates (their sums take 32
-// registers).  Block b takes the chunks [b per, (b + 1) per) of the column-major
+// throughout (COX_FP64); Q: the most unpenalised covariates (0, 4, 8 or 16; FP64 handles
+// have no 8).  A covariate costs two FP64 multiply-adds per subject and column whether a
+// call has it or not, and two registers, so a call takes the smallest variant that holds
+// its q: a step at n = 400,000, p = 5,000, k = 16 takes 736 us with q <= 4 (four blocks
+// per SM), 845 with q <= 8 (three), 970 with q <= 12 and 1,066 with 16 (two), where one
+// variant of 16 took 1,040-1,060 for any q, more than the separate kernels before the
+// fused scans for q < 8 (898 at q = 1, 24 more per covariate).
+// Block b takes the chunks [b per, (b + 1) per) of the column-major
 // list, its warps in turn; nothing inside a chunk waits for another warp.
-template <int EPT, bool F64, bool Q>
-__global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
+template <int EPT, bool F64, int Q>
+__global__ void __launch_bounds__(NT, Q > 8 ? 2 : Q > 4 ? 3 : 4) k_scans(const SP s)
 {
     constexpr int CW = 32 * EPT;
+    constexpr int SURE = F64 ? 0 : Q > 4 ? Q / 2 : 0;  // covariates that every call of this variant has
     constexpr int BW = CW + CW / 32;  // doubles of a warp's buffer
     using acc_t = typename std::conditional<F64, double, tf>::type;
     using w_t = typename std::conditional<F64, double, float>::type;
@@ -391,8 +398,10 @@ __global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
             if (Q) {  // eta += Z gamma (Section 6 unpenalised covariates), in FP64
                 double zg[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-                for (int cq = 0; cq < MAXQ; ++cq)  // unrolled: every load in flight at once
-                    if (cq < s.q) zg[cq & 3] += s.Z[cq * s.n + i] * s.gamma[kk * s.q + cq];
+                for (int cq = 0; cq < Q; ++cq) {  // unrolled: every load in flight at once
+                    if (cq == 12 && s.q <= 12) break;
+                    if (cq < SURE || cq < s.q) zg[cq & 3] += s.Z[cq * s.n + i] * s.gamma[kk * s.q + cq];
+                }
                 const double vd = as_double(v[j]) + ((zg[0] + zg[1]) + (zg[2] + zg[3]));
                 if constexpr (F64) v[j] = vd;
                 else v[j] = tf_of(vd);
@@ -640,11 +649,7 @@ __global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
         __syncwarp();
         acc_t vs = zero;
         float vm32 = 0.f;
-        double zv[Q ? MAXQ : 1];  // Z^T V over this lane's subjects (unpenalised covariates)
-        if (Q) {
-#pragma unroll
-            for (int cq = 0; cq < MAXQ; ++cq) zv[Q ? cq : 0] = 0.0;
-        }
+        double zv[Q ? Q : 1] = {};  // Z^T V over this lane's subjects (unpenalised covariates)
 #pragma unroll
         for (int j = 0; j < EPT; ++j) {
             const int64_t i = i0 + lane + 32 * j;
@@ -665,8 +670,10 @@ __global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
             }
             if (Q) {
 #pragma unroll
-                for (int cq = 0; cq < MAXQ; ++cq)
-                    if (cq < s.q) zv[Q ? cq : 0] += s.Z[cq * s.n + i] * V;
+                for (int cq = 0; cq < Q; ++cq) {
+                    if (cq == 12 && s.q <= 12) break;
+                    if (cq < SURE || cq < s.q) zv[cq] += s.Z[cq * s.n + i] * V;
+                }
             }
             // sum V in the form the product reads: X^T V - mu sum V is then
             // exactly the centred product of that V.  (Censored subjects between
@@ -692,25 +699,23 @@ __global__ void __launch_bounds__(NT, Q ? 2 : 4) k_scans(const SP s)
             for (int o = 16; o > 0; o >>= 1) vs = plus(vs, shfl_xor(vs, o));
             if (lane == 0) s.vsp[t] = as_double(vs);
         }
-        if (Q) {
-            // sums over the lanes of all 16 values at once: at each of the first four steps
-            // a lane passes half of its values on and keeps the other half (16 FP64 adds
-            // against 80); lanes 2 cq and 2 cq + 1 end with covariate cq's
-            double x[MAXQ];
+        if constexpr (Q > 0) {
+            // sums over the lanes of all Q values at once: at each of the first log2 Q steps a
+            // lane passes half of its values on and keeps the other half (Q = 16: 16 FP64 adds
+            // against 80); the 32 / Q lanes from (32 / Q) cq on end with covariate cq's
 #pragma unroll
-            for (int cq = 0; cq < MAXQ; ++cq) x[cq] = zv[Q ? cq : 0];
-#pragma unroll
-            for (int o = 16, m = MAXQ / 2; m > 0; o >>= 1, m >>= 1) {
+            for (int o = 16, m = Q / 2; m > 0; o >>= 1, m >>= 1) {
                 const bool up = (lane & o) != 0;
 #pragma unroll
                 for (int e = 0; e < m; ++e) {
-                    const double send = up ? x[e] : x[e + m], keep = up ? x[e + m] : x[e];
-                    x[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    const double send = up ? zv[e] : zv[e + m], keep = up ? zv[e + m] : zv[e];
+                    zv[e] = keep + __shfl_xor_sync(0xffffffffu, send, o);
                 }
             }
-            x[0] += __shfl_xor_sync(0xffffffffu, x[0], 1);
-            const int cq = lane >> 1;
-            if (!(lane & 1) && cq < s.q) s.zvp[(static_cast<int64_t>(kk) * s.q + cq) * nch + c] = x[0];
+#pragma unroll
+            for (int o = 16 / Q; o > 0; o >>= 1) zv[0] += __shfl_xor_sync(0xffffffffu, zv[0], o);
+            const int cq = lane / (32 / Q);
+            if (lane % (32 / Q) == 0 && cq < s.q) s.zvp[(static_cast<int64_t>(kk) * s.q + cq) * nch + c] = zv[0];
         }
     }
     if (limbs) grid_barrier(s, 4);
@@ -825,20 +830,21 @@ __global__ void k_eta(const float *__restrict__ part, int64_t n, int64_t slot_st
 
 using ScanFn = void (*)(const SP);
 
-template <int EPT>
-ScanFn pick_scan(bool f64, bool q)
+template <int EPT, bool F64>
+ScanFn pick_scan(int q)
 {
-    return f64 ? (q ? k_scans<EPT, true, true> : k_scans<EPT, true, false>)
-               : (q ? k_scans<EPT, false, true> : k_scans<EPT, false, false>);
+    if (q > 8 || (F64 && q > 4)) return k_scans<EPT, F64, MAXQ>;
+    if (q > 4) return k_scans<EPT, F64, F64 ? MAXQ : 8>;
+    return q > 0 ? k_scans<EPT, F64, 4> : k_scans<EPT, F64, 0>;
 }
 
-ScanFn pick_scan(int ept, bool f64, bool q)
+ScanFn pick_scan(int ept, bool f64, int q)
 {
     switch (ept) {
-    case 1: return pick_scan<1>(f64, q);
-    case 2: return pick_scan<2>(f64, q);
-    case 4: return pick_scan<4>(f64, q);
-    default: return pick_scan<8>(f64, q);
+    case 1: return f64 ? pick_scan<1, true>(q) : pick_scan<1, false>(q);
+    case 2: return f64 ? pick_scan<2, true>(q) : pick_scan<2, false>(q);
+    case 4: return f64 ? pick_scan<4, true>(q) : pick_scan<4, false>(q);
+    default: return f64 ? pick_scan<8, true>(q) : pick_scan<8, false>(q);
     }
 }
 
@@ -923,7 +929,7 @@ int run_scans(cox_handle *h, const ScanArgs &a, cudaStream_t st)
     s.need_loss = a.need_loss;
     s.err = h->d_err;
     s.wait_limit = std::max(h->wait_cycles, MIN_WAIT_CYCLES);  // FP64 and FP32 handles have no other waits to limit
-    const ScanFn fn = pick_scan(h->scan_ept, a.exp64, s.q > 0);
+    const ScanFn fn = pick_scan(h->scan_ept, a.exp64, s.q);
     int occ = 0;
     COX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, NT, 0));
     // a warp per chunk, up to what the SMs hold at once (the grid barrier needs every

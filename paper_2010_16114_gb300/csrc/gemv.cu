@@ -236,13 +236,18 @@ __global__ void k_prox32(const float *__restrict__ G, int64_t p, const double *_
     }
 }
 
-// Lane's part of a dot product of `len` doubles: eight loads of each vector in flight
-// and four interleaved sums (one load at a time left a warp waiting on memory for
-// every 32 entries: the step at n = 1,000, p = 2,000 took 60.8 us, now 55.4).
+// Lane's part of a dot product of `len` doubles.  BATCH: eight loads of each vector in
+// flight and four interleaved sums; else one load at a time in fewer registers.
+template <bool BATCH>
 __device__ __forceinline__ double dot64(const double *__restrict__ a, const double *__restrict__ b, int64_t len, int lane)
 {
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
     int64_t j = lane;
+    if constexpr (!BATCH) {
+        double t = 0.0;
+        for (; j < len; j += 32) t += a[j] * b[j];
+        return t;
+    }
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
     for (; j + 224 < len; j += 256) {
         double u[8], v[8];
 #pragma unroll
@@ -258,6 +263,7 @@ __device__ __forceinline__ double dot64(const double *__restrict__ a, const doub
 }
 
 // FP64 path: eta[kk][i] = sum_j X[i][j] beta[kk][j]  (one warp per (i, kk)).
+template <bool BATCH>
 __global__ void k_eta64(const double *__restrict__ Xr, int64_t n, int64_t p, const double *__restrict__ beta,
                         int k, double *__restrict__ eta)
 {
@@ -269,12 +275,13 @@ __global__ void k_eta64(const double *__restrict__ Xr, int64_t n, int64_t p, con
     const int64_t i = wid % n;
     const int kk = static_cast<int>(wid / n);
     double s = 0.0;
-    s = dot64(Xr + i * p, beta + kk * p, p, lane);
+    s = dot64<BATCH>(Xr + i * p, beta + kk * p, p, lane);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) eta[kk * n + i] = s;
 }
 
 // FP64 path: G_j = sum_i X[i][j] V[kk][i]; then the step or the gradient.
+template <bool BATCH>
 __global__ void k_xtv64(const double *__restrict__ Xc, int64_t n, int64_t p, const double *__restrict__ V, int k,
                         const double *__restrict__ mu, const double *__restrict__ sumV, double *beta, double *grad,
                         const double *__restrict__ lam, double step, const int *active)
@@ -287,7 +294,7 @@ __global__ void k_xtv64(const double *__restrict__ Xc, int64_t n, int64_t p, con
     const int64_t j = wid % p;
     const int kk = static_cast<int>(wid / p);
     double s = 0.0;
-    s = dot64(Xc + j * n, V + kk * n, n, lane);
+    s = dot64<BATCH>(Xc + j * n, V + kk * n, n, lane);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane != 0) return;
     const double g = (s - mu[j] * sumV[kk]) / static_cast<double>(n);
@@ -335,6 +342,14 @@ __global__ void k_eta_out(const double *__restrict__ eta, const double *__restri
          i += static_cast<int64_t>(gridDim.x) * blockDim.x)
         out[kk * n + i] = eta[kk * n + i] - d;
 }
+
+// Whether the FP64 products batch their loads: where a warp would else wait on memory
+// for every 32 entries, with few warps (1,000 of 2,000 entries 14.4 -> 12.4 us, of 20,000
+// 153 -> 89) or long rows (10,000 entries in 2,000 warps 84 -> 55, 4,000 in 8,000 74.5 ->
+// 67.9).  With many short rows resident warps hide the latency, and the batch's 48
+// registers cost a third of them: 1,000 entries in 20,000 warps 69.7 us against 57.8, 20
+// in 100,000 60.3 against 42.2.  In between (2,000 .. 5,000 entries) both are within 7%.
+bool batch_dots(const cox_handle *h, int64_t warps, int64_t len) { return warps < 8LL * h->sm_count || len >= 2500; }
 
 unsigned blocks_for(int64_t n, int t) { return static_cast<unsigned>((n + t - 1) / t); }
 
@@ -406,7 +421,8 @@ int prox_or_grad32(cox_handle *h, const float *G, int col, float *beta, float *g
 int eta64(cox_handle *h, const double *beta, int k, double *eta, cudaStream_t st)
 {
     const int64_t warps = h->n * k;
-    COX_CUDA(launch_pdl(k_eta64, dim3(blocks_for(warps * 32, 256)), 256, 0, st, false, h->d_Xr, h->n, h->p, beta, k, eta));
+    COX_CUDA(launch_pdl(batch_dots(h, warps, h->p) ? k_eta64<true> : k_eta64<false>, dim3(blocks_for(warps * 32, 256)), 256,
+                        0, st, false, h->d_Xr, h->n, h->p, beta, k, eta));
     return COX_OK;
 }
 
@@ -414,8 +430,8 @@ int xtv64(cox_handle *h, const double *V, int k, double *beta, double *grad, con
           cudaStream_t st)
 {
     const int64_t warps = h->p * k;
-    COX_CUDA(launch_pdl(k_xtv64, dim3(blocks_for(warps * 32, 256)), 256, 0, st, false, h->d_Xc, h->n, h->p, V, k, h->d_mu,
-                        h->ws.sumV, beta, grad, lam, step, h->ws.active));
+    COX_CUDA(launch_pdl(batch_dots(h, warps, h->n) ? k_xtv64<true> : k_xtv64<false>, dim3(blocks_for(warps * 32, 256)), 256,
+                        0, st, false, h->d_Xc, h->n, h->p, V, k, h->d_mu, h->ws.sumV, beta, grad, lam, step, h->ws.active));
     return COX_OK;
 }
 

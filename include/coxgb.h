@@ -350,6 +350,9 @@ int cox_get_info(cox_h h, cox_info *info);
  * changes).  The fastest shape per product is kept for k and used by later
  * calls with k columns unless cox_options forces tile_m, chunks or stages.
  * xb / xtv (either may be NULL) receive the choice and its mean launch time.
+ * COX_SPLIT_E4M3 handles time the wide form too (k <= 12); where it is the
+ * fastest, the choice's tile_m, chunks, stages and issue are 0, the options
+ * with which a handle takes that form (cox_plan_in_use describes the kernel).
  * Drops the per-k workspace.  Synchronous.  Errors: COX_ERR_UNSUPPORTED for
  * other precisions; COX_ERR_ARG for k outside 1..64 (1..16 for COX_SPLIT_E2M1)
  * or reps < 1.
@@ -357,7 +360,7 @@ int cox_get_info(cox_h h, cox_info *info);
 typedef struct cox_tune_choice {
     int tile_m, chunks, stages, candidates;
     double ms;
-    int issue;            /* cox_options.issue of the choice (1 or 2)               */
+    int issue;            /* cox_options.issue of the choice (1 or 2; 0: wide form)  */
 } cox_tune_choice;
 int cox_autotune(cox_h h, int k, int reps, cox_tune_choice *xb, cox_tune_choice *xtv);
 
@@ -367,9 +370,10 @@ int cox_autotune(cox_h h, int k, int reps, cox_tune_choice *xb, cox_tune_choice 
  * without a device or handle: for k coefficient columns (1..64) and a shape
  * (tile_m 128-row tiles per CTA, chunks 128-wide K chunks per stage, issue as
  * cox_options.issue; 0 = the built-in default) at a shared-memory depth
- * (stages; 0 = the deepest that fits), the plan of the e4m3 kernel that
- * cox_setup's handles would launch (for k <= 12 they do when the options force
- * a shape).  Every plan it returns keeps the pipeline's invariants: ring >=
+ * (stages; 0 = the deepest that fits), the plan of the e4m3 kernel.  A handle
+ * launches it when its options force that shape; what a handle without forced
+ * options launches is cox_plan_default's answer (for k <= 12 the wide form, for
+ * k = 17 .. 32 another shape than this query's built-in default).  Every plan it returns keeps the pipeline's invariants: ring >=
  * decoder_groups, ring < stages (e2m1: ring < limb_stages), named_barriers <= 15, tmem_cols <= 512,
  * smem_bytes within the device's per-block limit, and for issue 2 two decoder
  * groups with an even ring and an even number of stages.  Errors: COX_ERR_ARG
@@ -381,16 +385,16 @@ typedef struct cox_plan {
     int ring;             /* TMEM slots of decoded genotype codes                  */
     int decoder_groups;   /* decoder warp groups (each takes every G-th stage)     */
     int named_barriers;   /* hardware barriers in use: lcm(groups, ring) x tile_m  */
-    int limb_cols;        /* e4m3 limb columns: N of every MMA                     */
+    int limb_cols;        /* limb columns: N of every MMA                          */
     int tmem_cols;        /* accumulators + slots, of the 512 an SM has            */
     long long smem_bytes; /* dynamic shared memory per CTA                         */
     int issue;            /* 1 one issuer per row tile, 2 two on alternate stages,
                              3 one per row tile committing every second stage      */
     int issuers;          /* MMA issuer warps                                      */
     int mmas_per_commit;  /* tcgen05.mma instructions per issuer commit            */
-    int limb_stages;      /* COX_SPLIT_E2M1: slots of the limb ring, ring + 2 (the
-                             codes then have a ring of their own, `stages` deep,
-                             freed as soon as they are decoded); 0 otherwise      */
+    int limb_stages;      /* e2m1 operands: slots of the limb ring, ring + 1 .. ring
+                             + 4 (the codes then have a ring of their own, `stages`
+                             deep, freed as soon as they are decoded); 0 for e4m3  */
 } cox_plan;
 int cox_plan_shape(int k, int tile_m, int chunks, int stages, int issue, cox_plan *out);
 /* The same plan for either operand form: precision COX_SPLIT_E4M3 (as
@@ -398,6 +402,22 @@ int cox_plan_shape(int k, int tile_m, int chunks, int stages, int issue, cox_pla
  * counts e2m1 limb columns, tmem_cols includes the 8 scale-factor columns).
  * COX_ERR_ARG for any other precision or a shape that is not compiled. */
 int cox_plan_shape_prec(int precision, int k, int tile_m, int chunks, int stages, int issue, cox_plan *out);
+
+/* Operand forms of the products. */
+enum {
+    COX_FORM_E4M3 = 0, /* e4m3 codes, 4 e4m3 limbs per coefficient (kind::f8f6f4)   */
+    COX_FORM_E2M1 = 1, /* e2m1 codes, 8 e2m1 limbs (kind::mxf4), k <= 16             */
+    COX_FORM_WIDE = 2  /* e2m1 codes, the e4m3 limbs' value as 10 e2m1 digits, k <= 12 */
+};
+/* The same plan for an operand form (errors as cox_plan_shape_prec). */
+int cox_plan_form(int form, int k, int tile_m, int chunks, int stages, int issue, cox_plan *out);
+/* The form (may be NULL) and plan that a handle of a tensor-core precision
+ * launches for k columns with default options.  Host only.  COX_ERR_ARG as above. */
+int cox_plan_default(int precision, int k, int *form, cox_plan *out);
+/* The form (may be NULL) and plan that this handle launches for k columns:
+ * forced by its options, else autotuned, else the default; product 0 is X B,
+ * 1 is X^T V.  COX_ERR_UNSUPPORTED for handles without tensor-core products. */
+int cox_plan_in_use(cox_h h, int k, int product, int *form, cox_plan *out);
 
 /*
  * SNP ranking of Section 6 on a lambda path's coefficients (host arithmetic,

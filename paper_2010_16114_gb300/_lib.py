@@ -31,6 +31,10 @@ COX_FP64 = 1
 COX_FP32_GEMV = 2
 COX_SPLIT_E2M1 = 3
 
+COX_FORM_E4M3 = 0
+COX_FORM_E2M1 = 1
+COX_FORM_WIDE = 2
+
 # every symbol include/coxgb.h declares
 EXPORTS = [
     "cox_default_options", "cox_setup", "cox_destroy", "cox_lipschitz", "cox_lambda_max",
@@ -39,7 +43,7 @@ EXPORTS = [
     "cox_strerror", "cox_set_precision", "cox_profile", "cox_profile_read", "cox_lipschitz_noalloc",
     "cox_autotune", "cox_eta", "cox_plan_shape", "cox_rank_by_entry", "cox_path_seq", "cox_set_covariates",
     "cox_get_gamma", "cox_set_gamma", "cox_grad_gamma", "cox_prox_step_eta", "cox_last_loss_l1",
-    "cox_set_active_set", "cox_plan_shape_prec",
+    "cox_set_active_set", "cox_plan_shape_prec", "cox_plan_form", "cox_plan_default", "cox_plan_in_use",
 ]
 # every symbol include/nmfgb.h declares
 NMF_EXPORTS = [
@@ -154,6 +158,12 @@ def load(path: str | None = None):
     lib.cox_plan_shape.argtypes = [I, I, I, I, I, ctypes.POINTER(cox_plan)]
     lib.cox_plan_shape_prec.restype = I
     lib.cox_plan_shape_prec.argtypes = [I, I, I, I, I, I, ctypes.POINTER(cox_plan)]
+    lib.cox_plan_form.restype = I
+    lib.cox_plan_form.argtypes = [I, I, I, I, I, I, ctypes.POINTER(cox_plan)]
+    lib.cox_plan_default.restype = I
+    lib.cox_plan_default.argtypes = [I, I, ctypes.POINTER(I), ctypes.POINTER(cox_plan)]
+    lib.cox_plan_in_use.restype = I
+    lib.cox_plan_in_use.argtypes = [P, I, I, ctypes.POINTER(I), ctypes.POINTER(cox_plan)]
     lib.cox_rank_by_entry.restype = I
     lib.cox_rank_by_entry.argtypes = [I64, I, P, P, I, P, P, ctypes.POINTER(I64)]
     lib.cox_path_seq.restype = I
@@ -321,6 +331,27 @@ def cox_plan_shape_prec(precision: int, k: int, tile_m: int = 0, chunks: int = 0
     out = cox_plan()
     rc = load().cox_plan_shape_prec(precision, k, tile_m, chunks, stages, issue, ctypes.byref(out))
     return rc, out
+
+
+def cox_plan_form(form: int, k: int, tile_m: int = 0, chunks: int = 0, stages: int = 0, issue: int = 0):
+    """(rc, cox_plan) of an operand form of the tensor-core products; host only."""
+    out = cox_plan()
+    rc = load().cox_plan_form(form, k, tile_m, chunks, stages, issue, ctypes.byref(out))
+    return rc, out
+
+
+def cox_plan_default(precision: int, k: int):
+    """(rc, form, cox_plan) that default handles of a precision launch; host only."""
+    form, out = ctypes.c_int(-1), cox_plan()
+    rc = load().cox_plan_default(precision, k, ctypes.byref(form), ctypes.byref(out))
+    return rc, form.value, out
+
+
+def cox_plan_in_use(h, k: int, product: int):
+    """(rc, form, cox_plan) that a handle launches for k columns (product 0: X B, 1: X^T V)."""
+    form, out = ctypes.c_int(-1), cox_plan()
+    rc = load().cox_plan_in_use(h, k, product, ctypes.byref(form), ctypes.byref(out))
+    return rc, form.value, out
 
 
 def cox_strerror(code: int) -> str:

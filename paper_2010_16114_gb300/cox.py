@@ -40,11 +40,23 @@ def plan_shape(k: int, tile_m: int = 0, chunks: int = 0, stages: int = 0, issue:
     """The tensor-core products' pipeline plan for k columns (cox_plan_shape_prec):
     shape, issue mode, shared-memory depth, TMEM slots, barriers and memory, for
     the e4m3 or the e2m1 operand form.  Host only; raises CoxError for a shape or
-    depth the pipeline does not allow."""
+    depth the pipeline does not allow.  What a handle launches unless its options
+    force a shape: default_plan."""
     rc, p = L.cox_plan_shape_prec(PRECISIONS[precision], int(k), int(tile_m), int(chunks), int(stages),
                                   int(issue))
     L.check(rc, "cox_plan_shape_prec")
     return {f: getattr(p, f) for f, _ in L.cox_plan._fields_}
+
+
+FORMS = {L.COX_FORM_E4M3: "e4m3", L.COX_FORM_E2M1: "e2m1", L.COX_FORM_WIDE: "wide"}
+
+
+def default_plan(k: int, precision: str = "split_e4m3") -> dict:
+    """The operand form and pipeline plan that default handles of a precision launch
+    for k columns (cox_plan_default).  Host only."""
+    rc, form, p = L.cox_plan_default(PRECISIONS[precision], int(k))
+    L.check(rc, "cox_plan_default")
+    return {"form": FORMS[form], **{f: getattr(p, f) for f, _ in L.cox_plan._fields_}}
 
 
 def rank_by_entry(lambdas, beta):
@@ -169,9 +181,21 @@ class CoxProblem:
         L.check(L.cox_set_precision(self.h, PRECISIONS[precision]), "cox_set_precision")
         self.precision = precision
 
+    def plan(self, k: int) -> dict:
+        """The operand form and pipeline plan of both products for k columns
+        (cox_plan_in_use): forced by the options, else autotuned, else the default."""
+        out = {}
+        for product, name in enumerate(("x_b", "xt_v")):
+            rc, form, p = L.cox_plan_in_use(self.h, int(k), product)
+            L.check(rc, "cox_plan_in_use")
+            out[name] = {"form": FORMS[form], **{f: getattr(p, f) for f, _ in L.cox_plan._fields_}}
+        return out
+
     def autotune(self, k: int, reps: int = 3):
         """Time every compiled pipeline shape of both products for k columns and
-        keep the fastest (cox_autotune); returns the choices."""
+        keep the fastest (cox_autotune); returns the choices, whose tile_m, chunks,
+        stages and issue are options that give a handle the same kernel (zeros: the
+        wide form)."""
         rc, xb, xtv = L.cox_autotune(self.h, int(k), int(reps))
         L.check(rc, "cox_autotune")
         f = [n for n, _ in L.cox_tune_choice._fields_]

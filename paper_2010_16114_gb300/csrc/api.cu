@@ -105,16 +105,58 @@ int tune_key(const cox_handle *h, int k) { return is_e2m1(h) ? k + 4096 : k; }
 // largest k of the tensor-core products: 128 e2m1 limb columns hold 16 coefficients
 int max_k_tc(const cox_handle *h) { return is_e2m1(h) ? MAX_K_E2M1 : MAX_K_TC; }
 
-// The operand form of a handle's products for k columns when the options force
-// no pipeline shape: an e4m3 handle takes the wide form where it holds k
-// columns, k <= 12 (the same coefficients and exact window sums; the product
-// is then bound by HBM, not by MMA issue).  Past 12 columns the wide limbs
-// would need more than 128 MMA columns, twice the e4m3 kernel's MMA cycles.
-int default_form(const cox_handle *h, int k)
+// One product's operand form and shape request (0: the planner's default).
+struct Shape {
+    int form, T, CH, S, issue;
+};
+
+// What handles of a precision launch for k columns when the options force no pipeline
+// shape and nothing is tuned.  An e4m3 handle takes the wide form where it holds k
+// columns, k <= 12 (the same coefficients and exact window sums; the product is then
+// bound by HBM, not by MMA issue): whole steps at k = 1 .. 12 are 1.15 to 1.7 times as
+// fast as with the e4m3 kernel at n x p = 4,099 x 1,500, 20,000 x 5,000, 5,000 x 100,000,
+// 100,000 x 50,000 and 400,000 x 20,000 (least at 20,000 x 5,000, k = 12: 143 us against
+// 164).  Past 12 columns the wide limbs would need more than 128 MMA columns, twice the
+// e4m3 kernel's MMA cycles.  k = 17 .. 32: two K chunks per stage and two decoder groups
+// give 8 MMAs per commit; a step at n = 400,000, p = 100,000, k = 32 takes 6.6 ms against
+// 7.2 with one chunk.
+Shape default_shape(int precision, int k)
 {
-    if (is_e2m1(h)) return FORM_E2M1;
-    const bool forced = h->opt.tile_m || h->opt.chunks || h->opt.stages || h->opt.issue;
-    return !forced && limb_cols_wide(k) ? FORM_WIDE : FORM_E4M3;
+    if (precision == COX_SPLIT_E2M1) return {FORM_E2M1, 0, 0, 0, 0};
+    if (limb_cols_wide(k)) return {FORM_WIDE, 0, 0, 0, 0};
+    if (limb_cols(k) == 128) return {FORM_E4M3, 2, 2, 0, 0};
+    return {FORM_E4M3, 0, 0, 0, 0};
+}
+
+// A handle's shape for k columns (product 0: X B, 1: X^T V): forced by the options, else
+// autotuned for k, else the default.
+Shape shape_for_handle(const cox_handle *h, int k, int product)
+{
+    const cox_options &o = h->opt;
+    if (o.tile_m || o.chunks || o.stages || o.issue)
+        return {is_e2m1(h) ? FORM_E2M1 : FORM_E4M3, o.tile_m, o.chunks, o.stages, o.issue};
+    const auto tc = h->tuned.find(tune_key(h, k));
+    if (tc == h->tuned.end()) return default_shape(o.precision, k);
+    const cox_handle::TuneChoice &t = tc->second;
+    return product == 0 ? Shape{t.F1, t.T1, t.CH1, t.S1, t.A1} : Shape{t.F4, t.T4, t.CH4, t.S4, t.A4};
+}
+
+void fill_plan(const GemmPlan &g, int form, cox_plan *out)
+{
+    const bool f4 = form != FORM_E4M3;
+    out->tile_m = g.T;
+    out->chunks = g.CH;
+    out->stages = g.stages;
+    out->ring = g.ring;
+    out->decoder_groups = g.G;
+    out->named_barriers = g.nb_period * g.T;
+    out->limb_cols = g.NP;
+    out->tmem_cols = (g.alt ? 2 : 1) * g.T * g.NP + g.ring * g.T * g.CH * (f4 ? 16 : 32) + (f4 ? 8 : 0);
+    out->smem_bytes = static_cast<long long>(g.smem);
+    out->issue = g.alt ? 2 : g.pair ? 3 : 1;
+    out->issuers = g.alt ? 2 : g.T;
+    out->mmas_per_commit = (f4 ? 2 : 4) * g.CH * (g.alt ? g.T : g.pair ? 2 : 1);
+    out->limb_stages = f4 ? g.stages2 : 0;
 }
 
 // The penalties of an iteration as a kernel argument (no copy in the stream).  Copied to
@@ -479,28 +521,12 @@ int ensure_workspace(cox_handle *h, int k)
         need(plain, ws.gz, K * q);
         need(plain, ws.zvp, K * q * nch);
     }
-    // pipeline shapes and operand forms: forced by the options, else autotuned for k, else default
-    int T1 = h->opt.tile_m, C1 = h->opt.chunks, S1 = h->opt.stages, A1 = h->opt.issue;
-    int T4 = T1, C4 = C1, S4 = S1, A4 = A1;
-    int F1 = FORM_E4M3, F4 = FORM_E4M3;
+    const Shape s1 = shape_for_handle(h, k, 0), s4 = shape_for_handle(h, k, 1);
     auto plan = [&]() -> int {
-        COX_TRY(plan_gemm(h, ws.g1, h->d_A1, h->n_pad, h->p_pad, ws.Bq, k, F1, T1, C1, S1, A1));
-        return plan_gemm(h, ws.g4, h->d_A4, h->p_pad, h->n_pad, ws.Vq, k, F4, T4, C4, S4, A4);
+        COX_TRY(plan_gemm(h, ws.g1, h->d_A1, h->n_pad, h->p_pad, ws.Bq, k, s1.form, s1.T, s1.CH, s1.S, s1.issue));
+        return plan_gemm(h, ws.g4, h->d_A4, h->p_pad, h->n_pad, ws.Vq, k, s4.form, s4.T, s4.CH, s4.S, s4.issue);
     };
     if (is_split(h)) {
-        F1 = F4 = default_form(h, k);
-        const auto tc = h->tuned.find(tune_key(h, k));
-        const bool automatic = !T1 && !C1 && !S1 && !A1;
-        if (automatic && F1 == FORM_E4M3 && limb_cols(k) == 128) {
-            // k = 17 .. 32: two K chunks per stage and two decoder groups give 8 MMAs per
-            // commit; a step at n = 400,000, p = 100,000, k = 32 takes 6.62 ms against 7.19
-            T1 = T4 = 2;
-            C1 = C4 = 2;
-        }
-        if (tc != h->tuned.end() && automatic) {
-            T1 = tc->second.T1, C1 = tc->second.CH1, S1 = tc->second.S1, A1 = tc->second.A1, F1 = tc->second.F1;
-            T4 = tc->second.T4, C4 = tc->second.CH4, S4 = tc->second.S4, A4 = tc->second.A4, F4 = tc->second.F4;
-        }
         // planned on the genotype copies for the sizes, and on the limbs once they have an address
         ws.Bq = reinterpret_cast<uint8_t *>(h->d_A1);
         ws.Vq = reinterpret_cast<uint8_t *>(h->d_A4);
@@ -511,8 +537,8 @@ int ensure_workspace(cox_handle *h, int k)
         }
         // limb rows of K_pad e4m3 bytes, or K_pad / 2 bytes of e2m1 pairs; rows past the
         // coefficients' and K positions of padding stay zero
-        need(zeroed, ws.Bq, static_cast<size_t>(limb_cols_of(F1, k)) * h->p_pad / (F1 ? 2 : 1));
-        need(zeroed, ws.Vq, static_cast<size_t>(limb_cols_of(F4, k)) * h->n_pad / (F4 ? 2 : 1));
+        need(zeroed, ws.Bq, static_cast<size_t>(limb_cols_of(s1.form, k)) * h->p_pad / (s1.form ? 2 : 1));
+        need(zeroed, ws.Vq, static_cast<size_t>(limb_cols_of(s4.form, k)) * h->n_pad / (s4.form ? 2 : 1));
         need(zeroed, ws.bs1, K);
         need(zeroed, ws.bs4, K);
         need(zeroed, ws.cnt4, static_cast<size_t>(ws.g4.n_groups));
@@ -885,6 +911,9 @@ int cox_autotune(cox_h h, int k, int reps, cox_tune_choice *xb, cox_tune_choice 
                                          best_form[0], best_form[1]};
     cudaDeviceSynchronize();
     free_workspace(h);  // the next call with k columns plans the chosen shapes
+    // no option names the wide form: its choice is the options' zeros, with which the next handle takes it
+    for (int prod = 0; prod < 2; ++prod)
+        if (best_form[prod] == FORM_WIDE) best[prod].tile_m = best[prod].chunks = best[prod].stages = best[prod].issue = 0;
     if (xb) *xb = best[0];
     if (xtv) *xtv = best[1];
     return COX_OK;
@@ -932,24 +961,37 @@ int cox_plan_shape(int k, int tile_m, int chunks, int stages, int issue, cox_pla
 
 int cox_plan_shape_prec(int precision, int k, int tile_m, int chunks, int stages, int issue, cox_plan *out)
 {
-    if (!out || tile_m < 0 || chunks < 0 || stages < 0 || issue < 0 || issue > 3) return COX_ERR_ARG;
     if (precision != COX_SPLIT_E4M3 && precision != COX_SPLIT_E2M1) return COX_ERR_ARG;
-    const int f4 = precision == COX_SPLIT_E2M1;
+    return cox_plan_form(precision == COX_SPLIT_E2M1 ? COX_FORM_E2M1 : COX_FORM_E4M3, k, tile_m, chunks, stages, issue, out);
+}
+
+int cox_plan_form(int form, int k, int tile_m, int chunks, int stages, int issue, cox_plan *out)
+{
+    if (!out || tile_m < 0 || chunks < 0 || stages < 0 || issue < 0 || issue > 3) return COX_ERR_ARG;
+    if (form < COX_FORM_E4M3 || form > COX_FORM_WIDE) return COX_ERR_ARG;
     GemmPlan g;
-    COX_TRY(plan_shape(g, k, tile_m, chunks, stages, issue, f4));
-    out->tile_m = g.T;
-    out->chunks = g.CH;
-    out->stages = g.stages;
-    out->ring = g.ring;
-    out->decoder_groups = g.G;
-    out->named_barriers = g.nb_period * g.T;
-    out->limb_cols = g.NP;
-    out->tmem_cols = (g.alt ? 2 : 1) * g.T * g.NP + g.ring * g.T * g.CH * (f4 ? 16 : 32) + (f4 ? 8 : 0);
-    out->smem_bytes = static_cast<long long>(g.smem);
-    out->issue = g.alt ? 2 : g.pair ? 3 : 1;
-    out->issuers = g.alt ? 2 : g.T;
-    out->mmas_per_commit = (f4 ? 2 : 4) * g.CH * (g.alt ? g.T : g.pair ? 2 : 1);
-    out->limb_stages = f4 ? g.stages2 : 0;
+    COX_TRY(plan_shape(g, k, tile_m, chunks, stages, issue, form));
+    fill_plan(g, form, out);
+    return COX_OK;
+}
+
+int cox_plan_default(int precision, int k, int *form_out, cox_plan *out)
+{
+    if ((precision != COX_SPLIT_E4M3 && precision != COX_SPLIT_E2M1) || k < 1 || k > MAX_K_TC) return COX_ERR_ARG;
+    const Shape s = default_shape(precision, k);
+    COX_TRY(cox_plan_form(s.form, k, s.T, s.CH, s.S, s.issue, out));
+    if (form_out) *form_out = s.form;
+    return COX_OK;
+}
+
+int cox_plan_in_use(cox_h h, int k, int product, int *form_out, cox_plan *out)
+{
+    if (!h || product < 0 || product > 1) return COX_ERR_ARG;
+    if (!is_split(h)) return COX_ERR_UNSUPPORTED;
+    COX_TRY(validate_k(h, k));
+    const Shape s = shape_for_handle(h, k, product);
+    COX_TRY(cox_plan_form(s.form, k, s.T, s.CH, s.S, s.issue, out));
+    if (form_out) *form_out = s.form;
     return COX_OK;
 }
 

@@ -45,9 +45,9 @@ inline int limb_cols4(int k)
 
 // Operand forms of a product (GemmPlan::f4).
 enum Form : int {
-    FORM_E4M3 = 0,  // e4m3 codes, LIMBS e4m3 limbs (kind::f8f6f4)
-    FORM_E2M1 = 1,  // e2m1 codes, LIMBS4 e2m1 limbs (kind::mxf4)
-    FORM_WIDE = 2   // e2m1 codes, the LIMBS e4m3 limbs' value as LIMBS_W e2m1 limbs (kind::mxf4)
+    FORM_E4M3 = COX_FORM_E4M3,  // e4m3 codes, LIMBS e4m3 limbs (kind::f8f6f4)
+    FORM_E2M1 = COX_FORM_E2M1,  // e2m1 codes, LIMBS4 e2m1 limbs (kind::mxf4)
+    FORM_WIDE = COX_FORM_WIDE   // e2m1 codes, the LIMBS e4m3 limbs' value as LIMBS_W e2m1 limbs (kind::mxf4)
 };
 inline int limbs_of(int form) { return form == FORM_WIDE ? LIMBS_W : form == FORM_E2M1 ? LIMBS4 : LIMBS; }
 

@@ -178,12 +178,16 @@ __global__ void __launch_bounds__(640) k_nmf_update(const UpdArgs A)
                 for (int q = 0; q < CPW; ++q) sum[q] = tf_add(sum[q], tf{b[u][q], 0.f});
         }
 #pragma unroll
-        for (int q = 0; q < CPW; ++q) {
-            pc[q] = sum[q].h;  // the pair's sum rounded to FP32
-            if (!isfinite(pc[q])) {  // past FP32's range pairs give NaN: the infinity it is
+        for (int q = 0; q < CPW; ++q) pc[q] = sum[q].h;  // the pair's sum rounded to FP32
+        static_assert(CPW == 4, "one test for the warp's four rows");
+        const float test = ((pc[0] - pc[0]) + (pc[1] - pc[1])) + ((pc[2] - pc[2]) + (pc[3] - pc[3]));
+        if (!(test == 0.f)) {  // past FP32's range pairs give NaN: the infinity it is
+            for (int q = 0; q < CPW; ++q) {
                 double d = 0.0;
                 for (int sl = 0; sl < ns; ++sl) d += c0 + q < r ? static_cast<double>(pp[sl * ps + q * NT]) : 0.0;
-                pc[q] = static_cast<float>(d);
+#pragma unroll
+                for (int e = 0; e < CPW; ++e)
+                    if (e == q) pc[e] = static_cast<float>(d);
             }
         }
     }

@@ -624,13 +624,7 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
             tc_fence_after();
             if constexpr (FL == LIMBS_W) {
                 // lambda columns of ten e2m1 limbs (weights 8^-l), up to four (40 TMEM
-                // columns, five loads of eight) at a time.  Limbs are joined in pairs first:
-                // a window's sums are multiples of 1/2 below 512 per K chunk, so
-                // S_l + S_(l+1) / 8 is exact for windows of up to 1820 chunks, and only the
-                // four additions between pairs round, each 64 times finer than the next.
-                // The gradient at n = 150,001, p = 3,001, k = 1 is 2.33e-7 of its norm from
-                // FP64, as with the e4m3 kernel (2.32e-7); one limb after the other, nine
-                // roundings each 8 times finer, left 2.71e-7.  Same number of operations.
+                // columns, five loads of eight) at a time
 #pragma unroll
                 for (int tt = 0; tt < T; ++tt) {
 #pragma unroll
@@ -649,13 +643,9 @@ __global__ void __launch_bounds__(32 * (2 + (ALT ? 2 : T) + 4 * G), 1)
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
                             if (e0 + e < KH) {
-                                float x = 0.f;
+                                float x = __uint_as_float(u[10 * e + 9]);
 #pragma unroll
-                                for (int l = 8; l >= 0; l -= 2) {
-                                    const float pair =
-                                        fmaf(__uint_as_float(u[10 * e + l + 1]), 0.125f, __uint_as_float(u[10 * e + l]));
-                                    x = l == 8 ? pair : fmaf(x, 0.015625f, pair);
-                                }
+                                for (int l = 8; l >= 0; --l) x = fmaf(x, 0.125f, __uint_as_float(u[10 * e + l]));
                                 acc(tt, e0 + e) += x;
                             }
                     }

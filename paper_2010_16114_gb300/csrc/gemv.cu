@@ -345,11 +345,12 @@ __global__ void k_eta_out(const double *__restrict__ eta, const double *__restri
 
 // Whether the FP64 products batch their loads: where a warp would else wait on memory
 // for every 32 entries, with few warps (1,000 of 2,000 entries 14.4 -> 12.4 us, of 20,000
-// 153 -> 89) or long rows (10,000 entries in 2,000 warps 84 -> 55, 4,000 in 8,000 74.5 ->
-// 67.9).  With many short rows resident warps hide the latency, and the batch's 48
-// registers cost a third of them: 1,000 entries in 20,000 warps 69.7 us against 57.8, 20
-// in 100,000 60.3 against 42.2.  In between (2,000 .. 5,000 entries) both are within 7%.
-bool batch_dots(const cox_handle *h, int64_t warps, int64_t len) { return warps < 8LL * h->sm_count || len >= 2500; }
+// 153 -> 89; a step at n = 1,200, p = 1,700, k = 2 from HBM 70.6 -> 65.0) or long rows
+// (10,000 entries in 2,000 warps 84 -> 55, 4,000 in 8,000 74.5 -> 67.9).  With many short
+// rows resident warps hide the latency, and the batch's 48 registers cost a third of them:
+// 1,000 entries in 20,000 warps 69.7 us against 57.8, 20 in 100,000 60.3 against 42.2.
+// In between (5,000 to 8,000 warps of 2,000 to 5,000 entries) both are within 7%.
+bool batch_dots(const cox_handle *h, int64_t warps, int64_t len) { return warps < 32LL * h->sm_count || len >= 2500; }
 
 unsigned blocks_for(int64_t n, int t) { return static_cast<unsigned>((n + t - 1) / t); }
 

@@ -27,7 +27,7 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# the metric's published name; the batched split form measured here uses e4m3 limbs ("precision" key)
+# the metric's published name; the operand form measured here is in the "precision" key
 METRIC = "l1-Cox prox-grad iters/s & HBM GB/s: batched-lambda split-BF16 vs plain FP32"
 UNIT = "iter/s"
 
@@ -44,7 +44,7 @@ def parse():
     ap.add_argument("--p", type=int, default=None)
     ap.add_argument("--k", type=int, default=None)
     ap.add_argument("--precision", default="split_e2m1", choices=["split_e4m3", "split_e2m1"],
-                    help="operand form of the tensor-core products: e2m1 (kind::mxf4, six limbs) or e4m3 "
+                    help="operand form of the tensor-core products: e2m1 (kind::mxf4, eight limbs) or e4m3 "
                          "(kind::f8f6f4, four limbs)")
     ap.add_argument("--tile-m", type=int, default=0)
     ap.add_argument("--stages", type=int, default=0)
@@ -351,7 +351,7 @@ def run_nmf(args, stream, cpu_baseline: bool = False):
     out = {"workload": f"nmf_{m // 1000}k_{n // 1000}k_r{r}", "m": m, "n": n, "r": r,
            "data": "synthetic: X uniform on the grid k/256 (exact in bf16), V0, W0 uniform [0,1) FP32",
            "precision": "X bf16; V, W FP32 as 3 bf16 limbs on tcgen05 (kind::f16), FP32 accumulation; "
-                        "Gram matrices FP64",
+                        "Gram matrices FP64 from sums in pairs of floats",
            "limb_cols": info["limb_cols"], "stages": info["stages"]}
     iters = args.nmf_iters
     for algo in ("mult", "apg"):
@@ -485,10 +485,14 @@ def run_ours(args, rank, world):
 
     # algorithmic bytes (packed X padded to 128 per dimension, as streamed by each product)
     xb = (-(-n // 128) * 128) * (-(-p // 128) * 128) / 4.0
-    lb = 4  # limb bytes per coefficient: 8 e2m1 nibbles or 4 e4m3 bytes
-    b1 = xb + p * lb * k + k * n * 4              # X, beta limbs, eta partials
-    b4 = xb + n * lb * k + 8 * k * p              # X, V limbs, beta read+write
-    scan_bytes = k * n * 8 * 12                     # FP64 scan passes (eta, w, R, F, gathers, V)
+    # limb bytes per coefficient: 8 e2m1 nibbles or 4 e4m3 bytes; 10 nibbles in the wide form
+    plan = prob.plan(k)
+    lb1, lb4 = (5 if plan[q]["form"] == "wide" else 4 for q in ("x_b", "xt_v"))
+    b1 = xb + p * lb1 * k + k * n * 4              # X, beta limbs, eta partials
+    b4 = xb + n * lb4 * k + 8 * k * p              # X, V limbs, beta read+write
+    # scans, per subject and column: eta partials read (4), eta as a pair of floats, w and V written
+    # and read once (16 + 8 + 8), event-group index and flags (7), limbs written
+    scan_bytes = k * n * (43 + lb4)
     iter_bytes = b1 + b4 + scan_bytes + 12 * k * p  # + beta limbs / l1 pass
     gemm_ms = cls_ms[0] + cls_ms[1]
     gemm_n = cls_n[0] + cls_n[1]
@@ -539,7 +543,7 @@ def run_ours(args, rank, world):
         prob.set_precision(args.precision)
 
     # the path fit (Section 6 rule): every penalty from beta = 0 to
-    # |F_t - F_{t-10}| / |F_t + 1| < tol or the iteration cap, replays of 10 steps
+    # |F_t - F_{t-10}| / |F_t + 1| < tol or the iteration cap, 10 iterations at a time
     path = None
     if args.path_iters > 0:
         torch.cuda.synchronize()
@@ -554,7 +558,7 @@ def run_ours(args, rank, world):
                 "converged_columns": int(np.sum(np.asarray(iters) < args.path_iters)),
                 "final_objective": [float(x) for x in obj],
                 "timing": "wall clock around cox_path_fit (10 iterations at a time, host reads the "
-                          "k objectives after each replay), beta = 0 to the stopping rule or the cap"}
+                          "k objectives after each run of them), beta = 0 to the stopping rule or the cap"}
 
     # the active-set X B late in the path: the 8 largest penalties from the
     # path fit's coefficients, dense then with the active set, same iterations
@@ -614,10 +618,10 @@ def run_ours(args, rank, world):
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "e2m1" if args.precision == "split_e2m1" else "e4m3", "data": "synthetic",
         "precision": ("genotype products: codes and 8-limb split coefficients as e2m1 on tcgen05 "
-                      "(kind::mxf4, unit block scales), FP32 accumulation; risk-set scans and objective FP64"
+                      "(kind::mxf4, unit block scales), FP32 accumulation; risk-set scans in pairs of floats per subject, FP64 per event time and in the objective"
                       if args.precision == "split_e2m1" else
                       "genotype products: codes and 4-limb split coefficients as e4m3 on tcgen05 "
-                      "(kind::f8f6f4), FP32 accumulation; risk-set scans and objective FP64"),
+                      "(kind::f8f6f4), FP32 accumulation; risk-set scans in pairs of floats per subject, FP64 per event time and in the objective"),
         "config": {"workload": workload_name(r), "n": n, "p": p, "k": k,
                    "l2": "inputs larger than L2: 2 x ~50 GB of packed genotypes streamed per step",
                    "parallelism": "replicas" if world > 1 else "single GPU",

@@ -156,7 +156,9 @@ void cox_destroy(cox_h h);
  * most tol relative (tol <= 0: the paper's 1e-6) or after maxiter iterations
  * (maxiter <= 0: the paper's 1000).  start_host: p doubles, the start vector
  * (NULL: all ones).  Synchronous.  Genotype handles run it on the tensor-core
- * products: COX_ERR_TIMEOUT when one of their waits runs out.
+ * products (COX_ERR_TIMEOUT when one of their waits runs out) in work memory that
+ * came with the handle: 16 (n_pad + p_pad) bytes, 8 p for a start vector and one
+ * product's partial sums.
  */
 int cox_lipschitz(cox_h h, const double *start_host, double tol, int maxiter, double *L_out);
 

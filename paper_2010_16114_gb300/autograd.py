@@ -4,8 +4,8 @@ forward(beta) returns f(beta) = -(1/n) log partial likelihood (arXiv
 2010.16114, Section 5.3, with the Section 6 Breslow ties) for each row of
 beta (shape (k, p) or (p,)).  The backward pass is the gradient the solver
 itself uses: the library's loss-and-gradient call runs the same two
-genotype products and FP64 risk-set scans as one proximal-gradient step,
-without the soft-threshold epilogue.  forward computes f and grad f in one
+genotype products and risk-set scans as one proximal-gradient step, without
+the soft-threshold epilogue.  forward computes f and grad f in one
 call and keeps grad f for backward.
 """
 from __future__ import annotations

@@ -42,9 +42,10 @@
 // ten e2m1 digits (split_wide).  Same operands, exact window sums, half the MMA
 // instructions per code, so the product is bound by HBM instead of by MMA
 // issue (16 MMAs of ~57 cycles per 16 KB stage in the e4m3 kernel at any N up
-// to 64).  Ten limb columns per coefficient fill 128 at k = 12.  Measured at
-// k = 1: a whole step at n = 100,000, p = 50,000 takes 566 us against 695 with
-// the e4m3 kernel, 20 iterations at n = 200,000, p = 10,000 6.79 ms against 7.75.
+// to 64).  Ten limb columns per coefficient fill 128 at k = 12.  Measured when it
+// came, at k = 1: a whole step at n = 100,000, p = 50,000 566 us against 695 with
+// the e4m3 kernel, 20 iterations at n = 200,000, p = 10,000 6.79 ms against 7.75
+// (474 us and 5.08 ms now, with the scans and launches since changed).
 //
 // Pipeline per CTA (one per SM): two TMA warps fill a ring of shared-memory
 // stages (T row tiles x CH K chunks of codes, and the matching limb panels);

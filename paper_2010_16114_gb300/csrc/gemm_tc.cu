@@ -204,9 +204,9 @@ bool ring_safe(int G, int R, int n) { return n >= G + R || n % G == 0; }
 // of NP 128-byte rows, released once the stage's MMAs are complete), each with
 // one producer thread that loads every stage in order and reuses a slot only
 // after its release.  Both depths keep ring_safe; S2 > R keeps the limb
-// producer of stage i from waiting on the decoders of stage i, and S2 = R + 3
-// when it fits gives the limbs (from L2) three stages of look-ahead (R + 2
-// measured 0.65 of HBM against 0.84).  The code ring takes the rest of the
+// producer of stage i from waiting on the decoders of stage i, and S2 = R + 4
+// or R + 3, the first that is safe and fits, gives the limbs (from L2) three to
+// four stages of look-ahead (R + 2 measured 0.65 of HBM against 0.84).  The code ring takes the rest of the
 // shared memory (at most 12, at least G + 1), the deepest safe depth.  The
 // largest TMEM ring for which such depths exist is taken.
 int plan_e2m1(GemmPlan &g, int T, int CH, int NP, int form, int G, int stages_req, int fold_bytes)
@@ -371,7 +371,7 @@ int plan_gemm(cox_handle *h, GemmPlan &g, const uint32_t *A, int64_t rows_pad, i
     // Codes that do not stay in L2 between iterations are loaded evict-first, so that
     // they push out neither the limbs and partial sums between the kernels nor the
     // scans' vectors: 20 iterations at n = 200,000, p = 10,000 (514 MB a copy) take
-    // 5.08 ms against 5.45, a step at n = 100,000, p = 50,000 484 us against 502.
+    // 5.08 ms against 5.45, a step at n = 100,000, p = 50,000 474 us against about 490.
     g.stream = 2 * (rows_pad * K_pad / 4) > h->l2_bytes / 2;
     {
         // the two products (and the autotuner's candidates) share kernels with

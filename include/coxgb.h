@@ -157,7 +157,7 @@ void cox_destroy(cox_h h);
  * (maxiter <= 0: the paper's 1000).  start_host: p doubles, the start vector
  * (NULL: all ones).  Synchronous.  Genotype handles run it on the tensor-core
  * products (COX_ERR_TIMEOUT when one of their waits runs out) in work memory that
- * came with the handle: 16 (n_pad + p_pad) bytes, 8 p for a start vector and one
+ * came with the handle: 12 (n_pad + p_pad) bytes, 8 p for a start vector and one
  * product's partial sums.
  */
 int cox_lipschitz(cox_h h, const double *start_host, double tol, int maxiter, double *L_out);

@@ -306,8 +306,8 @@ struct Workspace {
 struct PowerWork {
     void *base = nullptr;         // one allocation
     uint8_t *Bq = nullptr, *Vq = nullptr;
-    float *part = nullptr;
-    double *a = nullptr, *b = nullptr, *start = nullptr;
+    float *part = nullptr, *a = nullptr, *b = nullptr;
+    double *start = nullptr;
     void *scal = nullptr;
     GemmPlan g1, g4;
 };

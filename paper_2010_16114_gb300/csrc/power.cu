@@ -4,17 +4,16 @@
 //
 // Each vector enters the product kernel as LIMBS_W e2m1 digits per entry (the
 // wide form, one column): with max |x| 2^-s in [1, 2), x 2^(28-s) rounded to an
-// integer and written in balanced radix 8, so an entry is held to 2^(s-29), and
-// the products' window sums are exact.  The vectors are FP64 up to that rounding,
-// and mu^T v and sum a are formed from the values the digits hold, so that the
-// products are exactly the centred ones of those values.  (With v and a rounded to
-// FP32 first, ||v|| and a's roundings, which all have the offset mu^T v in common,
-// left the estimate 1.6e-9 to 4.1e-9 from FP64; it is 0.7e-9 to 1.4e-9 now.)
+// integer and written in balanced radix 8, so an entry is held to 2^(s-29),
+// exactly where |x| >= 2^-5 max |x|, and the products' window sums are exact.  The
+// estimate is 1.6e-9 to 4.1e-9 from FP64 (root mean square, four sizes; ~1e-8 with the
+// FP32 product before): ||v|| after its rounding to FP32, and a's roundings, which have
+// the offset mu^T v in common.
 // One iteration is six kernels and one 8-byte copy:
 //   k_pow_v      v = b / ||b||, its digits, mu^T v
 //   (product)    X v, partial slots
-//   k_pow_a      a = X v - mu^T v, max |a|
-//   k_pow_alimbs digits of a in the K order of the SNP-major copy, block sums of a
+//   k_pow_a      a = X v - mu^T v, sum a, max |a|
+//   k_pow_alimbs digits of a in the K order of the SNP-major copy
 //   (product)    X^T a, partial slots
 //   k_pow_b      b = X^T a - mu sum a, ||b||^2, max |b|
 // Reductions leave one FP64 partial per block; the block that finishes last adds
@@ -38,12 +37,12 @@ constexpr int POW_BLOCKS = 256;  // most blocks of a reducing kernel
 struct PowScal {
     double nb2;        // ||b||^2
     double muv;        // mu^T v
+    double suma;       // sum a
     float maxb, maxa;  // max |b|, max |a|
     int s1, s4;        // scale exponents of the two digit matrices
     int err;           // device error bits of the products
     unsigned count;    // blocks done
     double part[POW_BLOCKS];
-    double asum[POW_BLOCKS];  // sums of a by the blocks of k_pow_alimbs
     float maxp[POW_BLOCKS];
 };
 
@@ -97,28 +96,17 @@ __device__ __forceinline__ bool reduce_last(PowScal *S, double &sum, float &mx)
     return true;
 }
 
-// 2^e for |e| < 1023 (an FP64 division or ldexp at the end of a block is latency)
-__device__ __forceinline__ double pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
-
-// Scale exponent s: max |x| 2^-s in [1, 2).
+// Scale exponent s (max |x| 2^-s in [1, 2)) and the digits of x.
 __device__ __forceinline__ int pow_scale(float mx) { return mx > 0.f && isfinite(mx) ? ilogbf(mx) : 0; }
 
-// x per_unit, per_unit = 2^(28-s), rounded to an integer by adding 1.5 2^52 (one FP64
-// instruction; its low word is the integer): the digits, the integer, and in `bad`
-// whether x was not finite (it then has no digits).
-constexpr double ROUND = 6755399441055744.0;
-__device__ __forceinline__ int digits(double x, double per_unit, uint8_t *d, bool &bad)
+__device__ __forceinline__ void digits(float x, int s, uint8_t *d)
 {
-    const double r = fma(x, per_unit, ROUND);  // |x| per_unit <= 2^29 (1 + 2^-23)
-    const bool ok = isfinite(r);
-    bad |= !ok;
-    const int q = ok ? __double2loint(r) : 0;
-    split_wide(q, d);
-    return q;
+    const float r = ldexpf(x, 28 - s);  // |r| < 2^29; a NaN has no digits (it reaches the sums instead)
+    split_wide(isfinite(r) ? __float2int_rn(r) : 0, d);
 }
 
 // b = start / ||start|| (start null: all entries 1/sqrt(p)) with ||b||^2 taken as 1; one block.
-__global__ void __launch_bounds__(PT) k_pow_start(const double *__restrict__ start, int64_t p, double *__restrict__ b,
+__global__ void __launch_bounds__(PT) k_pow_start(const double *__restrict__ start, int64_t p, float *__restrict__ b,
                                                   PowScal *S)
 {
     __shared__ double sh[PT / 32];
@@ -128,9 +116,9 @@ __global__ void __launch_bounds__(PT) k_pow_start(const double *__restrict__ sta
     const double inv = 1.0 / sqrt(block_sum(s, sh));
     float mx = 0.f;
     for (int64_t j = threadIdx.x; j < p; j += PT) {
-        const double v = (start ? start[j] : 1.0) * inv;
+        const float v = static_cast<float>((start ? start[j] : 1.0) * inv);
         b[j] = v;
-        mx = fmaxf(mx, fabsf(static_cast<float>(v)));
+        mx = fmaxf(mx, fabsf(v));
     }
     mx = block_max(mx, shf);
     if (threadIdx.x == 0) {
@@ -141,29 +129,32 @@ __global__ void __launch_bounds__(PT) k_pow_start(const double *__restrict__ sta
     }
 }
 
-// v = b / ||b||, its digits (byte t holds SNPs 16 (t / 8) + t mod 8 and that + 8), mu^T v
-__global__ void __launch_bounds__(PT) k_pow_v(const double *__restrict__ b, const double *__restrict__ mu, int64_t p,
+// v = b / ||b|| (FP32), its digits (byte t holds SNPs 16 (t / 8) + t mod 8 and that + 8), mu^T v
+__global__ void __launch_bounds__(PT) k_pow_v(const float *__restrict__ b, const double *__restrict__ mu, int64_t p,
                                               int64_t p_pad, uint8_t *__restrict__ Bq, PowScal *S)
 {
     const double inv = 1.0 / sqrt(S->nb2);
     const int s = pow_scale(static_cast<float>(static_cast<double>(S->maxb) * inv));
-    const double per_unit = pow2(28 - s);
     const int64_t rb = p_pad / 2;
-    double dot = 0.0;  // in units of 2^(s-28)
-    bool bad = false;
+    double dot = 0.0;
     for (int64_t t = static_cast<int64_t>(blockIdx.x) * PT + threadIdx.x; t < rb; t += static_cast<int64_t>(gridDim.x) * PT) {
         const int64_t j = ((t >> 3) << 4) + (t & 7);
         if (j >= p) continue;
         uint8_t d0[LIMBS_W], d1[LIMBS_W] = {};
-        dot = fma(mu[j], static_cast<double>(digits(b[j] * inv, per_unit, d0, bad)), dot);
-        if (j + 8 < p) dot = fma(mu[j + 8], static_cast<double>(digits(b[j + 8] * inv, per_unit, d1, bad)), dot);
+        const float v0 = static_cast<float>(static_cast<double>(b[j]) * inv);
+        dot += mu[j] * static_cast<double>(v0);
+        digits(v0, s, d0);
+        if (j + 8 < p) {
+            const float v1 = static_cast<float>(static_cast<double>(b[j + 8]) * inv);
+            dot += mu[j + 8] * static_cast<double>(v1);
+            digits(v1, s, d1);
+        }
 #pragma unroll
         for (int l = 0; l < LIMBS_W; ++l) Bq[l * rb + t] = static_cast<uint8_t>(d0[l] | (d1[l] << 4));
     }
-    if (bad) dot = NAN;  // not finite: the estimate is not either
     float mx = 0.f;
     if (reduce_last(S, dot, mx) && threadIdx.x == 0) {
-        S->muv = dot * pow2(s - 28);
+        S->muv = dot;
         S->s1 = s - 7;  // the product's wide limbs are worth 2^(scale + 7)
     }
 }
@@ -179,67 +170,57 @@ __device__ __forceinline__ double slots(const float *__restrict__ part, int64_t 
     return v;
 }
 
-// a = X v - mu^T v for the n subjects; max |a|
+// a = X v - mu^T v for the n subjects, in FP32; sum a, max |a|
 __global__ void __launch_bounds__(PT) k_pow_a(const float *__restrict__ part, int64_t stride, int group_rows, int KC,
-                                              int64_t L, int64_t n, double *__restrict__ a, PowScal *S)
+                                              int64_t L, int64_t n, float *__restrict__ a, PowScal *S)
 {
     const double muv = S->muv;
-    double none = 0.0;
+    double sum = 0.0;
     float mx = 0.f;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * PT + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * PT) {
-        const double v = slots(part, stride, i, group_rows, KC, L) - muv;
+        const float v = static_cast<float>(slots(part, stride, i, group_rows, KC, L) - muv);
         a[i] = v;
-        mx = fmaxf(mx, fabsf(static_cast<float>(v)));
+        sum += static_cast<double>(v);
+        mx = fmaxf(mx, fabsf(v));
     }
-    if (reduce_last(S, none, mx) && threadIdx.x == 0) {
+    if (reduce_last(S, sum, mx) && threadIdx.x == 0) {
+        S->suma = sum;
         S->maxa = mx;
         S->s4 = pow_scale(mx) - 7;
     }
 }
 
-// digits of a at the A4 K positions (byte order as k_pow_v's, in sorted blocks of 16), and
-// the blocks' sums of a, exact in integers
-__global__ void __launch_bounds__(PT) k_pow_alimbs(const double *__restrict__ a, int64_t n, int64_t n_pad, int64_t pa,
-                                                   int64_t pnb, uint8_t *__restrict__ Vq, PowScal *S)
+// digits of a at the A4 K positions (byte order as k_pow_v's, in sorted blocks of 16)
+__global__ void __launch_bounds__(PT) k_pow_alimbs(const float *__restrict__ a, int64_t n, int64_t n_pad, int64_t pa,
+                                                   int64_t pnb, uint8_t *__restrict__ Vq, const PowScal *S)
 {
-    __shared__ double sh[PT / 32];
-    const double per_unit = pow2(21 - S->s4);
+    const int s = S->s4 + 7;
     const int64_t rb = n_pad / 2;
-    long long sum = 0;
-    bool bad = false;
     for (int64_t t = static_cast<int64_t>(blockIdx.x) * PT + threadIdx.x; t < rb; t += static_cast<int64_t>(gridDim.x) * PT) {
         const int64_t i = ((t >> 3) << 4) + (t & 7);
         if (i >= n) continue;
         uint8_t d0[LIMBS_W], d1[LIMBS_W] = {};
-        sum += digits(a[i], per_unit, d0, bad);
-        if (i + 8 < n) sum += digits(a[i + 8], per_unit, d1, bad);
+        digits(a[i], s, d0);
+        if (i + 8 < n) digits(a[i + 8], s, d1);
         const int64_t byte = e2m1_byte(a4_pos(i, pa, pnb));
 #pragma unroll
         for (int l = 0; l < LIMBS_W; ++l) Vq[l * rb + byte] = static_cast<uint8_t>(d0[l] | (d1[l] << 4));
     }
-    const double t = block_sum(bad ? NAN : static_cast<double>(sum), sh);
-    if (threadIdx.x == 0) S->asum[blockIdx.x] = t * pow2(S->s4 - 21);
 }
 
-// b = X^T a - mu sum a; ||b||^2, max |b|
+// b = X^T a - mu sum a, in FP32; ||b||^2, max |b|
 __global__ void __launch_bounds__(PT) k_pow_b(const float *__restrict__ part, int64_t stride, int group_rows, int KC,
-                                              int64_t L, int64_t p, const double *__restrict__ mu, double *__restrict__ b,
-                                              int nsum, PowScal *S)
+                                              int64_t L, int64_t p, const double *__restrict__ mu, float *__restrict__ b,
+                                              PowScal *S)
 {
-    __shared__ double sh[PT / 32];
-    // the first row's loads are in flight while the block sums are added
-    int64_t j = static_cast<int64_t>(blockIdx.x) * PT + threadIdx.x;
-    double x = j < p ? slots(part, stride, j, group_rows, KC, L) : 0.0;
-    const double suma = block_sum(static_cast<int>(threadIdx.x) < nsum ? S->asum[threadIdx.x] : 0.0, sh);
+    const double suma = S->suma;
     double sum = 0.0;
     float mx = 0.f;
-    while (j < p) {
-        const double v = x - mu[j] * suma;
-        b[j] = v;
+    for (int64_t j = static_cast<int64_t>(blockIdx.x) * PT + threadIdx.x; j < p; j += static_cast<int64_t>(gridDim.x) * PT) {
+        const double v = slots(part, stride, j, group_rows, KC, L) - mu[j] * suma;
+        b[j] = static_cast<float>(v);
         sum += v * v;
         mx = fmaxf(mx, fabsf(static_cast<float>(v)));
-        j += static_cast<int64_t>(gridDim.x) * PT;
-        if (j < p) x = slots(part, stride, j, group_rows, KC, L);
     }
     if (reduce_last(S, sum, mx) && threadIdx.x == 0) {
         S->nb2 = sum;
@@ -265,15 +246,15 @@ int power_setup(cox_handle *h)
     COX_TRY(plan_gemm(h, w.g1, h->d_A1, n_pad, p_pad, reinterpret_cast<const uint8_t *>(h->d_A1), 1, FORM_WIDE, 0, 0, 0, 0));
     COX_TRY(plan_gemm(h, w.g4, h->d_A4, p_pad, n_pad, reinterpret_cast<const uint8_t *>(h->d_A4), 1, FORM_WIDE, 0, 0, 0, 0));
     const int64_t part = up256(4 * std::max(w.g1.max_slots * n_pad, w.g4.max_slots * p_pad));
-    const int64_t fb = up256(8 * p_pad), fa = up256(8 * n_pad), st = up256(8 * h->p), sc = up256(sizeof(PowScal));
+    const int64_t fb = up256(4 * p_pad), fa = up256(4 * n_pad), st = up256(8 * h->p), sc = up256(sizeof(PowScal));
     uint8_t *base = nullptr;
     COX_TRY(dmalloc(h, reinterpret_cast<void **>(&base), static_cast<size_t>(bq + vq + part + fb + fa + st + sc)));
     w.base = base;
     w.Bq = base;
     w.Vq = w.Bq + bq;
     w.part = reinterpret_cast<float *>(w.Vq + vq);
-    w.b = reinterpret_cast<double *>(w.Vq + vq + part);
-    w.a = reinterpret_cast<double *>(w.Vq + vq + part + fb);
+    w.b = reinterpret_cast<float *>(w.Vq + vq + part);
+    w.a = reinterpret_cast<float *>(w.Vq + vq + part + fb);
     w.start = reinterpret_cast<double *>(w.Vq + vq + part + fb + fa);
     w.scal = w.Vq + vq + part + fb + fa + st;
     // digit rows past LIMBS_W and K positions of padding stay zero
@@ -308,10 +289,10 @@ int power_method_tiles(cox_handle *h, const double *start, double tol, int maxit
         k_pow_v<<<blocks(h->p_pad / 2), PT, 0, st>>>(w.b, h->d_mu, p, h->p_pad, w.Bq, S);
         COX_TRY(product(w.g1, &S->s1));
         k_pow_a<<<blocks(n), PT, 0, st>>>(w.part, h->n_pad, w.g1.T * TILE, w.g1.KC, w.g1.L, n, w.a, S);
-        k_pow_alimbs<<<blocks(h->n_pad / 2), PT, 0, st>>>(w.a, n, h->n_pad, h->kperm_a, h->kperm_nb, w.Vq, S);
+        k_pow_alimbs<<<static_cast<unsigned>(std::min<int64_t>(8LL * h->sm_count, (h->n_pad / 2 + PT - 1) / PT)), PT, 0, st>>>(
+            w.a, n, h->n_pad, h->kperm_a, h->kperm_nb, w.Vq, S);
         COX_TRY(product(w.g4, &S->s4));
-        k_pow_b<<<blocks(p), PT, 0, st>>>(w.part, h->p_pad, w.g4.T * TILE, w.g4.KC, w.g4.L, p, h->d_mu, w.b,
-                                             static_cast<int>(blocks(h->n_pad / 2)), S);
+        k_pow_b<<<blocks(p), PT, 0, st>>>(w.part, h->p_pad, w.g4.T * TILE, w.g4.KC, w.g4.L, p, h->d_mu, w.b, S);
         COX_CUDA(cudaGetLastError());
         double nb2 = 0.0;
         COX_CUDA(cudaMemcpy(&nb2, &S->nb2, sizeof(double), cudaMemcpyDeviceToHost));

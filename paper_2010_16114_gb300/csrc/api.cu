@@ -113,13 +113,17 @@ struct Shape {
 // What handles of a precision launch for k columns when the options force no pipeline
 // shape and nothing is tuned.  An e4m3 handle takes the wide form where it holds k
 // columns, k <= 12 (the same coefficients and exact window sums; the product is then
-// bound by HBM, not by MMA issue): whole steps at k = 1 .. 12 are 1.15 to 1.7 times as
-// fast as with the e4m3 kernel at n x p = 4,099 x 1,500, 20,000 x 5,000, 5,000 x 100,000,
-// 100,000 x 50,000 and 400,000 x 20,000 (least at 20,000 x 5,000, k = 12: 143 us against
-// 164).  Past 12 columns the wide limbs would need more than 128 MMA columns, twice the
+// bound by HBM, not by MMA issue).  Both products, wide against the e4m3 kernel's 2 x 2
+// shape, at k = 1, 4, 8, 12: 400,000 x 20,000 689, 701, 733, 740 us against 902, 904, 923,
+// 944; 100,000 x 50,000 436, 444, 461, 469 against 564, 568, 577, 591; 5,000 x 100,000 82,
+// 84, 94, 99 against 89, 93, 99, 110; 20,000 x 5,000 45, 49, 64, 75 against 45, 49, 60, 76;
+// 4,099 x 1,500 33, 37, 46, 53 against 29, 34, 42, 53, where codes come from L2 and the
+// fold of ten limbs costs more than the instructions saved (3 us, 2 to 6% of a step).  The
+// line does not depend on the size, so that one handle's results have one rounding whatever
+// its data.  Past 12 columns the wide limbs would need more than 128 MMA columns, twice the
 // e4m3 kernel's MMA cycles.  k = 17 .. 32: two K chunks per stage and two decoder groups
-// give 8 MMAs per commit; a step at n = 400,000, p = 100,000, k = 32 takes 6.6 ms against
-// 7.2 with one chunk.
+// give 8 MMAs per commit; a step at n = 400,000, p = 100,000, k = 32 takes 6.3 ms, 6.6
+// when the shape came, against 7.2 with one chunk.
 Shape default_shape(int precision, int k)
 {
     if (precision == COX_SPLIT_E2M1) return {FORM_E2M1, 0, 0, 0, 0};
